@@ -19,8 +19,9 @@
 //               MMA issuer: tcgen05.mma kind::f16, M = 128, N = 256, K = 16,
 //               four per stage; commits free the stage and, after a tile's
 //               last step, hand the accumulator to the epilogue.
-//   warps 2..5  epilogue: thread = output row = TMEM lane (quarter = warp % 4),
-//               32 columns per tcgen05.ld; the next tile's MMAs run into the
+//   warps 2..9  epilogue: two warps per TMEM lane quarter (quarter = warp % 4,
+//               thread = output row = TMEM lane), which take the tile's 32-column
+//               chunks (QKV: heads) in turn; the next tile's MMAs run into the
 //               other accumulator meanwhile.
 // Epilogues (fp32 until the final bf16 rounding):
 //   STORE  out = acc + bias
@@ -29,6 +30,12 @@
 //   QKV    columns [q | k | v] of H heads of width d: q and k RMS-normalised
 //          per head with a [d] weight, then rotated by RoPE on interleaved
 //          pairs at the row's joint position; written head-major.
+// A tile whose MMAs take 4 us (K = 1024) left the epilogue of four warps, with
+// 16-byte accesses 32 rows apart and a global-load latency per 32 columns, as
+// the longer part (11 us a tile with GELU). So the per-column vectors of a tile
+// go to shared memory and the first residuals to registers before its
+// accumulator is ready, and global rows are read and written through a 2 KB
+// staging buffer per warp, 64 contiguous bytes of eight rows per instruction.
 // Reference segments may be gated on the per-sample mode: their tiles are
 // skipped when the mode is REUSE (Algorithm 1 skips reference rows) and, for
 // QKV, the K and V column tiles also when it is BOUNDARY (the block keeps its
@@ -56,9 +63,13 @@ constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr int OFF_BAR = STAGES * STAGE_BYTES;
 constexpr int NUM_BARS = 2 * STAGES + 2 + 2 + 1;  // full, empty, tfull[2], tempty[2], drain
 constexpr int OFF_MISC = OFF_BAR + NUM_BARS * 8;
-constexpr int SMEM_BYTES = OFF_MISC + 16;
+constexpr int EPI_WARPS = 8;
+constexpr int EPI_STAGE_BYTES = 32 * 64;                  // 32 rows x 32 bf16 (or 16 fp32) of one warp
+constexpr int EPI_WARP_BYTES = EPI_STAGE_BYTES + 2 * 512;  // and two per-column vectors of its 128 columns
+constexpr int OFF_EPI = (OFF_MISC + 16 + 127) / 128 * 128;
+constexpr int SMEM_BYTES = OFF_EPI + EPI_WARPS * EPI_WARP_BYTES;
 constexpr int SMEM_ALLOC = SMEM_BYTES + 1024;
-constexpr int THREADS = 192;
+constexpr int THREADS = 64 + 32 * EPI_WARPS;
 constexpr int TMEM_COLS = 512;
 static_assert(SMEM_ALLOC <= 232448, "shared memory budget");
 
@@ -77,7 +88,8 @@ constexpr int P_STAGE_BYTES = P_A_BYTES + P_B_BYTES;
 constexpr int P_OFF_BAR = P_STAGES * P_STAGE_BYTES;
 constexpr int P_NUM_BARS = 2 * P_STAGES + 2 + 2 + 1;
 constexpr int P_OFF_MISC = P_OFF_BAR + P_NUM_BARS * 8;
-constexpr int P_SMEM_BYTES = P_OFF_MISC + 16;
+constexpr int P_OFF_EPI = (P_OFF_MISC + 16 + 127) / 128 * 128;
+constexpr int P_SMEM_BYTES = P_OFF_EPI + EPI_WARPS * EPI_WARP_BYTES;
 constexpr int P_SMEM_ALLOC = P_SMEM_BYTES + 1024;
 static_assert(P_SMEM_ALLOC <= 232448, "shared memory budget");
 
@@ -116,7 +128,7 @@ struct Tile {
 
 constexpr int GROUP_M = 16;  // tile rows per band of the tile order
 
-template <int TM>  // output rows per tile: 128 (one CTA) or 256 (a CTA pair)
+template <int TM, int EPI>  // TM: output rows per tile, 128 (one CTA) or 256 (a CTA pair)
 __device__ __forceinline__ Tile decode(const Params& p, int64_t t) {
   Tile r;
   int g = 0;
@@ -142,147 +154,243 @@ __device__ __forceinline__ Tile decode(const Params& p, int64_t t) {
   if (sg.gated) {
     const int m = __ldg(p.mode + r.s);
     if (m == RA_MODE_REUSE) r.live = false;
-    if (p.epi == RA_EPI_QKV && m == RA_MODE_BOUNDARY && r.n0 >= p.C) r.live = false;
+    if (EPI == RA_EPI_QKV && m == RA_MODE_BOUNDARY && r.n0 >= p.C) r.live = false;
   }
   return r;
 }
 
-// GELU, tanh form, through the identity 0.5 x (1 + tanh(u)) = x / (1 + e^(-2u)),
-// u = sqrt(2/pi) (x + 0.044715 x^3): one exponential and one division instead
-// of tanhf (e^(-2u) overflowing to +inf for very negative x gives -0).
-__device__ __forceinline__ float gelu_tanh(float x) {
-  const float u = 0.7978845608028654f * fmaf(0.044715f * x * x, x, x);
-  return __fdividef(x, 1.f + __expf(-2.f * u));
+// GELU, tanh form, of two values through the identity
+// 0.5 x (1 + tanh(u)) = x / (1 + e^(-2u)), u = sqrt(2/pi) (x + 0.044715 x^3),
+// with e^(-2u) = 2^(x (c + 0.044715 c x^2)), c = -2 sqrt(2/pi) log2(e): one
+// exponential and one reciprocal (an exponential that overflows to +inf for
+// very negative x gives -0).
+__device__ __forceinline__ void gelu_tanh2(float& x0, float& x1) {
+  constexpr float c = -2.f * 0.7978845608028654f * 1.4426950408889634f;
+  const uint64_t x = f2_pack(x0, x1);
+  float z0, z1;
+  f2_unpack(f2_mul(x, f2_fma(f2_mul(x, x), f2_pack(0.044715f * c, 0.044715f * c), f2_pack(c, c))), z0, z1);
+  float d0, d1;
+  f2_unpack(f2_add(f2_pack(ex2_approx(z0), ex2_approx(z1)), f2_pack(1.f, 1.f)), d0, d1);
+  f2_unpack(f2_mul(x, f2_pack(rcp_approx(d0), rcp_approx(d1))), x0, x1);
 }
 
-__device__ __forceinline__ void store32(__nv_bfloat16* dst, const float (&x)[32]) {
-  uint32_t pk[16];
+// The 64-byte row slots of a warp's staging buffer: 16-byte piece q of row r.
+// The permutation keeps both access patterns free of bank conflicts (every
+// lane its own row; eight rows, four lanes a row).
+__device__ __forceinline__ uint4* stage_slot(uint8_t* stage, int r, int q) {
+  return reinterpret_cast<uint4*>(stage + r * 64 + ((q ^ ((r >> 1) & 3)) << 4));
+}
+// Four 16-byte loads per lane of up to 32 rows of 64 bytes at `src` (row
+// stride in bytes): load i is piece lane % 4 of row 8 i + lane / 4.
+__device__ __forceinline__ void rows_fetch(const char* src, int64_t stride, int nrow, uint4 (&v)[4]) {
+  const int lane = threadIdx.x & 31, r0 = lane >> 2;
+  const char* ptr = src + r0 * stride + (lane & 3) * 16;
 #pragma unroll
-  for (int i = 0; i < 16; ++i) pk[i] = pack_bf16x2(x[2 * i], x[2 * i + 1]);
-  uint4* d = reinterpret_cast<uint4*>(dst);
-  d[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-  d[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-  d[2] = make_uint4(pk[8], pk[9], pk[10], pk[11]);
-  d[3] = make_uint4(pk[12], pk[13], pk[14], pk[15]);
+  for (int i = 0; i < 4; ++i)
+    v[i] = (r0 + 8 * i < nrow) ? *reinterpret_cast<const uint4*>(ptr + 8 * i * stride) : make_uint4(0, 0, 0, 0);
+}
+// rows_fetch's registers -> the lane's own row (64 bytes), through the staging buffer.
+__device__ __forceinline__ void rows_turn(uint8_t* stage, const uint4 (&v)[4], uint4 (&own)[4]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) *stage_slot(stage, 8 * i + (lane >> 2), lane & 3) = v[i];
+  __syncwarp();
+#pragma unroll
+  for (int q = 0; q < 4; ++q) own[q] = *stage_slot(stage, lane, q);
+  __syncwarp();
+}
+// 32 fp32 of every lane's row -> bf16 -> up to 32 rows of 64 bytes at `dst`.
+__device__ __forceinline__ void rows_store(uint8_t* stage, const float (&x)[32], char* dst, int64_t stride, int nrow) {
+  const int lane = threadIdx.x & 31, r0 = lane >> 2;
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    *stage_slot(stage, lane, q) =
+        make_uint4(pack_bf16x2(x[8 * q], x[8 * q + 1]), pack_bf16x2(x[8 * q + 2], x[8 * q + 3]),
+                   pack_bf16x2(x[8 * q + 4], x[8 * q + 5]), pack_bf16x2(x[8 * q + 6], x[8 * q + 7]));
+  __syncwarp();
+  char* ptr = dst + r0 * stride + (lane & 3) * 16;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint4 v = *stage_slot(stage, r0 + 8 * i, lane & 3);
+    if (r0 + 8 * i < nrow) *reinterpret_cast<uint4*>(ptr + 8 * i * stride) = v;
+  }
+  __syncwarp();
 }
 
-__device__ __forceinline__ void load_acc(uint32_t taddr, const float* bias, int n, float (&x)[32]) {
-  uint32_t v[32];
-  tmem_ld32(taddr, v);
-  tmem_ld_wait();
-  if (bias) {
-    const float4* b4 = reinterpret_cast<const float4*>(bias + n);
+// What an epilogue warp works on: its 32 rows (row0 + lane, nrow of them in
+// the segment), its share of the tile's columns (half 0 or 1), its shared
+// memory (staging buffer, two vectors of 128 per-column values) and the TMEM
+// address of its lanes in the tile's accumulator.
+struct EpiWarp {
+  int row0, nrow, half;
+  uint8_t* stage;
+  float* vec0;
+  float* vec1;
+  uint32_t acc;
+};
+
+// 32 accumulators plus 32 per-column values from shared memory.
+__device__ __forceinline__ void add_cols(const uint32_t (&v)[32], const float* cols, float (&x)[32]) {
+  const float4* c4 = reinterpret_cast<const float4*>(cols);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float4 b = __ldg(b4 + i);
-      x[4 * i] = __uint_as_float(v[4 * i]) + b.x;
-      x[4 * i + 1] = __uint_as_float(v[4 * i + 1]) + b.y;
-      x[4 * i + 2] = __uint_as_float(v[4 * i + 2]) + b.z;
-      x[4 * i + 3] = __uint_as_float(v[4 * i + 3]) + b.w;
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < 32; ++i) x[i] = __uint_as_float(v[i]);
+  for (int i = 0; i < 8; ++i) {
+    const float4 c = c4[i];
+    x[4 * i] = __uint_as_float(v[4 * i]) + c.x;
+    x[4 * i + 1] = __uint_as_float(v[4 * i + 1]) + c.y;
+    x[4 * i + 2] = __uint_as_float(v[4 * i + 2]) + c.z;
+    x[4 * i + 3] = __uint_as_float(v[4 * i + 3]) + c.w;
   }
 }
 
-// Epilogue of one output tile for the calling thread's row r (within the
-// segment's sample): 256 accumulator columns at TMEM address `base`.
-__device__ __forceinline__ void epilogue_tile(const Params& p, const Tile& tl, int r, uint32_t base) {
+// STORE, GELU, RESID: chunk j of the warp is tile columns 32 (half + 2 j) ...
+template <int EPI, class Ready>
+__device__ __forceinline__ bool epilogue_linear(const Params& p, const Tile& tl, const EpiWarp& w, Ready ready) {
+  constexpr int CHUNKS = BN / 64;
   const Seg& sg = p.seg[tl.seg];
-  const bool valid = r < sg.rows;
-  if (p.epi == RA_EPI_QKV) {
-    const int part = tl.n0 / p.C;               // 0 q, 1 k, 2 v
-    const int h0 = (tl.n0 - part * p.C) / p.d;  // first head of the tile
-    const int pos = sg.pos_offset + r;
-    for (int hh = 0; hh < BN / p.d; ++hh) {
-      const int cb = hh * p.d;                  // tile column of the head
-      const int h = h0 + hh;
-      __nv_bfloat16* drow = sg.dst[part] + tl.s * sg.dst_sb[part] + h * sg.dst_sh[part] +
-                            int64_t(valid ? r : 0) * sg.dst_sn[part];
-      if (part == 2) {
-        for (int c0 = 0; c0 < p.d; c0 += 32) {
-          float x[32];
-          load_acc(base + cb + c0, sg.bias, tl.n0 + cb + c0, x);
-          if (valid) store32(drow + c0, x);
-        }
-        continue;
-      }
-      float ss = 0.f;
-      for (int c0 = 0; c0 < p.d; c0 += 32) {
-        float x[32];
-        load_acc(base + cb + c0, sg.bias, tl.n0 + cb + c0, x);
+  const int lane = threadIdx.x & 31, n0 = tl.n0 + 32 * w.half;
 #pragma unroll
-        for (int j = 0; j < 32; ++j) ss = fmaf(x[j], x[j], ss);
-      }
-      const float rstd = rsqrtf(ss / float(p.d) + p.norm_eps);
-      const float* w = sg.norm_w[part];
-      const float4* cs = p.rope + int64_t(valid ? pos : 0) * (p.d / 4);
-      for (int c0 = 0; c0 < p.d; c0 += 32) {
-        float x[32];
-        load_acc(base + cb + c0, sg.bias, tl.n0 + cb + c0, x);
-        const float4* w4 = reinterpret_cast<const float4*>(w + c0);
+  for (int j = 0; j < CHUNKS; ++j) {
+    w.vec0[32 * j + lane] = sg.bias ? __ldg(sg.bias + n0 + 64 * j + lane) : 0.f;
+    if (EPI == RA_EPI_RESID) w.vec1[32 * j + lane] = __ldg(sg.gate + int64_t(tl.s) * sg.gate_ss + n0 + 64 * j + lane);
+  }
+  const char* res = nullptr;
+  uint4 rnext[4];
+  if (EPI == RA_EPI_RESID) {
+    res = reinterpret_cast<const char*>(sg.resid + int64_t(tl.s) * sg.res_ss + int64_t(w.row0) * sg.res_sr + n0);
+    rows_fetch(res, 2 * sg.res_sr, w.nrow, rnext);
+  }
+  char* out = reinterpret_cast<char*>(sg.out + int64_t(tl.s) * sg.out_ss + int64_t(w.row0) * sg.out_sr + n0);
+  __syncwarp();
+  if (!ready()) return false;
+  if (w.nrow <= 0) return true;
+  uint32_t v[32];
+  tmem_ld32(w.acc + 32 * w.half, v);
+#pragma unroll 1
+  for (int j = 0; j < CHUNKS; ++j) {
+    float x[32];
+    tmem_ld_wait_for(v);
+    add_cols(v, w.vec0 + 32 * j, x);
+    if (j + 1 < CHUNKS) tmem_ld32(w.acc + 32 * w.half + 64 * (j + 1), v);
+    if (EPI == RA_EPI_GELU) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const float4 wv = __ldg(w4 + q);
-          const float4 rc = valid ? __ldg(cs + c0 / 4 + q) : make_float4(1.f, 0.f, 1.f, 0.f);
-          const float a0 = x[4 * q] * rstd * wv.x, a1 = x[4 * q + 1] * rstd * wv.y;
-          const float b0 = x[4 * q + 2] * rstd * wv.z, b1 = x[4 * q + 3] * rstd * wv.w;
-          x[4 * q] = a0 * rc.x - a1 * rc.y;
-          x[4 * q + 1] = a0 * rc.y + a1 * rc.x;
-          x[4 * q + 2] = b0 * rc.z - b1 * rc.w;
-          x[4 * q + 3] = b0 * rc.w + b1 * rc.z;
+      for (int i = 0; i < 32; i += 2) gelu_tanh2(x[i], x[i + 1]);
+    } else if (EPI == RA_EPI_RESID) {
+      uint4 r[4];
+      rows_turn(w.stage, rnext, r);
+      if (j + 1 < CHUNKS) rows_fetch(res + 128 * (j + 1), 2 * sg.res_sr, w.nrow, rnext);
+      const float4* g4 = reinterpret_cast<const float4*>(w.vec1 + 32 * j);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t rw[4] = {r[q].x, r[q].y, r[q].z, r[q].w};
+        const float4 g0 = g4[2 * q], g1 = g4[2 * q + 1];
+        const float gv[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          x[8 * q + 2 * e] = fmaf(gv[2 * e], x[8 * q + 2 * e], __uint_as_float(rw[e] << 16));
+          x[8 * q + 2 * e + 1] = fmaf(gv[2 * e + 1], x[8 * q + 2 * e + 1], __uint_as_float(rw[e] & 0xFFFF0000u));
         }
-        if (valid) store32(drow + c0, x);
       }
     }
-  } else {
-    const int64_t orow = int64_t(tl.s) * sg.out_ss + int64_t(valid ? r : 0) * sg.out_sr;
-    // RESID: the row's residual for the next 32 columns is loaded while the
-    // current 32 are computed (one global-load latency per tile, not per chunk).
-    const bool resid = p.epi == RA_EPI_RESID && valid;
-    const uint4* rrow = resid ? reinterpret_cast<const uint4*>(sg.resid + int64_t(tl.s) * sg.res_ss +
-                                                               int64_t(r) * sg.res_sr + tl.n0)
-                              : nullptr;
-    uint4 rnext[4];
-    if (resid) {
+    rows_store(w.stage, x, out + 128 * j, 2 * sg.out_sr, w.nrow);
+  }
+  return true;
+}
+
+// QKV: heads half, half + 2, ... of the tile.
+template <int D, class Ready>
+__device__ __forceinline__ bool epilogue_qkv(const Params& p, const Tile& tl, const EpiWarp& w, Ready ready) {
+  constexpr int HEADS = BN / D / 2, CH = D / 32;
+  const Seg& sg = p.seg[tl.seg];
+  const int lane = threadIdx.x & 31;
+  const int part = tl.n0 / p.C;  // 0 q, 1 k, 2 v
+  const int h0 = (tl.n0 - part * p.C) / D + w.half;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) rnext[q] = rrow[q];
-    }
-    for (int c0 = 0; c0 < BN; c0 += 32) {
-      const int n = tl.n0 + c0;
-      uint4 rcur[4];
+  for (int j = 0; j < 4; ++j) {
+    const int c = 32 * (j % CH) + lane;  // column within head h0 + 2 (j / CH)
+    w.vec0[32 * j + lane] = sg.bias ? __ldg(sg.bias + part * p.C + (h0 + 2 * (j / CH)) * D + c) : 0.f;
+    if (part < 2) w.vec1[32 * j + lane] = __ldg(sg.norm_w[part] + c);
+  }
+  __syncwarp();
+  // RoPE rows of the warp's positions: (cos, sin) of D / 2 pairs, 64 bytes = 16 columns at a time
+  const char* rope = reinterpret_cast<const char*>(p.rope + int64_t(sg.pos_offset + w.row0) * (D / 4));
+  uint4 cnext[4];
+  if (part < 2) rows_fetch(rope, 4 * D, w.nrow, cnext);
+  if (!ready()) return false;
+  if (w.nrow <= 0) return true;
+  char* dst0 = reinterpret_cast<char*>(sg.dst[part] + tl.s * sg.dst_sb[part] + int64_t(w.row0) * sg.dst_sn[part]);
+#pragma unroll 1
+  for (int hh = 0; hh < HEADS; ++hh) {
+    const uint32_t acc = w.acc + (w.half + 2 * hh) * D;
+    const float* bias = w.vec0 + 32 * CH * hh;
+    const float* nw = w.vec1 + 32 * CH * hh;
+    uint32_t v[32];
+    float rstd = 0.f;
+    tmem_ld32(acc, v);
+    if (part < 2) {
+      // a first pass over the head's accumulators for the mean square
+      float s0 = 0.f, s1 = 0.f;
+#pragma unroll 1
+      for (int c = 0; c < CH; ++c) {
+        float x[32];
+        tmem_ld_wait_for(v);
+        add_cols(v, bias + 32 * c, x);
+        tmem_ld32(acc + 32 * ((c + 1) % CH), v);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) rcur[q] = rnext[q];
-      if (resid && c0 + 32 < BN) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) rnext[q] = rrow[(c0 + 32) / 8 + q];
+        for (int i = 0; i < 32; i += 2) {
+          s0 = fmaf(x[i], x[i], s0);
+          s1 = fmaf(x[i + 1], x[i + 1], s1);
+        }
       }
+      rstd = rsqrtf((s0 + s1) / float(D) + p.norm_eps);
+    }
+    char* dst = dst0 + 2 * int64_t(h0 + 2 * hh) * sg.dst_sh[part];
+#pragma unroll 1
+    for (int c = 0; c < CH; ++c) {
       float x[32];
-      load_acc(base + c0, sg.bias, n, x);
-      if (p.epi == RA_EPI_GELU) {
+      tmem_ld_wait_for(v);
+      add_cols(v, bias + 32 * c, x);
+      if (c + 1 < CH) tmem_ld32(acc + 32 * (c + 1), v);
+      if (part < 2) {
 #pragma unroll
-        for (int j = 0; j < 32; ++j) x[j] = gelu_tanh(x[j]);
-      } else if (resid) {
-        const float4* gp = reinterpret_cast<const float4*>(sg.gate + int64_t(tl.s) * sg.gate_ss + n);
+        for (int hf = 0; hf < 2; ++hf) {
+          uint4 own[4];
+          rows_turn(w.stage, cnext, own);
+          // the next 16 columns' table entries (the next head starts over)
+          const int nx = (2 * c + hf + 1) % (2 * CH);
+          if (nx != 0 || hh + 1 < HEADS) rows_fetch(rope + 64 * nx, 4 * D, w.nrow, cnext);
+          const float4* w4 = reinterpret_cast<const float4*>(nw + 32 * c + 16 * hf);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const uint4 rv = rcur[q];
-          const uint32_t w4[4] = {rv.x, rv.y, rv.z, rv.w};
-          const float4 g0 = __ldg(gp + 2 * q), g1 = __ldg(gp + 2 * q + 1);
-          const float gv[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float lo = __uint_as_float(w4[e] << 16), hi = __uint_as_float(w4[e] & 0xFFFF0000u);
-            x[8 * q + 2 * e] = fmaf(gv[2 * e], x[8 * q + 2 * e], lo);
-            x[8 * q + 2 * e + 1] = fmaf(gv[2 * e + 1], x[8 * q + 2 * e + 1], hi);
+          for (int q = 0; q < 4; ++q) {
+            const float4 wv = w4[q];
+            const float cs[4] = {__uint_as_float(own[q].x), __uint_as_float(own[q].y), __uint_as_float(own[q].z),
+                                 __uint_as_float(own[q].w)};
+            float* xe = &x[16 * hf + 4 * q];
+            const float a0 = xe[0] * rstd * wv.x, a1 = xe[1] * rstd * wv.y;
+            const float b0 = xe[2] * rstd * wv.z, b1 = xe[3] * rstd * wv.w;
+            xe[0] = a0 * cs[0] - a1 * cs[1];
+            xe[1] = a0 * cs[1] + a1 * cs[0];
+            xe[2] = b0 * cs[2] - b1 * cs[3];
+            xe[3] = b0 * cs[3] + b1 * cs[2];
           }
         }
       }
-      if (valid) store32(sg.out + orow + n, x);
+      rows_store(w.stage, x, dst + 64 * c, 2 * sg.dst_sn[part], w.nrow);
     }
-  }}
+  }
+  return true;
+}
 
+// Epilogue of one warp's share of an output tile; ready() waits for the
+// accumulator (false: the wait was given up). D: head dim (QKV).
+template <int EPI, int D, class Ready>
+__device__ __forceinline__ bool epilogue_tile(const Params& p, const Tile& tl, const EpiWarp& w, Ready ready) {
+  if constexpr (EPI == RA_EPI_QKV)
+    return epilogue_qkv<D>(p, tl, w, ready);
+  else
+    return epilogue_linear<EPI>(p, tl, w, ready);
+}
+
+template <int EPI, int D>
 __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant__ Params p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -302,7 +410,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(tfull + b, 1);
-      mbar_init(tempty + b, 4);
+      mbar_init(tempty + b, EPI_WARPS);
     }
     mbar_init(drain, 1);
     *abort_flag = 0;
@@ -326,7 +434,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
       int64_t it = 0;  // K steps issued
       bool ok = true;
       for (int64_t t = blockIdx.x; ok && t < p.total_tiles; t += gridDim.x) {
-        const Tile tl = decode<BM>(p, t);
+        const Tile tl = decode<BM, EPI>(p, t);
         if (!tl.live) continue;
         for (int kb = 0; kb < p.kblocks; ++kb, ++it) {
           const int st = int(it % STAGES);
@@ -353,7 +461,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
       int i = 0;
       bool ok = true, issued = false;
       for (int64_t t = blockIdx.x; ok && t < p.total_tiles; t += gridDim.x) {
-        const Tile tl = decode<BM>(p, t);
+        const Tile tl = decode<BM, EPI>(p, t);
         if (!tl.live) continue;
         const int buf = i & 1, use = i >> 1;
         if (use > 0 && !(ok = mbar_wait(tempty + buf, uint32_t((use - 1) & 1), ctl))) break;
@@ -383,16 +491,25 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
   } else {
     // ---------------------------------------------------------------- epilogue
     const int quarter = warp & 3;
-    const int row = quarter * 32 + lane;
-    const uint32_t lane_off = uint32_t(quarter * 32) << 16;
+    EpiWarp w;
+    w.half = (warp - 2) >> 2;
+    w.stage = smem + OFF_EPI + (warp - 2) * EPI_WARP_BYTES;
+    w.vec0 = reinterpret_cast<float*>(w.stage + EPI_STAGE_BYTES);
+    w.vec1 = w.vec0 + 128;
     int i = 0;
     for (int64_t t = blockIdx.x; t < p.total_tiles; t += gridDim.x) {
-      const Tile tl = decode<BM>(p, t);
+      const Tile tl = decode<BM, EPI>(p, t);
       if (!tl.live) continue;
       const int buf = i & 1, use = i >> 1;
-      if (!__all_sync(0xffffffffu, mbar_wait(tfull + buf, uint32_t(use & 1), ctl))) break;
-      tc_fence_after();
-      epilogue_tile(p, tl, tl.m0 + row, tmem + lane_off + uint32_t(buf * BN));
+      w.row0 = tl.m0 + quarter * 32;
+      w.nrow = min(32, p.seg[tl.seg].rows - w.row0);
+      w.acc = tmem + (uint32_t(quarter * 32) << 16) + uint32_t(buf * BN);
+      if (!epilogue_tile<EPI, D>(p, tl, w, [&] {
+            const bool ok = __all_sync(0xffffffffu, mbar_wait(tfull + buf, uint32_t(use & 1), ctl));
+            tc_fence_after();
+            return ok;
+          }))
+        break;
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty + buf);
@@ -415,8 +532,9 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
 // bytes). Rank 0's MMA thread issues M = 256, N = 256 MMAs; commits are
 // multicast to both CTAs (stage free, accumulator ready). Each CTA's epilogue
 // reads its own TMEM rows and arrives on rank 0's accumulator-free barrier
-// (count 8). The two CTAs meet at a cluster barrier before TMEM is freed and
+// (count 16). The two CTAs meet at a cluster barrier before TMEM is freed and
 // before either exits, so no remote arrive or MMA outlives its target.
+template <int EPI, int D>
 __global__ void __launch_bounds__(THREADS, 1) gemm_pair_kernel(const __grid_constant__ Params p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -438,7 +556,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_pair_kernel(const __grid_cons
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(tfull + b, 1);
-      mbar_init(tempty + b, 8);
+      mbar_init(tempty + b, 2 * EPI_WARPS);
     }
     mbar_init(drain, 1);
     *abort_flag = 0;
@@ -464,7 +582,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_pair_kernel(const __grid_cons
       int64_t it = 0;
       bool ok = true;
       for (int64_t t = cid; ok && t < p.total_tiles; t += ncl) {
-        const Tile tl = decode<P_TM>(p, t);
+        const Tile tl = decode<P_TM, EPI>(p, t);
         if (!tl.live) continue;
         for (int kb = 0; kb < (p.kblocks + 1) / 2; ++kb, ++it) {
           const int st = int(it % P_STAGES);
@@ -504,7 +622,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_pair_kernel(const __grid_cons
       int i = 0;
       bool ok = true, issued = false;
       for (int64_t t = cid; ok && t < p.total_tiles; t += ncl) {
-        const Tile tl = decode<P_TM>(p, t);
+        const Tile tl = decode<P_TM, EPI>(p, t);
         if (!tl.live) continue;
         const int buf = i & 1, use = i >> 1;
         if (use > 0 && !(ok = mbar_wait_cluster(tempty + buf, uint32_t((use - 1) & 1), ctl))) break;
@@ -538,17 +656,26 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_pair_kernel(const __grid_cons
   } else {
     // ---------------------------------------------------------------- epilogue (both CTAs)
     const int quarter = warp & 3;
-    const int row = int(rank) * 128 + quarter * 32 + lane;
-    const uint32_t lane_off = uint32_t(quarter * 32) << 16;
+    EpiWarp w;
+    w.half = (warp - 2) >> 2;
+    w.stage = smem + P_OFF_EPI + (warp - 2) * EPI_WARP_BYTES;
+    w.vec0 = reinterpret_cast<float*>(w.stage + EPI_STAGE_BYTES);
+    w.vec1 = w.vec0 + 128;
     const uint32_t tempty0 = mapa_shared(smem_u32(tempty), 0);
     int i = 0;
     for (int64_t t = cid; t < p.total_tiles; t += ncl) {
-      const Tile tl = decode<P_TM>(p, t);
+      const Tile tl = decode<P_TM, EPI>(p, t);
       if (!tl.live) continue;
       const int buf = i & 1, use = i >> 1;
-      if (!__all_sync(0xffffffffu, mbar_wait(tfull + buf, uint32_t(use & 1), ctl))) break;
-      tc_fence_after();
-      epilogue_tile(p, tl, tl.m0 + row, tmem + lane_off + uint32_t(buf * BN));
+      w.row0 = tl.m0 + int(rank) * 128 + quarter * 32;
+      w.nrow = min(32, p.seg[tl.seg].rows - w.row0);
+      w.acc = tmem + (uint32_t(quarter * 32) << 16) + uint32_t(buf * BN);
+      if (!epilogue_tile<EPI, D>(p, tl, w, [&] {
+            const bool ok = __all_sync(0xffffffffu, mbar_wait(tfull + buf, uint32_t(use & 1), ctl));
+            tc_fence_after();
+            return ok;
+          }))
+        break;
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
@@ -577,6 +704,22 @@ __global__ void rope_table_kernel(float* table, int32_t n_pos, int32_t d, double
     sincos(ang, &s, &c);
     table[2 * i] = float(c);
     table[2 * i + 1] = float(s);
+  }
+}
+
+// The kernels by epilogue (QKV: by head dim too), one CTA per tile and CTA pairs.
+using Kernel = void (*)(Params);
+struct Kernels {
+  Kernel single, pair;
+};
+Kernels pick(int epi, int d) {
+  switch (epi) {
+    case RA_EPI_STORE: return {gemm_kernel<RA_EPI_STORE, 0>, gemm_pair_kernel<RA_EPI_STORE, 0>};
+    case RA_EPI_GELU: return {gemm_kernel<RA_EPI_GELU, 0>, gemm_pair_kernel<RA_EPI_GELU, 0>};
+    case RA_EPI_RESID: return {gemm_kernel<RA_EPI_RESID, 0>, gemm_pair_kernel<RA_EPI_RESID, 0>};
+    default:
+      return d == 128 ? Kernels{gemm_kernel<RA_EPI_QKV, 128>, gemm_pair_kernel<RA_EPI_QKV, 128>}
+                      : Kernels{gemm_kernel<RA_EPI_QKV, 64>, gemm_pair_kernel<RA_EPI_QKV, 64>};
   }
 }
 
@@ -742,14 +885,14 @@ extern "C" ra_status refadapt_gemm(const ra_gemm_args* a, void* stream) {
   }
   p.total_tiles = tiles;
   if (tiles == 0) return RA_OK;
-  ra_status as = ensure_dynamic_smem(reinterpret_cast<const void*>(gemm_kernel), SMEM_ALLOC, "refadapt_gemm");
-  if (as == RA_OK)
-    as = ensure_dynamic_smem(reinterpret_cast<const void*>(gemm_pair_kernel), P_SMEM_ALLOC, "refadapt_gemm");
+  const Kernels kn = pick(a->epilogue, a->d);
+  const ra_status as = ensure_dynamic_smem(reinterpret_cast<const void*>(pair ? kn.pair : kn.single),
+                                           pair ? P_SMEM_ALLOC : SMEM_ALLOC, "refadapt_gemm");
   if (as != RA_OK) return as;
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (!pair) {
     const int64_t grid = tiles < sms ? tiles : sms;
-    gemm_kernel<<<unsigned(grid), THREADS, SMEM_ALLOC, st>>>(p);
+    kn.single<<<unsigned(grid), THREADS, SMEM_ALLOC, st>>>(p);
     return launch_status("refadapt_gemm");
   }
   const int64_t clusters = tiles < sms / 2 ? tiles : (sms / 2 > 0 ? sms / 2 : 1);
@@ -766,7 +909,7 @@ extern "C" ra_status refadapt_gemm(const ra_gemm_args* a, void* stream) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_pair_kernel, p);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kn.pair, p);
   if (e != cudaSuccess) {
     set_error("refadapt_gemm: pair launch failed: %s", cudaGetErrorString(e));
     cudaGetLastError();
