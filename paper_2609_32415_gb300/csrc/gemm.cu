@@ -5,13 +5,13 @@
 //   D[r, n] = sum_k A[r, k] W[n, k]        (A rows of one segment and sample,
 //                                           W in nn.Linear layout [N][K])
 //
-// Two kernels: CTA pairs on 256 x 256 output tiles (gemm_pair_kernel, below,
-// used when a call has at least a wave of such tiles) and one CTA per SM on
-// 128 x 256 tiles (gemm_kernel), both persistent, K in 64-column steps. Tiles
-// are numbered segment-major, then sample, then in bands of GROUP_M row tiles,
-// rows fastest inside a band (so the CTAs that run at once share a few A row
-// blocks and a few W column blocks, both held in L2); CTA c takes tiles c,
-// c + G, c + 2G, ...
+// Two kernels: CTA pairs on 256-row output tiles (gemm_pair_kernel, below) and
+// one CTA per SM on 128-row tiles (gemm_kernel), both persistent, tiles up to
+// 256 columns wide; make_plan() picks the kernel and the width. Live tiles
+// (those the modes do not skip) are numbered segment-major, then sample, then
+// in bands of GROUP_M row tiles, rows fastest inside a band (so the CTAs that
+// run at once share a few A row blocks and a few W column blocks, both held in
+// L2); CTA c takes tiles c, c + G, c + 2G, ...
 //   warp 0      TMA producer: per K step one 128 x 64 A box and one 256 x 64 W
 //               box (128-byte swizzle, rows past a segment's end read as
 //               zeros) into a 4-stage ring.
@@ -73,8 +73,8 @@ constexpr int THREADS = 64 + 32 * EPI_WARPS;
 constexpr int TMEM_COLS = 512;
 static_assert(SMEM_ALLOC <= 232448, "shared memory budget");
 
-// CTA-pair kernel: 256 x 256 output tiles; each CTA stages its 128 rows of A
-// and its 128-column half of the W tile, 128 of K per stage (two 128-byte
+// CTA-pair kernel: 256-row output tiles; each CTA stages its 128 rows of A
+// and its half of the W tile (up to 128 columns), 128 of K per stage (two 128-byte
 // swizzle chunks per operand, 64 KB per stage, 3 stages): half the stage
 // hand-offs of 64-wide stages, which the fused epilogues gained from (GELU
 // +3 %); a K % 128 == 64 tail is a half stage.
@@ -94,7 +94,6 @@ constexpr int P_SMEM_ALLOC = P_SMEM_BYTES + 1024;
 static_assert(P_SMEM_ALLOC <= 232448, "shared memory budget");
 
 struct Seg {
-  int64_t tile_begin;
   int32_t rows, m_tiles, gated, pos_offset;
   const float* bias;
   __nv_bfloat16* out;
@@ -111,8 +110,8 @@ struct Seg {
 struct Params {
   CUtensorMap tm_a[3], tm_w[3];
   Seg seg[3];
-  int32_t n_seg, B, N, K, epi, H, d, C, n_tiles_n, kblocks;
-  int64_t total_tiles;
+  int32_t n_seg, B, N, K, C, kblocks;
+  int32_t bn;          // columns of a tile
   const int32_t* mode;
   const float4* rope;  // [pos][d/4]: (cos, sin) of two consecutive pairs
   int32_t rope_len;
@@ -123,41 +122,54 @@ struct Params {
 
 struct Tile {
   int seg, s, m0, n0;
-  bool live;
 };
 
 constexpr int GROUP_M = 16;  // tile rows per band of the tile order
 
+// Walks the live tiles in order; tile indices only grow. A piece is the tiles
+// of one (segment, sample): all column tiles, or none when the segment is gated
+// and the sample reuses, or only the query's (QKV at the boundary, which keeps
+// its cached K and V).
 template <int TM, int EPI>  // TM: output rows per tile, 128 (one CTA) or 256 (a CTA pair)
-__device__ __forceinline__ Tile decode(const Params& p, int64_t t) {
-  Tile r;
-  int g = 0;
-  while (g + 1 < p.n_seg && t >= p.seg[g + 1].tile_begin) ++g;
-  const Seg& sg = p.seg[g];
-  const int64_t local = t - sg.tile_begin;
-  const int64_t per_sample = int64_t(sg.m_tiles) * p.n_tiles_n;
-  r.seg = g;
-  r.s = int(local / per_sample);
-  const int64_t rem = local - int64_t(r.s) * per_sample;
-  // Grouped order: bands of GROUP_M tile rows, rows fastest inside a band, so
-  // the tiles in flight at once (one per CTA pair) share a few A row blocks
-  // and a few W column blocks that stay in L2, and W streams from HBM once per
-  // band instead of once per wave.
-  const int64_t band_tiles = int64_t(GROUP_M) * p.n_tiles_n;
-  const int band = int(rem / band_tiles);
-  const int m_first = band * GROUP_M;
-  const int rows = min(GROUP_M, sg.m_tiles - m_first);
-  const int idx = int(rem - int64_t(band) * band_tiles);
-  r.m0 = (m_first + idx % rows) * TM;
-  r.n0 = (idx / rows) * BN;
-  r.live = true;
-  if (sg.gated) {
-    const int m = __ldg(p.mode + r.s);
-    if (m == RA_MODE_REUSE) r.live = false;
-    if (EPI == RA_EPI_QKV && m == RA_MODE_BOUNDARY && r.n0 >= p.C) r.live = false;
+struct Walk {
+  int g = 0, s = 0, cols = -1;  // cols: column tiles of the piece
+  int64_t begin = 0;            // first tile of the piece
+
+  __device__ __forceinline__ int piece_cols(const Params& p) const {
+    if (p.seg[g].gated) {
+      const int m = __ldg(p.mode + s);
+      if (m == RA_MODE_REUSE) return 0;
+      if (EPI == RA_EPI_QKV && m == RA_MODE_BOUNDARY) return p.C / p.bn;
+    }
+    return (p.N + p.bn - 1) / p.bn;
   }
-  return r;
-}
+  // Tile t, or false past the last one.
+  __device__ __forceinline__ bool at(const Params& p, int64_t t, Tile& r) {
+    if (cols < 0) cols = piece_cols(p);
+    while (t - begin >= int64_t(p.seg[g].m_tiles) * cols) {
+      begin += int64_t(p.seg[g].m_tiles) * cols;
+      if (++s == p.B) {
+        s = 0;
+        if (++g == p.n_seg) return false;
+      }
+      cols = piece_cols(p);
+    }
+    r.seg = g;
+    r.s = s;
+    const uint32_t rem = uint32_t(t - begin);
+    // Grouped order: bands of GROUP_M tile rows, rows fastest inside a band, so
+    // the tiles in flight at once (one per CTA pair) share a few A row blocks
+    // and a few W column blocks that stay in L2, and W streams from HBM once per
+    // band instead of once per wave.
+    const uint32_t band_tiles = uint32_t(GROUP_M) * uint32_t(cols);
+    const uint32_t band = rem / band_tiles, idx = rem - band * band_tiles;
+    const int m_first = int(band) * GROUP_M;
+    const uint32_t rows = uint32_t(min(GROUP_M, p.seg[g].m_tiles - m_first));
+    r.m0 = (m_first + int(idx % rows)) * TM;
+    r.n0 = int(idx / rows) * p.bn;
+    return true;
+  }
+};
 
 // GELU, tanh form, of two values through the identity
 // 0.5 x (1 + tanh(u)) = x / (1 + e^(-2u)), u = sqrt(2/pi) (x + 0.044715 x^3),
@@ -245,39 +257,41 @@ __device__ __forceinline__ void add_cols(const uint32_t (&v)[32], const float* c
 // STORE, GELU, RESID: chunk j of the warp is tile columns 32 (half + 2 j) ...
 template <int EPI, class Ready>
 __device__ __forceinline__ bool epilogue_linear(const Params& p, const Tile& tl, const EpiWarp& w, Ready ready) {
-  constexpr int CHUNKS = BN / 64;
   const Seg& sg = p.seg[tl.seg];
   const int lane = threadIdx.x & 31, n0 = tl.n0 + 32 * w.half;
+  // this warp's; the last tile of a row may reach past N (a multiple of 32)
+  const int chunks = (min(p.bn, p.N - tl.n0) / 32 + 1 - w.half) >> 1;
 #pragma unroll
-  for (int j = 0; j < CHUNKS; ++j) {
+  for (int j = 0; j < 4; ++j) {
+    if (j >= chunks) break;
     w.vec0[32 * j + lane] = sg.bias ? __ldg(sg.bias + n0 + 64 * j + lane) : 0.f;
     if (EPI == RA_EPI_RESID) w.vec1[32 * j + lane] = __ldg(sg.gate + int64_t(tl.s) * sg.gate_ss + n0 + 64 * j + lane);
   }
   const char* res = nullptr;
   uint4 rnext[4];
-  if (EPI == RA_EPI_RESID) {
+  if (EPI == RA_EPI_RESID && chunks > 0) {
     res = reinterpret_cast<const char*>(sg.resid + int64_t(tl.s) * sg.res_ss + int64_t(w.row0) * sg.res_sr + n0);
     rows_fetch(res, 2 * sg.res_sr, w.nrow, rnext);
   }
   char* out = reinterpret_cast<char*>(sg.out + int64_t(tl.s) * sg.out_ss + int64_t(w.row0) * sg.out_sr + n0);
   __syncwarp();
   if (!ready()) return false;
-  if (w.nrow <= 0) return true;
+  if (w.nrow <= 0 || chunks <= 0) return true;
   uint32_t v[32];
   tmem_ld32(w.acc + 32 * w.half, v);
 #pragma unroll 1
-  for (int j = 0; j < CHUNKS; ++j) {
+  for (int j = 0; j < chunks; ++j) {
     float x[32];
     tmem_ld_wait_for(v);
     add_cols(v, w.vec0 + 32 * j, x);
-    if (j + 1 < CHUNKS) tmem_ld32(w.acc + 32 * w.half + 64 * (j + 1), v);
+    if (j + 1 < chunks) tmem_ld32(w.acc + 32 * w.half + 64 * (j + 1), v);
     if (EPI == RA_EPI_GELU) {
 #pragma unroll
       for (int i = 0; i < 32; i += 2) gelu_tanh2(x[i], x[i + 1]);
     } else if (EPI == RA_EPI_RESID) {
       uint4 r[4];
       rows_turn(w.stage, rnext, r);
-      if (j + 1 < CHUNKS) rows_fetch(res + 128 * (j + 1), 2 * sg.res_sr, w.nrow, rnext);
+      if (j + 1 < chunks) rows_fetch(res + 128 * (j + 1), 2 * sg.res_sr, w.nrow, rnext);
       const float4* g4 = reinterpret_cast<const float4*>(w.vec1 + 32 * j);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -299,13 +313,15 @@ __device__ __forceinline__ bool epilogue_linear(const Params& p, const Tile& tl,
 // QKV: heads half, half + 2, ... of the tile.
 template <int D, class Ready>
 __device__ __forceinline__ bool epilogue_qkv(const Params& p, const Tile& tl, const EpiWarp& w, Ready ready) {
-  constexpr int HEADS = BN / D / 2, CH = D / 32;
+  constexpr int CH = D / 32;
+  const int heads = (p.bn / D + 1 - w.half) >> 1;  // this warp's
   const Seg& sg = p.seg[tl.seg];
   const int lane = threadIdx.x & 31;
   const int part = tl.n0 / p.C;  // 0 q, 1 k, 2 v
   const int h0 = (tl.n0 - part * p.C) / D + w.half;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
+    if (j / CH >= heads) break;
     const int c = 32 * (j % CH) + lane;  // column within head h0 + 2 (j / CH)
     w.vec0[32 * j + lane] = sg.bias ? __ldg(sg.bias + part * p.C + (h0 + 2 * (j / CH)) * D + c) : 0.f;
     if (part < 2) w.vec1[32 * j + lane] = __ldg(sg.norm_w[part] + c);
@@ -316,10 +332,10 @@ __device__ __forceinline__ bool epilogue_qkv(const Params& p, const Tile& tl, co
   uint4 cnext[4];
   if (part < 2) rows_fetch(rope, 4 * D, w.nrow, cnext);
   if (!ready()) return false;
-  if (w.nrow <= 0) return true;
+  if (w.nrow <= 0 || heads <= 0) return true;
   char* dst0 = reinterpret_cast<char*>(sg.dst[part] + tl.s * sg.dst_sb[part] + int64_t(w.row0) * sg.dst_sn[part]);
 #pragma unroll 1
-  for (int hh = 0; hh < HEADS; ++hh) {
+  for (int hh = 0; hh < heads; ++hh) {
     const uint32_t acc = w.acc + (w.half + 2 * hh) * D;
     const float* bias = w.vec0 + 32 * CH * hh;
     const float* nw = w.vec1 + 32 * CH * hh;
@@ -357,7 +373,7 @@ __device__ __forceinline__ bool epilogue_qkv(const Params& p, const Tile& tl, co
           rows_turn(w.stage, cnext, own);
           // the next 16 columns' table entries (the next head starts over)
           const int nx = (2 * c + hf + 1) % (2 * CH);
-          if (nx != 0 || hh + 1 < HEADS) rows_fetch(rope + 64 * nx, 4 * D, w.nrow, cnext);
+          if (nx != 0 || hh + 1 < heads) rows_fetch(rope + 64 * nx, 4 * D, w.nrow, cnext);
           const float4* w4 = reinterpret_cast<const float4*>(nw + 32 * c + 16 * hf);
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
@@ -433,14 +449,14 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
         }
       int64_t it = 0;  // K steps issued
       bool ok = true;
-      for (int64_t t = blockIdx.x; ok && t < p.total_tiles; t += gridDim.x) {
-        const Tile tl = decode<BM, EPI>(p, t);
-        if (!tl.live) continue;
+      Walk<BM, EPI> walk;
+      Tile tl;
+      for (int64_t t = blockIdx.x; ok && walk.at(p, t, tl); t += gridDim.x) {
         for (int kb = 0; kb < p.kblocks; ++kb, ++it) {
           const int st = int(it % STAGES);
           if (it >= STAGES && !(ok = mbar_wait(empty + st, uint32_t((it / STAGES - 1) & 1), ctl))) break;
           uint8_t* sa = smem + st * STAGE_BYTES;
-          mbar_arrive_expect_tx(full + st, STAGE_BYTES);
+          mbar_arrive_expect_tx(full + st, A_BYTES + p.bn * BK * 2);
           tma_load_4d(sa, &p.tm_a[tl.seg], full + st, kb * BK, tl.m0, 0, tl.s);
           tma_load_4d(sa + A_BYTES, &p.tm_w[tl.seg], full + st, kb * BK, tl.n0, 0, 0);
         }
@@ -455,14 +471,14 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
   } else if (warp == 1) {
     if (lane == 0) {
       // -------------------------------------------------------------- MMA issuer
-      constexpr uint32_t IDESC = idesc_bf16_f32(BM, BN, 0, 0);
+      const uint32_t idesc = idesc_bf16_f32(BM, p.bn, 0, 0);
       const uint32_t s0 = smem_u32(smem);
       int64_t it = 0;
       int i = 0;
       bool ok = true, issued = false;
-      for (int64_t t = blockIdx.x; ok && t < p.total_tiles; t += gridDim.x) {
-        const Tile tl = decode<BM, EPI>(p, t);
-        if (!tl.live) continue;
+      Walk<BM, EPI> walk;
+      Tile tl;
+      for (int64_t t = blockIdx.x; ok && walk.at(p, t, tl); t += gridDim.x) {
         const int buf = i & 1, use = i >> 1;
         if (use > 0 && !(ok = mbar_wait(tempty + buf, uint32_t((use - 1) & 1), ctl))) break;
         tc_fence_after();
@@ -474,7 +490,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
           const uint32_t sa = s0 + st * STAGE_BYTES, sb = sa + A_BYTES;
 #pragma unroll
           for (int kk = 0; kk < BK / 16; ++kk)
-            umma_ss(d_t, sdesc_sw128(sa + kk * 32, 16, 1024), sdesc_sw128(sb + kk * 32, 16, 1024), IDESC,
+            umma_ss(d_t, sdesc_sw128(sa + kk * 32, 16, 1024), sdesc_sw128(sb + kk * 32, 16, 1024), idesc,
                     (kb > 0 || kk > 0) ? 1u : 0u);
           umma_commit(empty + st);
           issued = true;
@@ -497,9 +513,9 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
     w.vec0 = reinterpret_cast<float*>(w.stage + EPI_STAGE_BYTES);
     w.vec1 = w.vec0 + 128;
     int i = 0;
-    for (int64_t t = blockIdx.x; t < p.total_tiles; t += gridDim.x) {
-      const Tile tl = decode<BM, EPI>(p, t);
-      if (!tl.live) continue;
+    Walk<BM, EPI> walk;
+    Tile tl;
+    for (int64_t t = blockIdx.x; walk.at(p, t, tl); t += gridDim.x) {
       const int buf = i & 1, use = i >> 1;
       w.row0 = tl.m0 + quarter * 32;
       w.nrow = min(32, p.seg[tl.seg].rows - w.row0);
@@ -581,20 +597,20 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_pair_kernel(const __grid_cons
       const uint32_t full0 = mapa_shared(smem_u32(full), 0);  // rank 0's full barriers
       int64_t it = 0;
       bool ok = true;
-      for (int64_t t = cid; ok && t < p.total_tiles; t += ncl) {
-        const Tile tl = decode<P_TM, EPI>(p, t);
-        if (!tl.live) continue;
+      Walk<P_TM, EPI> walk;
+      Tile tl;
+      for (int64_t t = cid; ok && walk.at(p, t, tl); t += ncl) {
         for (int kb = 0; kb < (p.kblocks + 1) / 2; ++kb, ++it) {
           const int st = int(it % P_STAGES);
           if (it >= P_STAGES && !(ok = mbar_wait(empty + st, uint32_t((it / P_STAGES - 1) & 1), ctl))) break;
           uint8_t* sa = smem + st * P_STAGE_BYTES;
           const int chunks = (2 * kb + 1 < p.kblocks) ? 2 : 1;  // K % 128 == 64: the last stage is half
-          if (rank == 0) mbar_arrive_expect_tx(full + st, 4 * chunks * P_CHUNK);
+          if (rank == 0) mbar_arrive_expect_tx(full + st, chunks * (2 * P_CHUNK + p.bn * 128));
           for (int c = 0; c < chunks; ++c) {
             tma_load_4d_pair(sa + c * P_CHUNK, &p.tm_a[tl.seg], full0 + 8u * st, kb * P_BK + c * 64,
                              tl.m0 + int(rank) * 128, 0, tl.s);
             tma_load_4d_pair(sa + P_A_BYTES + c * P_CHUNK, &p.tm_w[tl.seg], full0 + 8u * st, kb * P_BK + c * 64,
-                             tl.n0 + int(rank) * 128, 0, 0);
+                             tl.n0 + int(rank) * (p.bn / 2), 0, 0);
           }
         }
       }
@@ -616,14 +632,14 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_pair_kernel(const __grid_cons
   } else if (warp == 1) {
     if (lane == 0 && rank == 0) {
       // -------------------------------------------------------------- MMA issuer (rank 0)
-      constexpr uint32_t IDESC = idesc_bf16_f32(P_TM, BN, 0, 0);
+      const uint32_t idesc = idesc_bf16_f32(P_TM, p.bn, 0, 0);
       const uint32_t s0 = smem_u32(smem);
       int64_t it = 0;
       int i = 0;
       bool ok = true, issued = false;
-      for (int64_t t = cid; ok && t < p.total_tiles; t += ncl) {
-        const Tile tl = decode<P_TM, EPI>(p, t);
-        if (!tl.live) continue;
+      Walk<P_TM, EPI> walk;
+      Tile tl;
+      for (int64_t t = cid; ok && walk.at(p, t, tl); t += ncl) {
         const int buf = i & 1, use = i >> 1;
         if (use > 0 && !(ok = mbar_wait_cluster(tempty + buf, uint32_t((use - 1) & 1), ctl))) break;
         tc_fence_after();
@@ -638,7 +654,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_pair_kernel(const __grid_cons
           for (int kk = 0; kk < P_BK / 16; ++kk) {
             if (kk >= ksteps) break;
             const uint32_t o = uint32_t((kk >> 2) * P_CHUNK + (kk & 3) * 32);
-            umma_ss_pair(d_t, sdesc_sw128(sa + o, 16, 1024), sdesc_sw128(sb + o, 16, 1024), IDESC,
+            umma_ss_pair(d_t, sdesc_sw128(sa + o, 16, 1024), sdesc_sw128(sb + o, 16, 1024), idesc,
                          (kb > 0 || kk > 0) ? 1u : 0u);
           }
           umma_commit_pair(empty + st, 0x3);
@@ -663,9 +679,9 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_pair_kernel(const __grid_cons
     w.vec1 = w.vec0 + 128;
     const uint32_t tempty0 = mapa_shared(smem_u32(tempty), 0);
     int i = 0;
-    for (int64_t t = cid; t < p.total_tiles; t += ncl) {
-      const Tile tl = decode<P_TM, EPI>(p, t);
-      if (!tl.live) continue;
+    Walk<P_TM, EPI> walk;
+    Tile tl;
+    for (int64_t t = cid; walk.at(p, t, tl); t += ncl) {
       const int buf = i & 1, use = i >> 1;
       w.row0 = tl.m0 + int(rank) * 128 + quarter * 32;
       w.nrow = min(32, p.seg[tl.seg].rows - w.row0);
@@ -725,6 +741,52 @@ Kernels pick(int epi, int d) {
 
 bool aligned16(const void* ptr) { return (reinterpret_cast<uintptr_t>(ptr) & 15u) == 0; }
 
+// How a call is cut into tiles: CTA pairs or single CTAs, and tile columns.
+struct Plan {
+  bool pair;
+  int bn;
+};
+
+// The cheapest cut by a model of the two kernels' time (microseconds), fitted to
+// single waves of 256 to 64 columns at K = 1024 and 4096 on a GB300 (each within
+// 6 %): what one round of tiles takes grows with the operand bytes a CTA stages
+// per K step (each is written to shared memory once and read once, which fills
+// its port before the tensor core is full), so a narrower tile costs nearly as
+// much as a wide one (256 columns 5.1 us per 1024 of K, 128 columns 4.0) and
+// pays only where it saves a round: 13 row tiles of 256 by N = 3072 make 156
+// tiles of 256 columns (three rounds of 76 pairs, the last one nearly empty;
+// 188 us at K = 12288) or 208 of 192 columns (three shorter rounds, 164 us).
+// Calls with gated segments are weighed with and without them.
+Plan make_plan(const ra_gemm_args& a, int sms) {
+  Plan best{false, 256};
+  double best_us = 1e30;
+  for (int pair = 0; pair < 2; ++pair) {
+    if ((a.tile_mode == 1 && pair) || (a.tile_mode == 2 && !pair) || (pair && sms < 2)) continue;
+    const int tm = pair ? P_TM : BM, slots = pair ? sms / 2 : sms;
+    for (int bn = 256; bn >= 64; bn -= 32) {
+      if (a.epilogue == RA_EPI_QKV && (bn % a.d != 0 || (a.H * a.d) % bn != 0)) continue;
+      const int64_t cols = (a.N + bn - 1) / bn;
+      int64_t all = 0, open = 0;  // tiles, and those of segments that are not gated
+      for (int g = 0; g < a.n_seg; ++g) {
+        const int64_t t = a.seg[g].rows > 0 ? int64_t(a.B) * ((a.seg[g].rows + tm - 1) / tm) * cols : 0;
+        all += t;
+        if (!a.seg[g].gated) open += t;
+      }
+      const double epilogue = 0.0085 * bn;  // of a tile, hidden behind the next one's MMAs
+      double round = a.K / 1024.0 * (pair ? 3.11 + 0.00766 * bn : 3.4 + 0.0127 * bn);
+      round = round > epilogue ? round : epilogue;
+      const double fixed = pair ? 4.4 + 0.0088 * bn : 3.6;
+      double us = fixed + round * double((all + slots - 1) / slots);
+      if (open > 0 && open < all) us += fixed + round * double((open + slots - 1) / slots);
+      if (us < best_us) {
+        best_us = us;
+        best = Plan{pair != 0, bn};
+      }
+    }
+  }
+  return best;
+}
+
 }  // namespace gemm
 }  // namespace ra
 
@@ -764,8 +826,6 @@ extern "C" ra_status refadapt_gemm(const ra_gemm_args* a, void* stream) {
   p.B = a->B;
   p.N = a->N;
   p.K = a->K;
-  p.epi = a->epilogue;
-  p.n_tiles_n = a->N / BN;
   p.kblocks = a->K / BK;
   p.mode = a->mode;
   p.err_word = a->err_word;
@@ -780,8 +840,6 @@ extern "C" ra_status refadapt_gemm(const ra_gemm_args* a, void* stream) {
       set_error("refadapt_gemm: QKV needs a 16-byte aligned rope table, rope_len >= 1 and norm_eps >= 0");
       return RA_EINVAL;
     }
-    p.H = a->H;
-    p.d = a->d;
     p.C = a->H * a->d;
     p.rope = reinterpret_cast<const float4*>(a->rope);
     p.rope_len = a->rope_len;
@@ -790,14 +848,12 @@ extern "C" ra_status refadapt_gemm(const ra_gemm_args* a, void* stream) {
     set_error("refadapt_gemm: tile_mode %d (0 auto, 1 one CTA per tile, 2 CTA pairs)", a->tile_mode);
     return RA_EINVAL;
   }
-  // One CTA per 128-row tile, or CTA pairs on 256-row tiles when there is a
-  // full wave of pair tiles (auto) or when asked.
-  int64_t pair_tiles = 0;
-  for (int g = 0; g < a->n_seg; ++g)
-    if (a->seg[g].rows > 0) pair_tiles += int64_t(a->B) * ((a->seg[g].rows + P_TM - 1) / P_TM) * p.n_tiles_n;
   const int sms = num_sms();
-  const bool pair = a->tile_mode == 2 || (a->tile_mode == 0 && sms >= 2 && pair_tiles >= sms / 2);
+  const Plan plan = make_plan(*a, sms);
+  const bool pair = plan.pair;
   const int tm = pair ? P_TM : BM;
+  p.bn = plan.bn;
+  const int64_t cols = (a->N + plan.bn - 1) / plan.bn;
   int64_t tiles = 0;
   for (int g = 0; g < a->n_seg; ++g) {
     const ra_gemm_seg& s = a->seg[g];
@@ -806,7 +862,6 @@ extern "C" ra_status refadapt_gemm(const ra_gemm_args* a, void* stream) {
       set_error("refadapt_gemm: seg %d rows < 0", g);
       return RA_EINVAL;
     }
-    d.tile_begin = tiles;
     d.rows = s.rows;
     d.m_tiles = (s.rows + tm - 1) / tm;
     d.gated = s.gated ? 1 : 0;
@@ -877,13 +932,16 @@ extern "C" ra_status refadapt_gemm(const ra_gemm_args* a, void* stream) {
     }
     ra_seg as{const_cast<void*>(s.a), s.a_stride_s, 0, s.a_stride_r, s.rows, 0};
     ra_seg ws{const_cast<void*>(s.w), 0, 0, a->K, a->N, 0};
-      // The pair kernel loads 128-row boxes of A and of W (each CTA its half).
+    // The pair kernel loads half a tile's rows of W per CTA.
     if (!encode_seg(&p.tm_a[g], as, a->B, 1, a->K, BK, BM, true) ||
-        !encode_seg(&p.tm_w[g], ws, 1, 1, a->K, BK, pair ? 128 : BN, true))
+        !encode_seg(&p.tm_w[g], ws, 1, 1, a->K, BK, pair ? plan.bn / 2 : plan.bn, true))
       return RA_EINVAL;
-    tiles += int64_t(a->B) * d.m_tiles * p.n_tiles_n;
+    if (int64_t(d.m_tiles) * cols > 2147483647) {
+      set_error("refadapt_gemm: seg %d: too many rows", g);
+      return RA_EINVAL;
+    }
+    tiles += int64_t(a->B) * d.m_tiles * cols;
   }
-  p.total_tiles = tiles;
   if (tiles == 0) return RA_OK;
   const Kernels kn = pick(a->epilogue, a->d);
   const ra_status as = ensure_dynamic_smem(reinterpret_cast<const void*>(pair ? kn.pair : kn.single),

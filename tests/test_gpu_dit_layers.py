@@ -154,17 +154,39 @@ def test_gemm_skips_gated_tiles_in_a_long_schedule(cuda_ok, tile_mode):
                gated=[False, True, False], modes=[COMPUTE, REUSE], tile_mode=tile_mode)
 
 
+# One row tile and just more columns than a round of the next narrower tiles
+# holds (76 pairs, 152 single CTAs): every tile width from 64 to 256, the last
+# tile of most of them reaching past N.
+@pytest.mark.parametrize("tile_mode,N", [(2, 512), (2, 5120), (2, 7424), (2, 9984), (2, 12288), (2, 14848),
+                                         (2, 17152), (1, 512), (1, 9984), (1, 14848)])
+@pytest.mark.parametrize("epi", ["gelu", "resid"])
+def test_gemm_tile_widths_match_oracle(cuda_ok, epi, tile_mode, N):
+    from paper_2609_32415_gb300._lib import RA_EPI_GELU, RA_EPI_RESID
+    _gemm_case(1, 512, N, [40], RA_EPI_GELU if epi == "gelu" else RA_EPI_RESID, torch.Generator().manual_seed(N),
+               tile_mode=tile_mode)
+
+
 @pytest.mark.parametrize("tile_mode", TILE_MODES)
 @pytest.mark.parametrize("H,d,modes", [(4, 64, [FULL, BOUNDARY]), (2, 128, [REUSE, COMPUTE])])
 def test_gemm_qkv_epilogue_matches_oracle(cuda_ok, H, d, modes, tile_mode):
     """QKV projection with per-head RMS norm and RoPE at the rows' joint
     positions; the reference segment is gated: REUSE writes nothing,
     BOUNDARY writes only its query (K/V stay the cached ones)."""
+    _qkv_case(H, d, modes, tile_mode, {"text": 37, "ref": 256, "tgt": 300})
+
+
+@pytest.mark.parametrize("tile_mode", TILE_MODES)
+@pytest.mark.parametrize("H,d,tgt", [(12, 64, 200), (12, 64, 700), (4, 64, 2100), (4, 64, 4500), (2, 128, 3500)])
+def test_gemm_qkv_wide_tiles_match_oracle(cuda_ok, H, d, tgt, tile_mode):
+    """Enough rows that tiles of one to four heads are picked."""
+    _qkv_case(H, d, [BOUNDARY, COMPUTE], tile_mode, {"text": 37, "ref": 300, "tgt": tgt})
+
+
+def _qkv_case(H, d, modes, tile_mode, n):
     from paper_2609_32415_gb300 import api
     from paper_2609_32415_gb300._lib import RA_EPI_QKV
     g = torch.Generator().manual_seed(H * d)
     B, C = 2, H * d
-    n = {"text": 37, "ref": 256, "tgt": 300}
     pos0 = {"text": 0, "ref": n["text"], "tgt": n["text"] + n["ref"]}
     rope = api.rope_table(sum(n.values()), d)
     mode = torch.tensor(modes, dtype=torch.int32, device="cuda")
