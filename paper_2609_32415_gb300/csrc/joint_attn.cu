@@ -1,8 +1,11 @@
 // refadapt_joint_attn: joint [text; reference; target] attention with the
 // per-tile reference mass, on tcgen05 tensor cores (sm_103a).
 //
-// One CTA computes a pair of 128-row Q tiles (A, B) of one role for one
-// (sample, head); both tiles share every K/V tile it streams:
+// One CTA computes an item: a pair of 128-row Q tiles (A, B) of one role for
+// one (sample, head), or one tile where that fits the launch in one round; both
+// tiles share every K/V tile it streams. Where items are too few for the SMs,
+// or leave a small rest after whole rounds, the CTAs of a cluster share an
+// item's keys (make_plan, merge_split):
 //   warp 0      TMA producer: Q tiles A and B once, then K and V tiles of the
 //               text, reference (cache slot) and target segments in that order
 //               into a STAGES-deep ring of 128-byte-swizzled shared buffers.
@@ -58,7 +61,10 @@ namespace attn {
 constexpr int BM = 128;  // query rows per tile (= TMEM lanes)
 constexpr int BN = 128;  // keys per tile
 constexpr int NUM_THREADS = 384;
+constexpr int MAX_SPLIT = 4;     // CTAs of a cluster that share one item's keys
+constexpr int MAX_SAMPLES = 32;  // samples per launch (one lane each)
 constexpr float kLog2e = 1.4426950408889634f;
+constexpr float kLowestMax = -1e30f;
 constexpr float kRescaleThresh = 8.0f;  // log2 units: p <= 2^8 between rescales
 
 template <int D>
@@ -71,27 +77,39 @@ struct Cfg {
   static constexpr int OFF_K = OFF_Q + 2 * TILE_BYTES;
   static constexpr int OFF_V = OFF_K + STAGES * TILE_BYTES;
   static constexpr int OFF_BAR = OFF_V + STAGES * TILE_BYTES;
-  // q_full, k_full[S], k_empty[S], v_full[S], v_empty[S], s_full[2], p_ready[2], o_done[2], drain
-  static constexpr int NUM_BARS = 1 + 4 * STAGES + 2 + 2 + 2 + 1;
+  // q_full, k_full[S], k_empty[S], v_full[S], v_empty[S], s_full[2], p_ready[2], o_done[2], drain, parts_full
+  static constexpr int NUM_BARS = 1 + 4 * STAGES + 2 + 2 + 2 + 1 + 1;
   static constexpr int OFF_MISC = OFF_BAR + NUM_BARS * 8;  // tmem slot, abort flag, 8 floats
-  static constexpr int SMEM_BYTES = OFF_MISC + 64;
+  static constexpr int OFF_ITEM = (OFF_MISC + 64 + 15) / 16 * 16;  // int4 per softmax warp
+  static constexpr int SMEM_BYTES = OFF_ITEM + 8 * 16;
   static constexpr int SMEM_ALLOC = SMEM_BYTES + 1024;  // slack for 1024-byte alignment
+  // Split launches: (m, l, l_ref) of every row from every rank of the cluster.
+  // The O parts to send and those received (up to 3/4 of 256 rows x D fp32
+  // each) reuse the tile buffers.
+  static constexpr int OFF_STATS = (SMEM_BYTES + 15) / 16 * 16;
+  static constexpr int SPLIT_BYTES = OFF_STATS + MAX_SPLIT * 2 * BM * 16;
+  static constexpr int SPLIT_ALLOC = SPLIT_BYTES + 1024;
+  static_assert(2 * (2 * BM * D * 4 / MAX_SPLIT) * (MAX_SPLIT - 1) <= OFF_BAR && 2 * BM * D * 4 <= OFF_BAR,
+                "O parts fit the tile buffers");
+  static_assert(SPLIT_ALLOC <= 232448, "shared memory budget");
   static constexpr uint32_t TMEM_COLS = 512;
   static constexpr uint32_t TM_S = 0, TM_O = 256;       // + 128 * tile
   static_assert(SMEM_ALLOC <= 232448, "shared memory budget");
 };
 
 struct Params {
-  CUtensorMap tm_q[3];
-  CUtensorMap tm_k[3];
-  CUtensorMap tm_v[3];
-  CUtensorMap tm_qf, tm_kf, tm_vf;  // this step's reference rows (fused cache update)
   __nv_bfloat16* o_ptr[3];
   int64_t o_sb[3], o_sh[3], o_sn[3];
   int32_t nq[3];  // query rows per role
   int32_t nk[3];  // key rows per role
   int32_t q_tiles[3];
-  int32_t q_blocks[3];  // pairs of Q tiles
+  int32_t q_blocks[3];  // items: groups of `group` Q tiles
+  int32_t group;        // Q tiles per item, 1 or 2
+  uint32_t per_inv[2];  // 2^32 / items per head, rounded up (with reference rows, without), or 0: divide
+  int32_t b0, nb;       // samples of this launch: [b0, b0 + nb)
+  int32_t part;         // PART_ALL, PART_ROUNDS or PART_REST of the live items
+  int32_t slots;        // CTAs of a full round
+  int32_t rest_max;     // largest rest that PART_REST takes
   int32_t kv_tiles[3];
   int32_t B, H;
   int32_t mass_rows;
@@ -108,7 +126,21 @@ struct Params {
   int32_t store_kv;  // ... and copy those K / V tiles into tm_k[1] / tm_v[1]
   int32_t store_q;   // ... and those Q tiles into tm_q[1]
   uint64_t budget_ns;
+  CUtensorMap tm_q[3];
+  CUtensorMap tm_k[3];
+  CUtensorMap tm_v[3];
+  CUtensorMap tm_qf, tm_kf, tm_vf;  // this step's reference rows (fused cache update)
 };
+
+// A launch runs all live items (reference items of reusing samples are not
+// live), or the whole rounds of them that fill the GPU, or the rest.
+enum { PART_ALL = 0, PART_ROUNDS = 1, PART_REST = 2 };
+
+// Live items in whole rounds, given all of them.
+__host__ __device__ __forceinline__ int round_items(int live, int slots, int rest_max) {
+  const int rest = live % slots;
+  return rest <= rest_max ? live - rest : live;
+}
 
 __device__ __forceinline__ bool refreshes(int m) { return m == RA_MODE_COMPUTE || m == RA_MODE_FULL; }
 
@@ -207,25 +239,114 @@ __device__ __forceinline__ float exp64_store(const float (&v)[64], int col0, int
   return (s0 + s1) + (s2 + s3);
 }
 
+__device__ __forceinline__ void wait_primary() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Merge of a split item (the softmax threads of every rank; thread = row of
+// tile t, rows of tile B follow A's). Each rank tells every other its row
+// maximum and sums; scales its O to the common maximum; keeps its own share of
+// the columns (D / nrank) and hands each other rank its share, by a bulk copy
+// between the CTAs' shared memory (plain remote stores took 15k cycles for
+// 128 KB). Then it adds the shares up in rank order, normalises and writes.
+// Leaves the item's l and l_ref in l, lref. Three cluster barriers: peers have
+// started (before the first remote store); statistics are there and every tile
+// buffer is idle; every part has arrived (the senders' buffers may go).
 template <int D>
+__device__ __forceinline__ void merge_split(const WaitCtl& ctl, uint8_t* smem, uint64_t* parts_full, uint32_t o_t,
+                                            bool ok, bool has_b, bool valid, int rank, int nrank, int t, int row,
+                                            float m, float& l, float& lref, __nv_bfloat16* orow) {
+  using C = Cfg<D>;
+  const int nrows = has_b ? 2 * BM : BM, lrow = t * BM + row;
+  const int cw = D / nrank;                         // columns per rank
+  const uint32_t part_bytes = uint32_t(nrows) * cw * 4;  // [column / 4][row] of 16 bytes
+  uint8_t* send = smem;                             // parts for the other ranks, in rank order
+  uint8_t* recv = smem + (nrank - 1) * part_bytes;  // parts from the other ranks, in rank order
+  const uint32_t stats = smem_u32(smem + C::OFF_STATS);
+  if (lrow == 0) mbar_arrive_expect_tx(parts_full, (nrank - 1) * part_bytes);
+  cluster_wait();
+  if (ok)
+    for (int q = 0; q < nrank; ++q)
+      st_cluster_f4(mapa_shared(stats, q) + uint32_t(rank * 2 * BM + lrow) * 16, m, l, lref, 0.f);
+  cluster_sync_all();
+  const float4* st = reinterpret_cast<const float4*>(smem + C::OFF_STATS) + lrow;
+  float scale = 0.f;
+  if (ok) {
+    float mx = st[0].x;
+    for (int r = 1; r < nrank; ++r) mx = fmaxf(mx, st[r * 2 * BM].x);
+    l = lref = 0.f;
+    for (int r = 0; r < nrank; ++r) {
+      const float4 v = st[r * 2 * BM];
+      const float a = ex2_approx(v.x - mx);
+      l = fmaf(v.y, a, l);
+      lref = fmaf(v.z, a, lref);
+    }
+    scale = ex2_approx(m - mx);
+    tc_fence_after();
+#pragma unroll 1
+    for (int c0 = 0; c0 < D; c0 += 16) {
+      const int q = c0 / cw;
+      if (q == rank) continue;
+      uint32_t v[16];
+      tmem_ld16(o_t + c0, v);
+      tmem_ld_wait();
+      float4* dst = reinterpret_cast<float4*>(send + (q - (q > rank ? 1 : 0)) * part_bytes) +
+                    ((c0 - q * cw) >> 2) * nrows + lrow;
+#pragma unroll
+      for (int i = 0; i < 16; i += 4)
+        dst[(i >> 2) * nrows] = make_float4(__uint_as_float(v[i]) * scale, __uint_as_float(v[i + 1]) * scale,
+                                            __uint_as_float(v[i + 2]) * scale, __uint_as_float(v[i + 3]) * scale);
+    }
+  }
+  fence_proxy_async_smem();  // the parts are next read by bulk copies
+  named_bar_sync(3, 256);
+  if (lrow == 0)
+    for (int q = 0; q < nrank; ++q)
+      if (q != rank)
+        bulk_copy_to_cta(mapa_shared(smem_u32(recv + (rank - (rank > q ? 1 : 0)) * part_bytes), q),
+                         send + (q - (q > rank ? 1 : 0)) * part_bytes, part_bytes,
+                         mapa_shared(smem_u32(parts_full), q));
+  const bool got = __all_sync(0xffffffffu, mbar_wait(parts_full, 0, ctl));
+  cluster_sync_all();
+  if (!ok || !got) return;
+  const float inv_l = 1.f / l;
+  for (int c0 = 0; c0 < cw; c0 += 16) {
+    uint32_t v[16];
+    float x[16];
+    tmem_ld16(o_t + rank * cw + c0, v);
+    tmem_ld_wait();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) x[i] = 0.f;
+    for (int r = 0; r < nrank; ++r) {
+      const float4* src = reinterpret_cast<const float4*>(recv + (r - (r > rank ? 1 : 0)) * part_bytes) +
+                          (c0 >> 2) * nrows + lrow;
+#pragma unroll
+      for (int i = 0; i < 16; i += 4) {
+        const float4 a = r == rank ? make_float4(__uint_as_float(v[i]) * scale, __uint_as_float(v[i + 1]) * scale,
+                                                 __uint_as_float(v[i + 2]) * scale, __uint_as_float(v[i + 3]) * scale)
+                                   : src[(i >> 2) * nrows];
+        x[i] += a.x, x[i + 1] += a.y, x[i + 2] += a.z, x[i + 3] += a.w;
+      }
+    }
+    if (valid) {
+      uint32_t pk[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) pk[i] = pack_bf16x2(x[2 * i] * inv_l, x[2 * i + 1] * inv_l);
+      uint4* dst = reinterpret_cast<uint4*>(orow + rank * cw + c0);
+      dst[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+      dst[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+    }
+  }
+}
+
+// SPLIT: a cluster of CTAs shares one item, each rank a contiguous range of
+// its key tiles; the ranks' partial results meet in distributed shared memory.
+template <int D, bool SPLIT>
 __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid_constant__ Params p) {
   using C = Cfg<D>;
   constexpr int S = C::STAGES;
-  const int b = blockIdx.z, h = blockIdx.y;
-  int qb = blockIdx.x, role;
-  if (qb < p.q_blocks[0]) {
-    role = 0;
-  } else if (qb - p.q_blocks[0] < p.q_blocks[1]) {
-    qb -= p.q_blocks[0];
-    role = 1;
-  } else {
-    qb -= p.q_blocks[0] + p.q_blocks[1];
-    role = 2;
-  }
-  const int mode = p.mode ? __ldg(p.mode + b) : int(RA_MODE_FULL);
-  if (role == 1 && mode == RA_MODE_REUSE) return;  // reference rows skipped (uniform exit)
-  const int tileA = 2 * qb;
-  const bool has_b = (tileA + 1) < p.q_tiles[role];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = SPLIT ? int(cluster_rank()) : 0, nrank = SPLIT ? int(cluster_size()) : 1;
+  const int lane_mode = (lane < p.nb && p.mode) ? __ldg(p.mode + p.b0 + lane) : int(RA_MODE_FULL);
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -239,11 +360,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
   uint64_t* p_ready = bars + 3 + 4 * S;  // [tile]
   uint64_t* o_done = bars + 5 + 4 * S;   // [tile]
   uint64_t* drain = bars + 7 + 4 * S;
+  uint64_t* parts_full = bars + 8 + 4 * S;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + C::OFF_MISC);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + C::OFF_MISC + 4);
   float* red = reinterpret_cast<float*>(smem + C::OFF_MISC + 16);  // [tile][quarter]
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
     for (int s = 0; s < S; ++s) {
@@ -258,6 +379,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
       mbar_init(o_done + t, 1);
     }
     mbar_init(drain, 1);
+    mbar_init(parts_full, 1);
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -266,8 +388,50 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  // The item (the modes have arrived during the set-up): live items are
+  // numbered sample-major, then head, then role and Q tiles (consecutive items
+  // share their K/V tiles in L2).
+  const uint32_t reuse = __ballot_sync(0xffffffffu, lane < p.nb && lane_mode == RA_MODE_REUSE);
+  const int per_reuse = p.q_blocks[0] + p.q_blocks[2];
+  int item = SPLIT ? int(blockIdx.x) / nrank : int(blockIdx.x);
+  {
+    const int live = p.H * (p.nb * per_reuse + (p.nb - __popc(reuse)) * p.q_blocks[1]);
+    const int rounds = p.part == PART_ALL ? live : round_items(live, p.slots, p.rest_max);
+    if (p.part == PART_REST) item += rounds;
+    if (item >= (p.part == PART_REST ? live : rounds)) {  // uniform over the cluster
+      if (warp == 1) tmem_dealloc(tmem, C::TMEM_COLS);
+      if (p.part == PART_REST && blockIdx.x == 0) wait_primary();
+      return;
+    }
+  }
+  int bl = 0, per = 0;
+  for (;; ++bl) {
+    per = per_reuse + ((reuse >> bl) & 1 ? 0 : p.q_blocks[1]);
+    if (item < p.H * per) break;
+    item -= p.H * per;
+  }
+  const int b = p.b0 + bl, mode = __shfl_sync(0xffffffffu, lane_mode, bl);
+  const uint32_t inv = p.per_inv[per == per_reuse ? 1 : 0];
+  const int h = inv ? int(__umulhi(uint32_t(item), inv)) : item / per;
+  const int first = item - h * per;  // 0: the first item of its (sample, head)
+  int qb = first, role;
+  const int n_ref_items = per - per_reuse;
+  if (qb < p.q_blocks[0]) {
+    role = 0;
+  } else if (qb - p.q_blocks[0] < n_ref_items) {
+    qb -= p.q_blocks[0];
+    role = 1;
+  } else {
+    qb -= p.q_blocks[0] + n_ref_items;
+    role = 2;
+  }
+  const int tileA = p.group * qb;
+  const bool has_b = p.group == 2 && (tileA + 1) < p.q_tiles[role];
+  if (SPLIT) cluster_arrive();  // this CTA has started: its shared memory exists
   const WaitCtl ctl{abort_flag, p.err_word, p.budget_ns};
-  const int nkv = p.kv_tiles[0] + p.kv_tiles[1] + p.kv_tiles[2];
+  const int nkv_all = p.kv_tiles[0] + p.kv_tiles[1] + p.kv_tiles[2];
+  const int j0 = SPLIT ? nkv_all * rank / nrank : 0;  // this CTA's first key tile
+  const int nkv = SPLIT ? nkv_all * (rank + 1) / nrank - j0 : nkv_all;
   // Register split: warpgroup 0 (producer, MMA issuer, two idle warps) gives
   // up registers to the two softmax warpgroups: 4 x 56 + 8 x 224 = 12 x 168,
   // the launch allocation.
@@ -277,10 +441,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
       if (lane == 0) {
         // ------------------------------------------------------------ TMA producer
         const bool fresh = p.fresh && refreshes(mode);
-        const bool store_kv = fresh && p.store_kv && blockIdx.x == 0;
-        const bool store_q = fresh && p.store_q && role == 1;
+        const bool store_kv = fresh && p.store_kv && first == 0;
+        const bool store_q = fresh && p.store_q && role == 1 && rank == 0;
         const CUtensorMap* tq = (role == 1 && fresh) ? &p.tm_qf : &p.tm_q[role];
-        if (fresh && blockIdx.x == 0 && h == 0 && p.a_b) p.a_b[b] = p.step;
+        if (fresh && first == 0 && h == 0 && rank == 0 && p.a_b) p.a_b[b] = p.step;
         tma_prefetch_desc(tq);
         for (int r = 0; r < 3; ++r)
           if (p.kv_tiles[r] > 0) {
@@ -304,7 +468,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
             q_stored = true;
           }
           int r, row0;
-          kv_tile(p, jj, r, row0);
+          kv_tile(p, j0 + jj, r, row0);
           if (!store_kv || r != 1) return true;
           const int s = jj % S;
           const uint32_t ph = (jj / S) & 1;
@@ -327,7 +491,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
           const int s = j % S;
           const uint32_t ph = (j / S) & 1;
           int r, row0;
-          kv_tile(p, j, r, row0);
+          kv_tile(p, j0 + j, r, row0);
           if (j >= S && !mbar_wait(k_empty + s, ph ^ 1, ctl)) break;
           if (stored_stages & (1u << s)) {  // stage s still feeds a store of tile j - S
             bulk_wait_read_all();
@@ -414,24 +578,40 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
         }
       }
     }
+    if (SPLIT) {  // the softmax warps' cluster barriers (merge_split)
+      __syncwarp();
+      cluster_wait();
+      cluster_sync_all();
+      cluster_sync_all();
+    }
   } else {
     setmaxnreg_inc<224>();
     // -------------------------------------------------------------- softmax
     const int t = (warp >= 8) ? 1 : 0;   // which Q tile this warpgroup owns
+    // What only the epilogue needs waits in shared memory, not in registers.
+    volatile int4* item_sh = reinterpret_cast<volatile int4*>(smem + C::OFF_ITEM) + (warp - 4);
+    if (lane == 0) {
+      item_sh->x = b;
+      item_sh->y = h;
+      item_sh->z = role;
+      item_sh->w = tileA + t;
+    }
+    __syncwarp();
     const int quarter = warp & 3;        // TMEM lane quarter this warp may access
     const int row = quarter * 32 + lane;
     const uint32_t lane_off = uint32_t(quarter * 32) << 16;
     const uint32_t s_t = tmem + lane_off + C::TM_S + 128 * t;
     const uint32_t o_t = tmem + lane_off + C::TM_O + 128 * t;
-    const int tile = tileA + t;
     const bool active = (t == 0) || has_b;
     const float sl2 = p.scale_log2;
     const float bias_l2 = (role == 2 && p.bias) ? __ldg(p.bias + h) * kLog2e : 0.f;
-    float m = -INFINITY, l = 0.f, lref = 0.f;
+    // A range of a split item may hold masked keys alone (a reference bias of
+    // -inf): a finite start keeps their probabilities 0.
+    float m = SPLIT ? kLowestMax : -INFINITY, l = 0.f, lref = 0.f;
     bool ok = active;
     for (int j = 0; ok && j < nkv; ++j) {
       int r, row0;
-      kv_tile(p, j, r, row0);
+      kv_tile(p, j0 + j, r, row0);
       const int nvalid = min(BN, p.nk[r] - row0);
       const float badd = (r == 1) ? bias_l2 : 0.f;
       ok = __all_sync(0xffffffffu, mbar_wait(s_full + t, j & 1, ctl));
@@ -517,12 +697,19 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
       mbar_arrive(p_ready + t);
     }
     if (ok) ok = __all_sync(0xffffffffu, mbar_wait(o_done + t, 0, ctl));
+    const int eb = item_sh->x, eh = item_sh->y, erole = item_sh->z, tile = item_sh->w;
     const int grow = tile * BM + row;
-    const bool valid = active && grow < p.nq[role];
-    const float inv_l = 1.f / l;
-    if (ok) {
+    const bool valid = active && grow < p.nq[erole];
+    __nv_bfloat16* orow = p.o_ptr[erole] + eb * p.o_sb[erole] + eh * p.o_sh[erole] + int64_t(grow) * p.o_sn[erole];
+    float inv_l;
+    if (SPLIT) {
+      merge_split<D>(ctl, smem, parts_full, o_t, ok && active, has_b, valid, rank, nrank, t, row, m, l, lref, orow);
+      inv_l = 1.f / l;
+    } else {
+      inv_l = 1.f / l;
+    }
+    if (!SPLIT && ok) {
       tc_fence_after();
-      __nv_bfloat16* orow = p.o_ptr[role] + b * p.o_sb[role] + h * p.o_sh[role] + int64_t(grow) * p.o_sn[role];
 #pragma unroll
       for (int c0 = 0; c0 < D; c0 += 32) {
         uint32_t ov[32];
@@ -543,16 +730,16 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
     }
     // Per-tile mass partial: sum over the tile's mass rows of l_ref / l, in a
     // fixed order (warp butterfly, then quarters 0..3).
-    const bool in_mass = ((role == 2) || (role == 0 && p.mass_rows == 1)) &&
+    const bool in_mass = ((erole == 2) || (erole == 0 && p.mass_rows == 1)) &&
                          (p.mass_stride <= 1 || grow % p.mass_stride == 0);
     float mv = (ok && valid && in_mass) ? lref * inv_l : 0.f;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mv += __shfl_xor_sync(0xffffffffu, mv, o);
     if (lane == 0) red[4 * t + quarter] = mv;
     named_bar_sync(1 + t, 128);
-    if (ok && active && role != 1 && quarter == 0 && lane == 0) {
-      const int idx = (role == 0) ? tile : p.q_tiles[0] + tile;
-      p.mass_partial[(int64_t(b) * p.H + h) * p.mpl + idx] =
+    if (ok && active && erole != 1 && rank == 0 && quarter == 0 && lane == 0) {
+      const int idx = (erole == 0) ? tile : p.q_tiles[0] + tile;
+      p.mass_partial[(int64_t(eb) * p.H + eh) * p.mpl + idx] =
           ((red[4 * t] + red[4 * t + 1]) + red[4 * t + 2]) + red[4 * t + 3];
     }
   }
@@ -562,16 +749,211 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
     tc_fence_after();
     tmem_dealloc(tmem, C::TMEM_COLS);
   }
+  // PART_REST starts beside the launch of the rounds (programmatic dependent
+  // launch) and needs nothing of it, but must not complete before it: what
+  // comes next in the stream waits for this launch alone.
+  if (SPLIT && p.part == PART_REST && blockIdx.x == 0) wait_primary();
 }
 
 // ------------------------------------------------------------------ host side
-template <int D>
-ra_status launch(const Params& p, dim3 grid, cudaStream_t st) {
-  const ra_status as = ensure_dynamic_smem(reinterpret_cast<const void*>(joint_attn_kernel<D>), Cfg<D>::SMEM_ALLOC,
-                                           "refadapt_joint_attn");
+using Kernel = void (*)(Params);
+struct KernelInfo {
+  Kernel fn;
+  int smem;
+};
+inline KernelInfo kernel_of(int d, bool split) {
+  if (d == 128)
+    return split ? KernelInfo{joint_attn_kernel<128, true>, Cfg<128>::SPLIT_ALLOC}
+                 : KernelInfo{joint_attn_kernel<128, false>, Cfg<128>::SMEM_ALLOC};
+  return split ? KernelInfo{joint_attn_kernel<64, true>, Cfg<64>::SPLIT_ALLOC}
+               : KernelInfo{joint_attn_kernel<64, false>, Cfg<64>::SMEM_ALLOC};
+}
+
+// Clusters of cs CTAs of the split kernel that can run at once on the current
+// device (they live inside one GPC, so the floorplan decides); cached per
+// device, -1 with the error set on failure.
+int max_clusters(int d, int cs) {
+  static std::mutex mu;
+  static int cache[64][2][MAX_SPLIT + 1];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+    set_error("refadapt_joint_attn: no usable current device");
+    return -1;
+  }
+  std::lock_guard<std::mutex> lk(mu);
+  int& n = cache[dev][d == 128 ? 1 : 0][cs];
+  if (n == 0) {
+    const KernelInfo k = kernel_of(d, true);
+    cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem);
+    cudaLaunchConfig_t cfg;
+    std::memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3(cs, 1, 1);
+    cfg.blockDim = dim3(NUM_THREADS, 1, 1);
+    cfg.dynamicSmemBytes = k.smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cs;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int found = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&found, k.fn, &cfg);
+    if (e != cudaSuccess) {
+      set_error("refadapt_joint_attn: cluster occupancy query: %s", cudaGetErrorString(e));
+      cudaGetLastError();
+      return -1;
+    }
+    n = found > 0 ? found : -2;  // none fits
+  }
+  return n > 0 ? n : 0;
+}
+
+// Launches `items` items of p.part: one CTA each, or a cluster of cs CTAs each.
+ra_status launch(const Params& p, int d, int64_t items, int cs, cudaStream_t st) {
+  const char* who = "refadapt_joint_attn";
+  if (items * cs > 2147483647) {
+    set_error("%s: too many rows", who);
+    return RA_EINVAL;
+  }
+  const KernelInfo k = kernel_of(d, cs > 1);
+  const ra_status as = ensure_dynamic_smem(reinterpret_cast<const void*>(k.fn), k.smem, who);
   if (as != RA_OK) return as;
-  joint_attn_kernel<D><<<grid, NUM_THREADS, Cfg<D>::SMEM_ALLOC, st>>>(p);
-  return launch_status("refadapt_joint_attn");
+  cudaLaunchConfig_t cfg;
+  std::memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(unsigned(items * cs), 1, 1);
+  cfg.blockDim = dim3(NUM_THREADS, 1, 1);
+  cfg.dynamicSmemBytes = k.smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  int na = 0;
+  if (cs > 1) {
+    attr[na].id = cudaLaunchAttributeClusterDimension;
+    attr[na].val.clusterDim.x = cs;
+    attr[na].val.clusterDim.y = 1;
+    attr[na].val.clusterDim.z = 1;
+    ++na;
+  }
+  if (p.part == PART_REST) {
+    attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[na].val.programmaticStreamSerializationAllowed = 1;
+    ++na;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = na;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k.fn, p);
+  if (e != cudaSuccess) {
+    set_error("%s: launch failed: %s", who, cudaGetErrorString(e));
+    cudaGetLastError();
+    return RA_ECUDA;
+  }
+  return launch_status(who);
+}
+
+// How a call's items are launched.
+struct Plan {
+  int group;     // Q tiles per item
+  int cs;        // CTAs per split item, 1: nothing is split
+  int rest_max;  // whole rounds unsplit and a rest of at most this many items split; 0: one launch
+};
+
+// Items of the launch's samples when every reference row runs / none does.
+struct Live {
+  int64_t most, least;
+};
+Live live_items(const Params& p, int group, int nb) {
+  int64_t q[3];
+  for (int r = 0; r < 3; ++r) q[r] = (p.q_tiles[r] + group - 1) / group;
+  return {int64_t(p.H) * nb * (q[0] + q[1] + q[2]), int64_t(p.H) * nb * (q[0] + q[2])};
+}
+
+// The cheapest launch by a model of a CTA's time (microseconds on a GB300,
+// from clock counters and whole launches): a fixed part (first mode load,
+// set-up, first loads, cold instruction fetches, epilogue), so much per key tile
+// with two Q tiles or one, and the merge of a split item. A split pays where an
+// unsplit launch leaves SMs idle for long: 72 items of 98 key tiles (every 8th
+// target row of the image-edit shape) take 82 us in clusters of two, 145 us
+// unsplit; 312 items of 26 key tiles (two rounds of 152 and 8) 112 us with the
+// rest in clusters of four, 133 us in three rounds. One Q tile per item pays
+// when all items fit one round (two samples of 77 + 1000 + 500 rows, 8 heads,
+// d = 64: 21.5 against 23.9 us). Modes are on the device, so a call with modes
+// is weighed with and without its reference rows.
+ra_status make_plan(const Params& p, int d, int nb, int slots, Plan* out) {
+  const int n = p.kv_tiles[0] + p.kv_tiles[1] + p.kv_tiles[2];
+  const double merge = 6.0, second_launch = 2.0, fixed[3] = {0, 3.7, 4.7};
+  const double tile[3] = {0, d == 128 ? 1.22 : 1.15, d == 128 ? 1.41 : 1.3};
+  auto cta = [&](int group, int cs) {
+    return fixed[group] + (n + cs - 1) / cs * tile[group] + (cs > 1 ? merge : 0.0);
+  };
+  auto rounds = [](int64_t items, int64_t width) { return double((items + width - 1) / width); };
+  *out = Plan{2, 1, 0};
+  double best = 0;
+  for (int group = 2; group >= 1; --group) {
+    const Live lv = live_items(p, group, nb);
+    const int64_t cases[2] = {lv.most, p.mode ? lv.least : lv.most};
+    for (int cs = 1; cs <= MAX_SPLIT && cs <= n; cs *= 2) {
+      int clusters = slots;
+      if (cs > 1) {
+        clusters = max_clusters(d, cs);
+        if (clusters < 0) return RA_ECUDA;
+        if (clusters == 0) continue;
+      }
+      int rest_max = 0;
+      if (cs > 1 && lv.most >= slots) {
+        const double whole = cta(group, 1) - second_launch;
+        rest_max = int(whole / cta(group, cs)) * clusters;
+        if (rest_max > slots - 1) rest_max = slots - 1;
+        if (rest_max == 0 || group == 1 || lv.most > 2147483647) continue;
+      }
+      double us = 0;
+      for (int64_t live : cases) {
+        if (rest_max == 0) {
+          us += rounds(live, clusters) * cta(group, cs);
+          continue;
+        }
+        const int64_t whole = round_items(int(live), slots, rest_max);
+        us += rounds(whole, slots) * cta(group, 1) + second_launch;
+        if (live > whole) us += rounds(live - whole, clusters) * cta(group, cs);
+      }
+      if (best == 0 || us < 0.97 * best) {
+        best = us;
+        *out = Plan{group, cs, rest_max};
+      }
+    }
+  }
+  return RA_OK;
+}
+
+// Plans and launches a call, MAX_SAMPLES samples at a time.
+ra_status run(Params& p, int d, cudaStream_t st) {
+  p.slots = num_sms();
+  for (p.b0 = 0; p.b0 < p.B; p.b0 += MAX_SAMPLES) {
+    p.nb = p.B - p.b0 < MAX_SAMPLES ? p.B - p.b0 : MAX_SAMPLES;
+    Plan plan;
+    ra_status s = make_plan(p, d, p.nb, p.slots, &plan);
+    if (s != RA_OK) return s;
+    p.group = plan.group;
+    for (int r = 0; r < 3; ++r) p.q_blocks[r] = (p.q_tiles[r] + plan.group - 1) / plan.group;
+    for (int i = 0; i < 2; ++i) {
+      // exact while item * per < 2^32 for every item < H * per
+      const uint64_t per = uint64_t(p.q_blocks[0]) + p.q_blocks[2] + (i == 0 ? p.q_blocks[1] : 0);
+      p.per_inv[i] = per > 1 && per * per * p.H < (uint64_t(1) << 32) ? uint32_t(((uint64_t(1) << 32) + per - 1) / per) : 0;
+    }
+    const Live lv = live_items(p, plan.group, p.nb);
+    if (plan.rest_max == 0) {
+      p.part = PART_ALL;
+      s = launch(p, d, lv.most, plan.cs, st);
+    } else {
+      // No modes leave more whole rounds than all items do, or a larger split rest.
+      p.rest_max = plan.rest_max;
+      p.part = PART_ROUNDS;
+      s = launch(p, d, round_items(int(lv.most), p.slots, p.rest_max), 1, st);
+      p.part = PART_REST;
+      if (s == RA_OK) s = launch(p, d, p.rest_max, plan.cs, st);
+    }
+    if (s != RA_OK) return s;
+  }
+  return RA_OK;
 }
 
 }  // namespace attn
@@ -647,7 +1029,6 @@ extern "C" ra_status refadapt_joint_attn(const ra_attn_args* a, void* stream) {
     p.nq[r] = nq;
     p.kv_tiles[r] = (nk + BN - 1) / BN;
     p.q_tiles[r] = (nq + BM - 1) / BM;
-    p.q_blocks[r] = (p.q_tiles[r] + 1) / 2;
     if (nk > 0 && (!encode_seg(&p.tm_k[r], a->k[r], a->B, a->H, d, 64, BN, true) ||
                    !encode_seg(&p.tm_v[r], a->v[r], a->B, a->H, d, 64, BN, true)))
       return RA_EINVAL;
@@ -724,8 +1105,5 @@ extern "C" ra_status refadapt_joint_attn(const ra_attn_args* a, void* stream) {
   p.mass_partial = a->mass_partial;
   p.err_word = a->err_word;
   p.budget_ns = wait_budget_ns();
-  const int blocks = p.q_blocks[0] + p.q_blocks[1] + p.q_blocks[2];
-  dim3 grid(blocks, a->H, a->B);
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  return d == 128 ? launch<128>(p, grid, st) : launch<64>(p, grid, st);
+  return run(p, d, static_cast<cudaStream_t>(stream));
 }

@@ -335,18 +335,6 @@ struct ClusterParams {
   gate::Params gp;        // gp.qd == d_out
 };
 
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// Arrival that only says "this CTA has started": no release (nothing is
-// published by it; the final cluster_sync_all orders the remote stores).
-__device__ __forceinline__ void cluster_arrive() {
-  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait() {
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
 template <int S, int UB>
 __global__ void __launch_bounds__(ClLayout<S, UB>::THREADS)
     q_delta_cluster_kernel(const __grid_constant__ ClusterParams p) {
@@ -369,7 +357,7 @@ __global__ void __launch_bounds__(ClLayout<S, UB>::THREADS)
   float d_val = 0.f;  // the slab's D (leader, thread 0)
   // This CTA has started (its shared memory exists): the remote stores at the
   // end wait for every CTA's arrival, the loads below need no one else.
-  cluster_arrive();
+  cluster_arrive();  // no release: the final cluster_sync_all orders the remote stores
   const WaitCtl ctl{abort_flag, nullptr, p.budget_ns};
   // Programmatic dependent launch: this grid may start while the previous
   // kernel of the stream finishes. Each role waits for that kernel (complete,
