@@ -39,6 +39,15 @@ bool check_seg(const ra_seg& s, const char* what, bool allow_null_if_empty = tru
 bool encode_seg(CUtensorMap* tm, const ra_seg& s, int B, int H, int d, int box_cols, int box_rows,
                 bool swizzle128);
 
+// Launch attribute: the kernel may start while the previous one of the stream
+// finishes (it calls pdl_wait() before it touches global memory).
+inline cudaLaunchAttribute pdl_attribute() {
+  cudaLaunchAttribute a;
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  return a;
+}
+
 inline ra_status launch_status(const char* what) {
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {

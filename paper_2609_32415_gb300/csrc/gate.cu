@@ -12,6 +12,7 @@
 
 #include "api_common.h"
 #include "gate_body.cuh"
+#include "tc_ptx.cuh"
 
 namespace ra {
 namespace gate {
@@ -33,6 +34,8 @@ __global__ void init_kernel(ra_state* st, int32_t B) {
 __global__ void __launch_bounds__(THREADS) gate_kernel(const Params p) {
   extern __shared__ float m_sh[];  // [B * H]
   __shared__ int32_t full_step;
+  pdl_launch();
+  pdl_wait();
   decide(p, m_sh, &full_step);
 }
 
@@ -90,7 +93,20 @@ ra_status make_params(const ra_gate_args* a, const char* who, Params* p) {
 
 ra_status launch(const Params& p, cudaStream_t stream, const char* who) {
   const size_t sh_bytes = size_t(p.B) * p.H * sizeof(float);
-  gate_kernel<<<1, THREADS, sh_bytes, stream>>>(p);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(1);
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = sh_bytes;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr = pdl_attribute();
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, gate_kernel, p);
+  if (e != cudaSuccess) {
+    set_error("%s: launch failed: %s", who, cudaGetErrorString(e));
+    cudaGetLastError();
+    return RA_ECUDA;
+  }
   return launch_status(who);
 }
 

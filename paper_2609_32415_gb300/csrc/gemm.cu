@@ -438,6 +438,8 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const WaitCtl ctl{abort_flag, p.err_word, p.budget_ns};
+  pdl_launch();
+  pdl_wait();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -585,6 +587,8 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_pair_kernel(const __grid_cons
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const WaitCtl ctl{abort_flag, p.err_word, p.budget_ns};
+  pdl_launch();
+  pdl_wait();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -948,28 +952,24 @@ extern "C" ra_status refadapt_gemm(const ra_gemm_args* a, void* stream) {
                                            pair ? P_SMEM_ALLOC : SMEM_ALLOC, "refadapt_gemm");
   if (as != RA_OK) return as;
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (!pair) {
-    const int64_t grid = tiles < sms ? tiles : sms;
-    kn.single<<<unsigned(grid), THREADS, SMEM_ALLOC, st>>>(p);
-    return launch_status("refadapt_gemm");
-  }
-  const int64_t clusters = tiles < sms / 2 ? tiles : (sms / 2 > 0 ? sms / 2 : 1);
   cudaLaunchConfig_t cfg;
   std::memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3(unsigned(2 * clusters), 1, 1);
   cfg.blockDim = dim3(THREADS, 1, 1);
-  cfg.dynamicSmemBytes = P_SMEM_ALLOC;
+  cfg.dynamicSmemBytes = pair ? P_SMEM_ALLOC : SMEM_ALLOC;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 2;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0] = pdl_attribute();
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 2;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kn.pair, p);
+  cfg.numAttrs = pair ? 2 : 1;
+  const int64_t slots = pair ? (sms / 2 > 0 ? sms / 2 : 1) : sms;
+  cfg.gridDim = dim3(unsigned((tiles < slots ? tiles : slots) * (pair ? 2 : 1)), 1, 1);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, pair ? kn.pair : kn.single, p);
   if (e != cudaSuccess) {
-    set_error("refadapt_gemm: pair launch failed: %s", cudaGetErrorString(e));
+    set_error("refadapt_gemm: launch failed: %s", cudaGetErrorString(e));
     cudaGetLastError();
     return RA_ECUDA;
   }

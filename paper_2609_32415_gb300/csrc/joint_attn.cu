@@ -239,8 +239,6 @@ __device__ __forceinline__ float exp64_store(const float (&v)[64], int col0, int
   return (s0 + s1) + (s2 + s3);
 }
 
-__device__ __forceinline__ void wait_primary() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // Merge of a split item (the softmax threads of every rank; thread = row of
 // tile t, rows of tile B follow A's). Each rank tells every other its row
 // maximum and sums; scales its O to the common maximum; keeps its own share of
@@ -343,7 +341,10 @@ template <int D, bool SPLIT>
 __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid_constant__ Params p) {
   using C = Cfg<D>;
   constexpr int S = C::STAGES;
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // The rest of a call starts beside its whole rounds and depends on nothing of
+  // theirs; it starts after their pdl_launch(), so after what they wait for.
+  if (!SPLIT || p.part != PART_REST) pdl_wait();
+  pdl_launch();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = SPLIT ? int(cluster_rank()) : 0, nrank = SPLIT ? int(cluster_size()) : 1;
   const int lane_mode = (lane < p.nb && p.mode) ? __ldg(p.mode + p.b0 + lane) : int(RA_MODE_FULL);
@@ -400,7 +401,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
     if (p.part == PART_REST) item += rounds;
     if (item >= (p.part == PART_REST ? live : rounds)) {  // uniform over the cluster
       if (warp == 1) tmem_dealloc(tmem, C::TMEM_COLS);
-      if (p.part == PART_REST && blockIdx.x == 0) wait_primary();
+      if (p.part == PART_REST && blockIdx.x == 0) pdl_wait();
       return;
     }
   }
@@ -752,7 +753,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
   // PART_REST starts beside the launch of the rounds (programmatic dependent
   // launch) and needs nothing of it, but must not complete before it: what
   // comes next in the stream waits for this launch alone.
-  if (SPLIT && p.part == PART_REST && blockIdx.x == 0) wait_primary();
+  if (SPLIT && p.part == PART_REST && blockIdx.x == 0) pdl_wait();
 }
 
 // ------------------------------------------------------------------ host side
@@ -834,11 +835,7 @@ ra_status launch(const Params& p, int d, int64_t items, int cs, cudaStream_t st)
     attr[na].val.clusterDim.z = 1;
     ++na;
   }
-  if (p.part == PART_REST) {
-    attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[na].val.programmaticStreamSerializationAllowed = 1;
-    ++na;
-  }
+  attr[na++] = pdl_attribute();
   cfg.attrs = attr;
   cfg.numAttrs = na;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, k.fn, p);

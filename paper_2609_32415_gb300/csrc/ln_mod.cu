@@ -41,6 +41,8 @@ struct Params {
 
 template <int G>  // 8-feature groups per lane: C = 256 G
 __global__ void __launch_bounds__(32 * WARPS) ln_mod_kernel(const __grid_constant__ Params p) {
+  pdl_launch();
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   const int64_t gr = int64_t(blockIdx.x) * WARPS + (threadIdx.x >> 5);
   if (gr >= p.total_rows) return;
@@ -170,14 +172,27 @@ extern "C" ra_status refadapt_ln_modulate(const ra_lnmod_args* a, void* stream) 
     return RA_EINVAL;
   }
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(unsigned(blocks));
+  cfg.blockDim = dim3(32 * WARPS);
+  cfg.stream = st;
+  cudaLaunchAttribute attr = pdl_attribute();
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaError_t e = cudaSuccess;
   switch (p.groups) {
 #define RA_LNMOD_CASE(G) \
-  case G: ln_mod_kernel<G><<<unsigned(blocks), 32 * WARPS, 0, st>>>(p); break;
+  case G: e = cudaLaunchKernelEx(&cfg, ln_mod_kernel<G>, p); break;
     RA_LNMOD_CASE(1) RA_LNMOD_CASE(2) RA_LNMOD_CASE(3) RA_LNMOD_CASE(4) RA_LNMOD_CASE(5) RA_LNMOD_CASE(6)
     RA_LNMOD_CASE(7) RA_LNMOD_CASE(8) RA_LNMOD_CASE(9) RA_LNMOD_CASE(10) RA_LNMOD_CASE(11) RA_LNMOD_CASE(12)
     RA_LNMOD_CASE(13) RA_LNMOD_CASE(14) RA_LNMOD_CASE(15) RA_LNMOD_CASE(16)
 #undef RA_LNMOD_CASE
     default: break;
+  }
+  if (e != cudaSuccess) {
+    set_error("refadapt_ln_modulate: launch failed: %s", cudaGetErrorString(e));
+    cudaGetLastError();
+    return RA_ECUDA;
   }
   return launch_status("refadapt_ln_modulate");
 }

@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(ClLayout<S, UB>::THREADS)
   // kernel of the stream finishes. Each role waits for that kernel (complete,
   // its writes visible) before it touches global memory; the next kernel of
   // the stream may start its own set-up as soon as every CTA got here.
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  pdl_launch();
 
   if (warp == CL_CONSUMERS) {
     // The producer warp sets up the ring itself and releases the consumers
@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(ClLayout<S, UB>::THREADS)
       bulk_prefetch_l2(p.base_c + b * p.c_sb + h * p.c_sh + off, bytes);
       bulk_prefetch_l2(p.base_p + b * p.p_sb + h * p.p_sh + off, bytes);
     }
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_wait();
     if (lane == 0) {
       // ---------------------------------------------------------- producer
       if (!p.bulk) {
@@ -427,7 +427,7 @@ __global__ void __launch_bounds__(ClLayout<S, UB>::THREADS)
   } else {
     // ------------------------------------------------------------ consumers
     named_bar_sync(2, L::THREADS);  // the ring's barriers are initialised
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // orders the final store of D
+    pdl_wait();  // orders the final store of D
     // Fused gate: the leader's first warp reduces this slab's mass partials of
     // the previous step (they need nothing of this launch) while the first
     // units are still on their way.
@@ -729,8 +729,7 @@ ra_status launch(const char* who, const ra_seg* q_cur, const ra_seg* q_prev, int
       attr[0].val.clusterDim.z = 1;
       // may overlap the previous kernel's tail (the kernel waits for it with
       // griddepcontrol.wait before touching global memory)
-      attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-      attr[1].val.programmaticStreamSerializationAllowed = 1;
+      attr[1] = pdl_attribute();
       cfg.attrs = attr;
       cfg.numAttrs = 2;
       const cudaError_t e = cudaLaunchKernelEx(&cfg, cv.fn, c);

@@ -481,6 +481,14 @@ __device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
   return r;
 }
 
+// Programmatic dependent launch. A kernel launched with it may start while the
+// previous kernel of its stream finishes: pdl_wait() returns once that one is
+// complete and its writes are visible, and comes before anything that depends
+// on it (every global access). pdl_launch() lets the next kernel of the stream
+// start its own set-up (once every CTA of this grid got there or ended).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Named barrier over `nthreads` threads (id 1..15; 0 is __syncthreads).
 __device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
