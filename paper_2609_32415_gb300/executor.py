@@ -286,7 +286,7 @@ class Executor:
         blocks before it, never an attention of the same step, so the results
         are those of the one-stream order. Every event is recorded inside the
         step, which can be captured as a CUDA graph."""
-        if not self.overlap or self.n_blocks == 1:  # one block: nothing to run beside
+        if not self.overlap:
             for b in range(self.n_blocks):
                 out = outs[b] if outs is not None else self.scratch_outputs(b % 2)
                 self.block(t, b, inputs[b], out, log_index, stream)
@@ -304,15 +304,15 @@ class Executor:
             out = outs[b] if outs is not None else self.scratch_outputs(b % 2)
             if b >= 2:
                 side.wait_event(self._attn_done[b - 2])
-            self.gate_block(t, b, inputs[b]["tgt"][0], log_index, side)
-            if not self.fused_cache:
-                self.update_cache(t, b, inputs[b], log_index, side)
-            self._decided[b].record(side)
-            main.wait_event(self._decided[b])
-            # the attention's hook records on the current stream
-            with torch.cuda.stream(main) if self.attn_hook is not None else contextlib.nullcontext():
-                self.attend(t, b, inputs[b], out, log_index, main)
-            self._attn_done[b].record(main)
+            with torch.cuda.stream(side):
+                self.gate_block(t, b, inputs[b]["tgt"][0], log_index)
+                if not self.fused_cache:
+                    self.update_cache(t, b, inputs[b], log_index)
+                self._decided[b].record(side)
+            with torch.cuda.stream(main):
+                main.wait_event(self._decided[b])
+                self.attend(t, b, inputs[b], out, log_index)
+                self._attn_done[b].record(main)
             if after_block is not None:
                 with torch.cuda.stream(main):
                     after_block(t, b)
