@@ -150,6 +150,23 @@ def load():
     return lib
 
 
+_native = None
+
+
+def native():
+    """The native argument marshalling (_binding.so, csrc/binding.cpp)."""
+    global _native
+    if _native is None:
+        load()
+        try:
+            from . import _binding
+        except ImportError as e:
+            raise RuntimeError("_binding.so is missing or was built for another torch (%s): build it with "
+                               "`python -m paper_2609_32415_gb300.build`" % e) from e
+        _native = _binding
+    return _native
+
+
 def check(fn, status):
     if status != RA_OK:
         msg = load().refadapt_last_error().decode(errors="replace")

@@ -1,7 +1,8 @@
 """Thin Python binding of the C ABI (include/refadapt.h), same names.
 
-Only argument marshalling happens here: torch tensors supply device memory and
-streams; every step of the computation runs in librefadapt.so's kernels.
+Only argument marshalling happens here (natively, csrc/binding.cpp, for the
+calls of a step): torch tensors supply device memory and streams; every step
+of the computation runs in librefadapt.so's kernels.
 Tensors are [B, H, n, d] bf16 CUDA views with a contiguous last axis (any
 other strides, 16-byte aligned).
 """
@@ -10,7 +11,7 @@ import ctypes
 import torch
 
 from . import _lib
-from ._lib import RaAttnArgs, RaGateArgs, RaSeg, check
+from ._lib import RaSeg, check
 
 __all__ = ["seg", "refadapt_joint_attn", "refadapt_mass_partial_len", "refadapt_q_delta",
            "refadapt_q_delta_workspace_size", "refadapt_q_delta_noalloc", "refadapt_state_size", "refadapt_state_init",
@@ -29,6 +30,13 @@ def _stream(stream):
     if isinstance(stream, torch.cuda.Stream):
         return ctypes.c_void_p(stream.cuda_stream)
     return ctypes.c_void_p(int(stream))
+
+
+def _handle(stream):
+    """A stream argument for the native calls: None (the current stream) or the raw handle."""
+    if stream is None:
+        return None
+    return stream.cuda_stream if isinstance(stream, torch.cuda.Stream) else int(stream)
 
 
 def seg(t, n=None) -> RaSeg:
@@ -56,32 +64,11 @@ def refadapt_joint_attn(q, k, v, o, mass_partial, mode=None, softmax_scale=0.0, 
     """q, k, v, o: sequences (text, ref, tgt) of [B, H, n, d] tensors; q[1] / o[1] may be None.
     ref_fresh: optional (q, k, v) of this step's reference rows for the fused
     cache update (q may be None when q[1] is); a_b, step: the stamp it writes."""
-    lib = _lib.load()
-    B, H, _, d = k[2].shape
-    a = RaAttnArgs()
-    a.B, a.H, a.d, a.mass_rows = B, H, d, int(mass_rows)
-    for r in range(3):
-        n_q = q[r].shape[2] if q[r] is not None else k[r].shape[2]
-        a.q[r] = seg(q[r], n_q)
-        a.k[r] = seg(k[r])
-        a.v[r] = seg(v[r])
-        a.o[r] = seg(o[r], n_q)
-    a.softmax_scale = float(softmax_scale)
-    a.mass_row_stride = int(mass_row_stride)
-    a.ref_logit_bias = _ptr(ref_logit_bias)
-    a.mode = _ptr(mode)
-    a.mass_partial = _ptr(mass_partial)
-    a.err_word = _ptr(err_word)
-    if ref_fresh is not None:
-        fq, fk, fv = ref_fresh
-        a.ref_fresh_q = seg(fq)
-        a.ref_fresh_k = seg(fk)
-        a.ref_fresh_v = seg(fv)
-        a.a_b = _ptr(a_b)
-        a.step = int(step)
-    elif a_b is not None:
+    if ref_fresh is None and a_b is not None:
         raise ValueError("refadapt_joint_attn: a_b is written only with ref_fresh")
-    return check("refadapt_joint_attn", lib.refadapt_joint_attn(ctypes.byref(a), _stream(stream)))
+    return check("refadapt_joint_attn", _lib.native().joint_attn(
+        q, k, v, o, mass_partial, mode, float(softmax_scale), ref_logit_bias, int(mass_rows), err_word,
+        int(mass_row_stride), ref_fresh, a_b, int(step), _handle(stream)))
 
 
 def refadapt_q_delta_workspace_size(B, H) -> int:
@@ -94,12 +81,8 @@ def q_delta_workspace(B, H, device="cuda"):
 
 
 def refadapt_q_delta(q_cur, q_prev, d_out, workspace, eps=1e-6, stream=None):
-    lib = _lib.load()
-    B, H, _, d = q_cur.shape
-    sc, sp = seg(q_cur), seg(q_prev)
-    return check("refadapt_q_delta", lib.refadapt_q_delta(
-        ctypes.byref(sc), ctypes.byref(sp), B, H, d, float(eps), _ptr(d_out), _ptr(workspace),
-        workspace.numel() * workspace.element_size(), _stream(stream)))
+    return check("refadapt_q_delta", _lib.native().q_delta(q_cur, q_prev, d_out, workspace, float(eps),
+                                                           _handle(stream)))
 
 
 def refadapt_q_delta_noalloc(q_cur, q_prev, d_out, eps=1e-6, stream=None):
@@ -126,30 +109,11 @@ def new_state(B, device="cuda", stream=None):
     return st
 
 
-def _gate_args(t, b, state, mode_out, theta, delta_max, B, H, q_delta, mass_partial_prev, mass_row_count,
-               forced_boundary, gbar_out, m_out, cue):
-    a = RaGateArgs()
-    a.theta = float(theta)
-    a.t, a.b, a.B, a.H = int(t), int(b), int(B), int(H)
-    a.delta_max = int(delta_max)
-    a.forced_boundary = int(forced_boundary)
-    a.mass_partial_len = int(mass_partial_prev.shape[-1]) if mass_partial_prev is not None else 0
-    a.mass_row_count = int(mass_row_count)
-    a.cue = int(cue)
-    a.q_delta = _ptr(q_delta)
-    a.mass_partial_prev = _ptr(mass_partial_prev)
-    a.state = _ptr(state)
-    a.mode_out = _ptr(mode_out)
-    a.gbar_out = _ptr(gbar_out)
-    a.m_out = _ptr(m_out)
-    return a
-
-
 def refadapt_gate(t, b, state, mode_out, theta, delta_max, B, H, q_delta=None, mass_partial_prev=None,
                   mass_row_count=0, forced_boundary=-1, gbar_out=None, m_out=None, cue=0, stream=None):
-    a = _gate_args(t, b, state, mode_out, theta, delta_max, B, H, q_delta, mass_partial_prev, mass_row_count,
-                   forced_boundary, gbar_out, m_out, cue)
-    return check("refadapt_gate", _lib.load().refadapt_gate(ctypes.byref(a), _stream(stream)))
+    return check("refadapt_gate", _lib.native().gate(
+        int(t), int(b), state, mode_out, float(theta), int(delta_max), int(B), int(H), q_delta, mass_partial_prev,
+        int(mass_row_count), int(forced_boundary), gbar_out, m_out, int(cue), _handle(stream)))
 
 
 def refadapt_q_delta_gate(q_cur, q_prev, d_out, workspace, t, b, state, mode_out, theta, delta_max,
@@ -157,14 +121,9 @@ def refadapt_q_delta_gate(q_cur, q_prev, d_out, workspace, t, b, state, mode_out
                           m_out=None, cue=0, stream=None):
     """refadapt_q_delta then refadapt_gate on its D (t >= 1), in one launch
     when the Q change takes its cluster path."""
-    lib = _lib.load()
-    B, H, _, d = q_cur.shape
-    sc, sp = seg(q_cur), seg(q_prev)
-    a = _gate_args(t, b, state, mode_out, theta, delta_max, B, H, d_out, mass_partial_prev, mass_row_count,
-                   forced_boundary, gbar_out, m_out, cue)
-    return check("refadapt_q_delta_gate", lib.refadapt_q_delta_gate(
-        ctypes.byref(sc), ctypes.byref(sp), B, H, d, float(eps), _ptr(d_out), _ptr(workspace),
-        workspace.numel() * workspace.element_size(), ctypes.byref(a), _stream(stream)))
+    return check("refadapt_q_delta_gate", _lib.native().q_delta_gate(
+        q_cur, q_prev, d_out, workspace, float(eps), _handle(stream), int(t), int(b), state, mode_out, float(theta),
+        int(delta_max), mass_partial_prev, int(mass_row_count), int(forced_boundary), gbar_out, m_out, int(cue)))
 
 
 def refadapt_ref_cache_update(k_src, v_src, k_cache, v_cache, mode, t, a_b=None, x_src=None, x_cache=None,
@@ -202,14 +161,6 @@ def refadapt_version() -> int:
 
 
 # --------------------------------------------------------------------------- DiT block around the attention
-def _rows(t, what):
-    """(ptr, stride_s, stride_r, rows) of a [B, rows, F] CUDA tensor with contiguous last axis."""
-    if t.dim() != 3 or not t.is_cuda or (t.shape[2] > 1 and t.stride(2) != 1):
-        raise ValueError("%s: expected a [B, rows, F] CUDA tensor with contiguous last axis, got %s"
-                         % (what, tuple(t.shape)))
-    return (t.data_ptr() if t.numel() > 0 else None), t.stride(0), t.stride(1), t.shape[1]
-
-
 def refadapt_rope_table(table, n_pos, d, base=10000.0, stream=None):
     return check("refadapt_rope_table", _lib.load().refadapt_rope_table(
         _ptr(table), int(n_pos), int(d), float(base), _stream(stream)))
@@ -225,26 +176,8 @@ def rope_table(n_pos, d, base=10000.0, device="cuda", stream=None):
 def refadapt_ln_modulate(segs, C, eps=1e-6, mode=None, stream=None):
     """segs: up to three dicts with h, x ([B, rows, C] bf16), shift, scale
     ([B, C] fp32) and optional gated (bool)."""
-    a = _lib.RaLnmodArgs()
-    B = None
-    for i, sd in enumerate(segs):
-        hp, hs, hr, rows = _rows(sd["h"], "h")
-        xp, xs, xr, xrows = _rows(sd["x"], "x")
-        if xrows != rows:
-            raise ValueError("h and x rows differ")
-        B = sd["h"].shape[0]
-        s = a.seg[i]
-        s.h, s.h_stride_s, s.h_stride_r = hp, hs, hr
-        s.x, s.x_stride_s, s.x_stride_r = xp, xs, xr
-        s.shift, s.scale = _ptr(sd["shift"]), _ptr(sd["scale"])
-        s.mod_stride_s = sd["shift"].stride(0)
-        if sd["scale"].stride(0) != s.mod_stride_s:
-            raise ValueError("shift and scale must share a row stride")
-        s.rows, s.gated = int(rows), int(bool(sd.get("gated", False)))
-    a.B, a.C, a.n_seg = int(B), int(C), len(segs)
-    a.eps = float(eps)
-    a.mode = _ptr(mode)
-    return check("refadapt_ln_modulate", _lib.load().refadapt_ln_modulate(ctypes.byref(a), _stream(stream)))
+    return check("refadapt_ln_modulate",
+                 _lib.native().ln_modulate(segs, int(C), float(eps), mode, _handle(stream)))
 
 
 def refadapt_gemm(segs, N, K, epilogue, mode=None, rope=None, H=0, d=0, norm_eps=1e-6, err_word=None,
@@ -253,36 +186,6 @@ def refadapt_gemm(segs, N, K, epilogue, mode=None, rope=None, H=0, d=0, norm_eps
     optional bias ([N] fp32), gated; plus per epilogue out ([B, rows, N]),
     resid and gate ([B, N] fp32) for RESID, or q, k, v ([B, H, rows, d]),
     q_norm, k_norm ([d] fp32) and pos_offset for QKV."""
-    a = _lib.RaGemmArgs()
-    B = None
-    for i, sd in enumerate(segs):
-        ap, ass, asr, rows = _rows(sd["a"], "a")
-        B = sd["a"].shape[0]
-        s = a.seg[i]
-        s.a, s.a_stride_s, s.a_stride_r, s.rows = ap, ass, asr, int(rows)
-        s.gated = int(bool(sd.get("gated", False)))
-        w = sd["w"]
-        if tuple(w.shape) != (int(N), int(K)) or not w.is_contiguous() or w.dtype != torch.bfloat16:
-            raise ValueError("w: expected a contiguous [N, K] = [%d, %d] bf16 tensor, got %s"
-                             % (N, K, tuple(w.shape)))
-        s.w = _ptr(w)
-        s.bias = _ptr(sd.get("bias"))
-        if sd.get("out") is not None:
-            s.out, s.out_stride_s, s.out_stride_r, _ = _rows(sd["out"], "out")
-        if sd.get("resid") is not None:
-            s.resid, s.resid_stride_s, s.resid_stride_r, _ = _rows(sd["resid"], "resid")
-        if sd.get("gate") is not None:
-            s.gate, s.gate_stride_s = _ptr(sd["gate"]), sd["gate"].stride(0)
-        if epilogue == _lib.RA_EPI_QKV:
-            s.q_out, s.k_out, s.v_out = seg(sd["q"]), seg(sd["k"]), seg(sd["v"])
-            s.q_norm, s.k_norm = _ptr(sd["q_norm"]), _ptr(sd["k_norm"])
-            s.pos_offset = int(sd.get("pos_offset", 0))
-    a.B, a.N, a.K, a.epilogue = int(B), int(N), int(K), int(epilogue)
-    a.H, a.d, a.n_seg = int(H), int(d), len(segs)
-    a.rope_len = int(rope.shape[0]) if rope is not None else 0
-    a.mode = _ptr(mode)
-    a.rope = _ptr(rope)
-    a.norm_eps = float(norm_eps)
-    a.tile_mode = int(tile_mode)
-    a.err_word = _ptr(err_word)
-    return check("refadapt_gemm", _lib.load().refadapt_gemm(ctypes.byref(a), _stream(stream)))
+    return check("refadapt_gemm", _lib.native().gemm(
+        segs, int(N), int(K), int(epilogue), mode, rope, int(H), int(d), float(norm_eps), err_word, int(tile_mode),
+        _handle(stream)))

@@ -1,9 +1,11 @@
-"""Build librefadapt.so (the C-ABI library) in-tree with nvcc for sm_103a.
+"""Build librefadapt.so (the C-ABI library) in-tree with nvcc for sm_103a, and
+_binding.so, the Python binding's native argument marshalling.
 
 Each .cu under csrc/ is compiled in parallel to an object file, then all are
 linked into paper_2609_32415_gb300/librefadapt.so (static CUDA runtime, no
-torch dependency). Rebuilds only when a source or header is newer than the
-library.
+torch dependency). csrc/binding.cpp is compiled with the host compiler against
+the installed torch's headers meanwhile and linked to that library. Rebuilds
+only when a source or header is newer than the libraries.
 """
 import glob
 import os
@@ -18,6 +20,8 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD_DIR = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "librefadapt.so")
+BINDING_SRC = os.path.join(CSRC, "binding.cpp")
+BINDING = os.path.join(PKG, "_binding.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -33,15 +37,46 @@ def _sources():
 
 
 def _deps():
-    return _sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) + \
+    return _sources() + [BINDING_SRC] + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) + \
         glob.glob(os.path.join(INCLUDE, "*.h")) + [os.path.abspath(__file__)]
 
 
 def up_to_date() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(BINDING):
         return False
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(BINDING))
     return all(os.path.getmtime(f) <= t for f in _deps())
+
+
+def _compile_binding() -> str:
+    """csrc/binding.cpp -> object file (host compiler, the installed torch's headers)."""
+    import sysconfig
+
+    import torch
+    inc = os.path.join(os.path.dirname(torch.__file__), "include")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(_nvcc()))), "include")
+    obj = os.path.join(BUILD_DIR, "binding.o")
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-I", INCLUDE]
+    for d in (inc, os.path.join(inc, "torch", "csrc", "api", "include"), cuda, sysconfig.get_paths()["include"]):
+        cmd += ["-isystem", d]
+    _run(cmd + ["-c", BINDING_SRC, "-o", obj], "compiling binding.cpp")
+    return obj
+
+
+def _run(cmd, what):
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        sys.stderr.write(res.stdout + res.stderr)
+        raise RuntimeError("%s failed" % what)
+
+
+def _link_binding(obj):
+    import torch
+    lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    tmp = BINDING + ".tmp.%d" % os.getpid()
+    _run([os.environ.get("CXX", "g++"), "-shared", "-o", tmp, obj, "-L", PKG, "-l:librefadapt.so", "-Wl,-rpath,$ORIGIN",
+          "-L", lib, "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"], "linking _binding.so")
+    os.replace(tmp, BINDING)
 
 
 def build(force: bool = False, verbose: bool = False, extra_flags=None) -> str:
@@ -64,8 +99,10 @@ def build(force: bool = False, verbose: bool = False, extra_flags=None) -> str:
             raise RuntimeError("nvcc failed on %s" % os.path.basename(src))
         return obj
 
-    with ThreadPoolExecutor(max_workers=max(1, min(len(srcs), os.cpu_count() or 1))) as ex:
+    with ThreadPoolExecutor(max_workers=max(1, min(len(srcs) + 1, os.cpu_count() or 1))) as ex:
+        binding = ex.submit(_compile_binding)
         objs = list(ex.map(compile_one, srcs))
+        binding_obj = binding.result()
     tmp = LIB + ".tmp.%d" % os.getpid()
     cmd = [nvcc] + ARCH + ["-shared", "-o", tmp] + objs
     res = subprocess.run(cmd, capture_output=True, text=True)
@@ -73,6 +110,7 @@ def build(force: bool = False, verbose: bool = False, extra_flags=None) -> str:
         sys.stderr.write(res.stdout + res.stderr)
         raise RuntimeError("linking librefadapt.so failed")
     os.replace(tmp, LIB)
+    _link_binding(binding_obj)
     return LIB
 
 

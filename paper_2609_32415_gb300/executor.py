@@ -146,6 +146,12 @@ class Executor:
                                             device=dev)
             self._o_fresh = [{"text": torch.empty((B, H, n_text, d), dtype=torch.bfloat16, device=dev),
                               "tgt": torch.empty((B, H, n_s, d), dtype=torch.bfloat16, device=dev)} for _ in range(2)]
+        # The views a block's launches take, made once: indexing a tensor costs
+        # microseconds of host time, and a block takes ten of them.
+        self._block = list(zip(self.cache_x.unbind(0), self.cache_k.unbind(0), self.cache_v.unbind(0),
+                               self.a_b.unbind(0), self.mass.unbind(0), self.D.unbind(0)))
+        self._logs = [list(zip(m.unbind(0), g.unbind(0), e.unbind(0)))
+                      for m, g, e in zip(self.modes.unbind(0), self.gbar.unbind(0), self.M.unbind(0))]
         self._out = [None, None]
         self.attn_hook = None   # optional callable(phase in {"pre", "post"}, t, b), e.g. CUDA events
         self.nvtx = bool(nvtx)
@@ -180,26 +186,28 @@ class Executor:
         not read). The caller keeps qt alive until step t + 1's gate of this
         block has been enqueued (it is read as q_{t-1})."""
         li = (t % self.log_steps) if log_index is None else log_index
-        mode = self.modes[li, b]
+        mode = self._logs[li][b][0]
         have_prev = t >= 1 and self._prev_qtgt[b] is not None
         with self._range("t%d b%d decision" % (t, b)):
             self._decide(t, b, qt, li, mode, have_prev, stream)
         self._prev_qtgt[b] = qt
 
     def _decide(self, t, b, qt, li, mode, have_prev, stream):
+        _, gbar, M = self._logs[li][b]
+        mass, D = self._block[b][4:]
         if have_prev:
             # Eq. 1 and the decision in one call (one launch on the cluster path)
             ref_q = self.anchor[b] if self.anchor is not None else self._prev_qtgt[b]
             k = self.sample_stride
             api.refadapt_q_delta_gate(qt[:, :, ::k, :] if k > 1 else qt, ref_q[:, :, ::k, :] if k > 1 else ref_q,
-                                      self.D[b], self.workspace, t, b, self.state, mode, self.theta,
-                                      self.delta_max, self.mass[b], self.mass_row_count, eps=self.eps,
-                                      forced_boundary=self.forced_boundary, gbar_out=self.gbar[li, b],
-                                      m_out=self.M[li, b], cue=CUES[self.cue], stream=stream)
+                                      D, self.workspace, t, b, self.state, mode, self.theta,
+                                      self.delta_max, mass, self.mass_row_count, eps=self.eps,
+                                      forced_boundary=self.forced_boundary, gbar_out=gbar, m_out=M,
+                                      cue=CUES[self.cue], stream=stream)
         else:
             api.refadapt_gate(t, b, self.state, mode, self.theta, self.delta_max, self.B, self.H,
                               mass_row_count=self.mass_row_count, forced_boundary=self.forced_boundary,
-                              gbar_out=self.gbar[li, b], m_out=self.M[li, b], cue=CUES[self.cue], stream=stream)
+                              gbar_out=gbar, m_out=M, cue=CUES[self.cue], stream=stream)
         if self.anchor is not None:
             # Materialising blocks move their anchor to this step's target Q (the
             # V copy is skipped: source and destination coincide).
@@ -230,7 +238,7 @@ class Executor:
         step's gate reads. With fused_cache, materialising samples read x[ref]
         and the kernel writes it into the cache slot and stamps a_b = t."""
         li = (t % self.log_steps) if log_index is None else log_index
-        mode = self.modes[li, b]
+        mode = self._logs[li][b][0]
         qt = x["tgt"][0]
         if self.attn_hook is not None:
             self.attn_hook("pre", t, b)
@@ -242,15 +250,13 @@ class Executor:
             self._diagnose(t, b, li, x, out, stream)
 
     def _attend(self, t, b, x, out, mode, qt, stream):
+        cache_x, cache_k, cache_v, a_b, mass, _ = self._block[b]
         api.refadapt_joint_attn(
-            (x["text"][0], self.cache_x[b], qt),
-            (x["text"][1], self.cache_k[b], x["tgt"][1]),
-            (x["text"][2], self.cache_v[b], x["tgt"][2]),
-            (out["text"], out["ref"], out["tgt"]),
-            self.mass[b], mode=mode, softmax_scale=self.softmax_scale, ref_logit_bias=self.bias,
+            (x["text"][0], cache_x, qt), (x["text"][1], cache_k, x["tgt"][1]), (x["text"][2], cache_v, x["tgt"][2]),
+            (out["text"], out["ref"], out["tgt"]), mass, mode=mode, softmax_scale=self.softmax_scale, ref_logit_bias=self.bias,
             mass_rows=self.mass_rows, err_word=self.err, mass_row_stride=self.sample_stride,
             ref_fresh=x["ref"] if self.fused_cache else None,
-            a_b=self.a_b[b] if self.fused_cache else None, step=t, stream=stream)
+            a_b=a_b if self.fused_cache else None, step=t, stream=stream)
 
     def _diagnose(self, t, b, li, x, out, stream):
         k = self.diag_row_stride
@@ -286,7 +292,7 @@ class Executor:
         blocks before it, never an attention of the same step, so the results
         are those of the one-stream order. Every event is recorded inside the
         step, which can be captured as a CUDA graph."""
-        if not self.overlap:
+        if not self.overlap or self.n_blocks == 1:  # one block: nothing to run beside
             for b in range(self.n_blocks):
                 out = outs[b] if outs is not None else self.scratch_outputs(b % 2)
                 self.block(t, b, inputs[b], out, log_index, stream)
@@ -304,15 +310,15 @@ class Executor:
             out = outs[b] if outs is not None else self.scratch_outputs(b % 2)
             if b >= 2:
                 side.wait_event(self._attn_done[b - 2])
-            with torch.cuda.stream(side):
-                self.gate_block(t, b, inputs[b]["tgt"][0], log_index)
-                if not self.fused_cache:
-                    self.update_cache(t, b, inputs[b], log_index)
-                self._decided[b].record(side)
-            with torch.cuda.stream(main):
-                main.wait_event(self._decided[b])
-                self.attend(t, b, inputs[b], out, log_index)
-                self._attn_done[b].record(main)
+            self.gate_block(t, b, inputs[b]["tgt"][0], log_index, side)
+            if not self.fused_cache:
+                self.update_cache(t, b, inputs[b], log_index, side)
+            self._decided[b].record(side)
+            main.wait_event(self._decided[b])
+            # the attention's hook records on the current stream
+            with torch.cuda.stream(main) if self.attn_hook is not None else contextlib.nullcontext():
+                self.attend(t, b, inputs[b], out, log_index, main)
+            self._attn_done[b].record(main)
             if after_block is not None:
                 with torch.cuda.stream(main):
                     after_block(t, b)
