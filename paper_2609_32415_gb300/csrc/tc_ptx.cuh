@@ -481,6 +481,11 @@ __device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
   return r;
 }
 
+// The two bf16 of a 32-bit word as a packed fp32 pair (exact).
+__device__ __forceinline__ uint64_t bf2_unpack(uint32_t w) {
+  return f2_pack(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
+}
+
 // Programmatic dependent launch. A kernel launched with it may start while the
 // previous kernel of its stream finishes: pdl_wait() returns once that one is
 // complete and its writes are visible, and comes before anything that depends

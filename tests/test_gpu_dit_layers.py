@@ -75,6 +75,33 @@ def test_ln_modulate_segments_and_gating(cuda_ok, C):
             assert ok, (r, s, nbad, eq)
 
 
+@pytest.mark.parametrize("C,B,rows", [(256, 40, (3, 5, 2)), (512, 1, (1, 0, 0)), (1280, 3, (1, 900, 130)),
+                                      (2304, 2, (700, 4, 33)), (3328, 2, (5, 600, 1500)), (4096, 1, (17, 9, 3000))])
+def test_ln_modulate_pieces(cuda_ok, C, B, rows):
+    """Row shares of a CTA that cross segments and samples, more samples than
+    lanes, rings of two to four rows, fewer rows than SMs."""
+    from paper_2609_32415_gb300 import api
+    g = torch.Generator().manual_seed(C + B)
+    mode = torch.tensor([REUSE if s % 3 == 1 else COMPUTE for s in range(B)], dtype=torch.int32, device="cuda")
+    segs = [{"h": _bf((B, n, C), g).cuda(), "x": torch.full((B, n, C), float("nan"), dtype=torch.bfloat16, device="cuda"),
+             "shift": (torch.randn((B, C), generator=g) * 0.1).cuda(),
+             "scale": (torch.randn((B, C), generator=g) * 0.1).cuda(), "gated": i == 1} for i, n in enumerate(rows)]
+    api.refadapt_ln_modulate(segs, C, mode=mode)
+    torch.cuda.synchronize()
+    for i, sd in enumerate(segs):
+        for s in range(B):
+            got = f64(sd["x"][s])
+            if i == 1 and s % 3 == 1:
+                assert np.isnan(got).all()
+                continue
+            if got.size == 0:
+                continue
+            ref = dit.round_bf16(dit.layer_norm_modulate(f64(sd["h"][s]), sd["shift"][s].double().cpu().numpy(),
+                                                         sd["scale"][s].double().cpu().numpy(), 1e-6))
+            ok, nbad, eq = _close(got, ref, 0.99)
+            assert ok, (i, s, nbad, eq)
+
+
 def _gemm_case(B, K, N, rows_list, epi, g, gated=None, modes=None, inplace=False, tile_mode=0):
     from paper_2609_32415_gb300 import api
     from paper_2609_32415_gb300._lib import RA_EPI_GELU, RA_EPI_RESID, RA_EPI_STORE
