@@ -58,21 +58,21 @@ __device__ __forceinline__ void g_ff_add(float& hi, float& lo, float x) {
 
 // Thread 0 of the deciding CTA: at block 0 opens step t (t = 0 or an expired
 // bounded age forces a full refresh); returns the step's full-refresh flag.
-__device__ __forceinline__ int32_t open_step(const Params& p) {
+// a_full, full_step: the state's, loaded by the caller (early, where it can).
+__device__ __forceinline__ int32_t open_step(const Params& p, int32_t a_full, int32_t full_step) {
   ra_state* st = p.st;
   if (p.b == 0) {
-    if (p.t == 0) {
-      st->full_step = 1;
-      st->a_full = 0;
-    } else if (p.t - st->a_full >= p.delta_max) {
-      st->full_step = 1;
-      st->a_full = p.t;
-    } else {
-      st->full_step = 0;
-    }
+    full_step = (p.t == 0 || p.t - a_full >= p.delta_max) ? 1 : 0;
+    st->full_step = full_step;
+    if (full_step) st->a_full = p.t;
     st->step = p.t;
   }
-  return st->full_step;
+  return full_step;
+}
+
+// Sample s's reactivated latch before this block's decision (block 0 clears it).
+__device__ __forceinline__ int32_t reactivated_before(const Params& p, int s) {
+  return p.b == 0 ? 0 : reinterpret_cast<const int32_t*>(p.st + 1)[s];
 }
 
 // One warp: M_{t-1,b,h} of (sample, head) row sh from its mass partials
@@ -111,8 +111,10 @@ __device__ __forceinline__ void score_term(int cue, float dh, float mh, float& g
 // Sample s's decision given its per-head terms term(h, g, e) (have: a score
 // exists, t >= 1 with D and M): gbar = mean_h g in two-float sums over the
 // heads in order, compared with theta in fp64; mode and latch per Algorithm 1.
+// latch: reactivated_before(p, s).
 template <class Term>
-__device__ __forceinline__ void decide_sample(const Params& p, int s, int32_t full_step, bool have, Term term) {
+__device__ __forceinline__ void decide_sample(const Params& p, int s, int32_t full_step, int32_t latch, bool have,
+                                              Term term) {
   int32_t* reactivated = reinterpret_cast<int32_t*>(p.st + 1);
   int32_t* boundary = reactivated + p.B;
   if (p.b == 0) {
@@ -134,7 +136,7 @@ __device__ __forceinline__ void decide_sample(const Params& p, int s, int32_t fu
   int32_t mode;
   if (full_step) {
     mode = RA_MODE_FULL;
-  } else if (reactivated[s]) {
+  } else if (latch) {
     mode = RA_MODE_COMPUTE;
   } else {
     const bool cross = (p.forced_boundary >= 0) ? (p.b >= p.forced_boundary) : (have && gbar >= p.theta);
@@ -156,7 +158,7 @@ __device__ __forceinline__ void decide_sample(const Params& p, int s, int32_t fu
 __device__ __forceinline__ void decide(const Params& p, float* m_sh, volatile int32_t* full_step_sh) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nwarps = blockDim.x >> 5;
-  if (threadIdx.x == 0) *full_step_sh = open_step(p);
+  if (threadIdx.x == 0) *full_step_sh = open_step(p, p.st->a_full, p.st->full_step);
   for (int sh = warp; sh < p.B * p.H; sh += nwarps) {
     const float m = p.mp ? head_exposure(p, sh) : 0.f;
     if (lane == 0) {
@@ -168,7 +170,7 @@ __device__ __forceinline__ void decide(const Params& p, float* m_sh, volatile in
   const int32_t full_step = *full_step_sh;
   const bool have = (p.t >= 1) && p.qd && p.mp;
   for (int s = threadIdx.x; s < p.B; s += blockDim.x)
-    decide_sample(p, s, full_step, have, [&](int h, float& g, float& e) {
+    decide_sample(p, s, full_step, reactivated_before(p, s), have, [&](int h, float& g, float& e) {
       score_term(p.cue, p.qd[s * p.H + h], m_sh[s * p.H + h], g, e);
     });
 }
