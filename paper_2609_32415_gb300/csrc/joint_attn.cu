@@ -67,14 +67,15 @@ constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLowestMax = -1e30f;
 constexpr float kRescaleThresh = 8.0f;  // log2 units: p <= 2^8 between rescales
 
-template <int D>
+// DUAL: one Q tile and a deeper ring for two streams of key tiles.
+template <int D, bool DUAL = false>
 struct Cfg {
   static constexpr int CHUNKS = D / 64;           // 64-element (128-byte) swizzle chunks per row
   static constexpr int CHUNK_BYTES = BM * 128;    // one chunk of a 128-row tile
   static constexpr int TILE_BYTES = BM * D * 2;   // one Q, K or V tile (BN == BM)
-  static constexpr int STAGES = (D == 128) ? 2 : 4;
+  static constexpr int STAGES = DUAL ? (D == 128 ? 3 : 6) : (D == 128 ? 2 : 4);
   static constexpr int OFF_Q = 0;                 // Q tiles A and B
-  static constexpr int OFF_K = OFF_Q + 2 * TILE_BYTES;
+  static constexpr int OFF_K = OFF_Q + (DUAL ? 1 : 2) * TILE_BYTES;
   static constexpr int OFF_V = OFF_K + STAGES * TILE_BYTES;
   static constexpr int OFF_BAR = OFF_V + STAGES * TILE_BYTES;
   // q_full, k_full[S], k_empty[S], v_full[S], v_empty[S], s_full[2], p_ready[2], o_done[2], drain, parts_full
@@ -89,9 +90,9 @@ struct Cfg {
   static constexpr int OFF_STATS = (SMEM_BYTES + 15) / 16 * 16;
   static constexpr int SPLIT_BYTES = OFF_STATS + MAX_SPLIT * 2 * BM * 16;
   static constexpr int SPLIT_ALLOC = SPLIT_BYTES + 1024;
-  static_assert(2 * (2 * BM * D * 4 / MAX_SPLIT) * (MAX_SPLIT - 1) <= OFF_BAR && 2 * BM * D * 4 <= OFF_BAR,
+  static_assert(DUAL || (2 * (2 * BM * D * 4 / MAX_SPLIT) * (MAX_SPLIT - 1) <= OFF_BAR && 2 * BM * D * 4 <= OFF_BAR),
                 "O parts fit the tile buffers");
-  static_assert(SPLIT_ALLOC <= 232448, "shared memory budget");
+  static_assert(DUAL || SPLIT_ALLOC <= 232448, "shared memory budget");
   static constexpr uint32_t TMEM_COLS = 512;
   static constexpr uint32_t TM_S = 0, TM_O = 256;       // + 128 * tile
   static_assert(SMEM_ALLOC <= 232448, "shared memory budget");
@@ -104,7 +105,7 @@ struct Params {
   int32_t nk[3];  // key rows per role
   int32_t q_tiles[3];
   int32_t q_blocks[3];  // items: groups of `group` Q tiles
-  int32_t group;        // Q tiles per item, 1 or 2
+  int32_t group;        // Q tiles per item: 2, or 1 (KIND_DUAL)
   uint32_t per_inv[2];  // 2^32 / items per head, rounded up (with reference rows, without), or 0: divide
   int32_t b0, nb;       // samples of this launch: [b0, b0 + nb)
   int32_t part;         // PART_ALL, PART_ROUNDS or PART_REST of the live items
@@ -335,11 +336,68 @@ __device__ __forceinline__ void merge_split(const WaitCtl& ctl, uint8_t* smem, u
   }
 }
 
+// Merge of the two streams of an item (both warpgroups; thread = row): each
+// reads the other's row maximum and sums (through the Q buffer, idle by then),
+// then combines both accumulators over its half of the columns. Leaves the
+// item's l and l_ref in l, lref.
+template <int D>
+__device__ __forceinline__ void merge_dual(const WaitCtl& ctl, uint8_t* smem, uint64_t* o_done, uint32_t o_tmem, bool ok,
+                                           bool second, bool valid, int t, int row, float m, float& l, float& lref,
+                                           __nv_bfloat16* orow) {
+  float4* st = reinterpret_cast<float4*>(smem + Cfg<D, true>::OFF_Q);  // [stream][row]
+  const bool done = __all_sync(0xffffffffu, mbar_wait(o_done, 0, ctl) && (!second || mbar_wait(o_done + 1, 0, ctl)));
+  if (done) st[t * BM + row] = make_float4(m, ok ? l : NAN, lref, 0.f);
+  named_bar_sync(3, 256);
+  if (!done) return;
+  tc_fence_after();
+  const float4 s0 = st[row], s1 = st[BM + row];
+  float a0 = 1.f, a1 = 0.f;
+  l = s0.y;
+  lref = s0.z;
+  if (second) {
+    const float mx = fmaxf(s0.x, s1.x);
+    a0 = ex2_approx(s0.x - mx);
+    a1 = ex2_approx(s1.x - mx);
+    l = fmaf(s1.y, a1, s0.y * a0);
+    lref = fmaf(s1.z, a1, s0.z * a0);
+  }
+  const float inv_l = 1.f / l;
+  a0 *= inv_l;
+  a1 *= inv_l;
+#pragma unroll 1
+  for (int c = t * (D / 2); c < (t + 1) * (D / 2); c += 16) {
+    uint32_t v0[16], v1[16];
+    tmem_ld16(o_tmem + c, v0);
+    tmem_ld16(o_tmem + 128 + (second ? c : 0), v1);
+    tmem_ld_wait();
+    uint32_t pk[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      float x = __uint_as_float(v0[2 * i]) * a0, y = __uint_as_float(v0[2 * i + 1]) * a0;
+      if (second) {
+        x = fmaf(__uint_as_float(v1[2 * i]), a1, x);
+        y = fmaf(__uint_as_float(v1[2 * i + 1]), a1, y);
+      }
+      pk[i] = pack_bf16x2(x, y);
+    }
+    if (valid) {
+      uint4* dst = reinterpret_cast<uint4*>(orow + c);
+      dst[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+      dst[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+    }
+  }
+}
+
 // SPLIT: a cluster of CTAs shares one item, each rank a contiguous range of
 // its key tiles; the ranks' partial results meet in distributed shared memory.
-template <int D, bool SPLIT>
+// DUAL: an item is one Q tile; two streams, the even and the odd key tiles, take
+// the places of the two tiles (the same issue order: one stream's products run
+// while the other's softmax does) and are merged in TMEM at the end.
+enum { KIND_PAIR = 0, KIND_SPLIT = 1, KIND_DUAL = 2 };
+template <int D, int KIND>
 __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid_constant__ Params p) {
-  using C = Cfg<D>;
+  constexpr bool SPLIT = KIND == KIND_SPLIT, DUAL = KIND == KIND_DUAL;
+  using C = Cfg<D, DUAL>;
   constexpr int S = C::STAGES;
   // The rest of a call starts beside its whole rounds and depends on nothing of
   // theirs; it starts after their pdl_launch(), so after what they wait for.
@@ -427,12 +485,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
     role = 2;
   }
   const int tileA = p.group * qb;
-  const bool has_b = p.group == 2 && (tileA + 1) < p.q_tiles[role];
+  const bool has_b = !DUAL && (tileA + 1) < p.q_tiles[role];  // a second Q tile
   if (SPLIT) cluster_arrive();  // this CTA has started: its shared memory exists
   const WaitCtl ctl{abort_flag, p.err_word, p.budget_ns};
   const int nkv_all = p.kv_tiles[0] + p.kv_tiles[1] + p.kv_tiles[2];
   const int j0 = SPLIT ? nkv_all * rank / nrank : 0;  // this CTA's first key tile
   const int nkv = SPLIT ? nkv_all * (rank + 1) / nrank - j0 : nkv_all;
+  const bool second = DUAL ? nkv > 1 : has_b;  // the second softmax warpgroup works
   // Register split: warpgroup 0 (producer, MMA issuer, two idle warps) gives
   // up registers to the two softmax warpgroups: 4 x 56 + 8 x 224 = 12 x 168,
   // the launch allocation.
@@ -535,43 +594,74 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
         const uint32_t sq = smem_u32(smem + C::OFF_Q);
         const uint32_t sk = smem_u32(smem + C::OFF_K);
         const uint32_t sv = smem_u32(smem + C::OFF_V);
-        const int ntile = has_b ? 2 : 1;
         bool issued_any = false;
+        // Q K_j^T into S_t, Q tile t (DUAL: the one tile).
         auto qk = [&](int j, int t) {
           const int s = j % S;
-          umma_ss_ksteps<D / 16>(tmem + C::TM_S + 128 * t, sdesc_sw128(sq + t * C::TILE_BYTES, 16, 1024),
+          umma_ss_ksteps<D / 16>(tmem + C::TM_S + 128 * t,
+                                 sdesc_sw128(sq + (DUAL ? 0 : t) * C::TILE_BYTES, 16, 1024),
                                  sdesc_sw128(sk + s * C::TILE_BYTES, 16, 1024), IDESC_QK, 0u);
           umma_commit(s_full + t);
         };
-        auto pv = [&](int j, int t) {
+        // O_t += P_t V_j. O_t is read only after the last P V (the epilogue); a
+        // rescale reads it after s_full of the next tile, whose commit covers
+        // this P V too.
+        auto pv = [&](int j, int t, bool first, bool last) {
           const int s = j % S;
           umma_ts_ksteps8(tmem + C::TM_O + 128 * t, tmem + C::TM_S + 128 * t,
-                          sdesc_sw128(sv + s * C::TILE_BYTES, C::CHUNK_BYTES, 1024), IDESC_PV, j > 0 ? 1u : 0u);
-          // O_t is read only after the last P V (the epilogue); a rescale reads it
-          // after s_full of the next tile, whose commit covers this P V too.
-          if (j + 1 == nkv) umma_commit(o_done + t);
+                          sdesc_sw128(sv + s * C::TILE_BYTES, C::CHUNK_BYTES, 1024), IDESC_PV, first ? 0u : 1u);
+          if (last) umma_commit(o_done + t);
         };
         bool ok = mbar_wait(q_full, 0, ctl) && mbar_wait(k_full, 0, ctl);
-        if (ok) {
-          tc_fence_after();
-          for (int t = 0; t < ntile; ++t) qk(0, t);
-          umma_commit(k_empty);
-          issued_any = true;
-        }
-        for (int j = 0; ok && j < nkv; ++j) {
-          const int s = j % S;
-          const bool next = j + 1 < nkv;
-          if (!(ok = mbar_wait(v_full + s, (j / S) & 1, ctl))) break;
-          if (next && !(ok = mbar_wait(k_full + (j + 1) % S, ((j + 1) / S) & 1, ctl))) break;
-          for (int t = 0; t < ntile; ++t) {
-            if (!(ok = mbar_wait(p_ready + t, j & 1, ctl))) break;
+        if (DUAL) {
+          if (ok) {
             tc_fence_after();
-            pv(j, t);
-            if (next) qk(j + 1, t);  // S_t is free: PV_t(j) was issued first
+            qk(0, 0);
+            umma_commit(k_empty);
+            issued_any = true;
+            if (nkv > 1 && (ok = mbar_wait(k_full + 1, 0, ctl))) {
+              tc_fence_after();
+              qk(1, 1);
+              umma_commit(k_empty + 1);
+            }
           }
-          if (!ok) break;
-          umma_commit(v_empty + s);
-          if (next) umma_commit(k_empty + (j + 1) % S);
+          for (int j = 0; ok && j < nkv; ++j) {
+            const int s = j % S, t = j & 1;
+            const bool next = j + 2 < nkv;  // S_t's next key tile
+            if (!(ok = mbar_wait(v_full + s, (j / S) & 1, ctl))) break;
+            if (next && !(ok = mbar_wait(k_full + (j + 2) % S, ((j + 2) / S) & 1, ctl))) break;
+            if (!(ok = mbar_wait(p_ready + t, (j >> 1) & 1, ctl))) break;
+            tc_fence_after();
+            pv(j, t, j < 2, !next);
+            umma_commit(v_empty + s);
+            if (next) {
+              qk(j + 2, t);  // S_t is free: PV_t was issued first
+              umma_commit(k_empty + (j + 2) % S);
+            }
+          }
+        } else {
+          const int ntile = has_b ? 2 : 1;
+          if (ok) {
+            tc_fence_after();
+            for (int t = 0; t < ntile; ++t) qk(0, t);
+            umma_commit(k_empty);
+            issued_any = true;
+          }
+          for (int j = 0; ok && j < nkv; ++j) {
+            const int s = j % S;
+            const bool next = j + 1 < nkv;
+            if (!(ok = mbar_wait(v_full + s, (j / S) & 1, ctl))) break;
+            if (next && !(ok = mbar_wait(k_full + (j + 1) % S, ((j + 1) / S) & 1, ctl))) break;
+            for (int t = 0; t < ntile; ++t) {
+              if (!(ok = mbar_wait(p_ready + t, j & 1, ctl))) break;
+              tc_fence_after();
+              pv(j, t, j == 0, !next);
+              if (next) qk(j + 1, t);  // S_t is free: PV_t(j) was issued first
+            }
+            if (!ok) break;
+            umma_commit(v_empty + s);
+            if (next) umma_commit(k_empty + (j + 1) % S);
+          }
         }
         if (!ok && issued_any) {
           umma_commit(drain);
@@ -595,7 +685,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
       item_sh->x = b;
       item_sh->y = h;
       item_sh->z = role;
-      item_sh->w = tileA + t;
+      item_sh->w = DUAL ? tileA : tileA + t;
     }
     __syncwarp();
     const int quarter = warp & 3;        // TMEM lane quarter this warp may access
@@ -603,16 +693,17 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
     const uint32_t lane_off = uint32_t(quarter * 32) << 16;
     const uint32_t s_t = tmem + lane_off + C::TM_S + 128 * t;
     const uint32_t o_t = tmem + lane_off + C::TM_O + 128 * t;
-    const bool active = (t == 0) || has_b;
+    const bool active = (t == 0) || second;
     const float sl2 = p.scale_log2;
     const float bias_l2 = (role == 2 && p.bias) ? __ldg(p.bias + h) * kLog2e : 0.f;
     // A range of a split item may hold masked keys alone (a reference bias of
     // -inf): a finite start keeps their probabilities 0.
-    float m = SPLIT ? kLowestMax : -INFINITY, l = 0.f, lref = 0.f;
+    float m = KIND != KIND_PAIR ? kLowestMax : -INFINITY, l = 0.f, lref = 0.f;
     bool ok = active;
-    for (int j = 0; ok && j < nkv; ++j) {
+    // DUAL: this warpgroup's key tiles are t, t + 2, ...
+    for (int j = 0; ok && (DUAL ? 2 * j + t : j) < nkv; ++j) {
       int r, row0;
-      kv_tile(p, j0 + j, r, row0);
+      kv_tile(p, DUAL ? 2 * j + t : j0 + j, r, row0);
       const int nvalid = min(BN, p.nk[r] - row0);
       const float badd = (r == 1) ? bias_l2 : 0.f;
       ok = __all_sync(0xffffffffu, mbar_wait(s_full + t, j & 1, ctl));
@@ -700,16 +791,19 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
     if (ok) ok = __all_sync(0xffffffffu, mbar_wait(o_done + t, 0, ctl));
     const int eb = item_sh->x, eh = item_sh->y, erole = item_sh->z, tile = item_sh->w;
     const int grow = tile * BM + row;
-    const bool valid = active && grow < p.nq[erole];
+    const bool valid = (active || DUAL) && grow < p.nq[erole];
     __nv_bfloat16* orow = p.o_ptr[erole] + eb * p.o_sb[erole] + eh * p.o_sh[erole] + int64_t(grow) * p.o_sn[erole];
     float inv_l;
     if (SPLIT) {
       merge_split<D>(ctl, smem, parts_full, o_t, ok && active, has_b, valid, rank, nrank, t, row, m, l, lref, orow);
       inv_l = 1.f / l;
+    } else if (DUAL) {
+      merge_dual<D>(ctl, smem, o_done, tmem + lane_off + C::TM_O, ok && active, second, valid, t, row, m, l, lref, orow);
+      inv_l = 1.f / l;
     } else {
       inv_l = 1.f / l;
     }
-    if (!SPLIT && ok) {
+    if (KIND == KIND_PAIR && ok) {
       tc_fence_after();
 #pragma unroll
       for (int c0 = 0; c0 < D; c0 += 32) {
@@ -738,7 +832,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
     for (int o = 16; o > 0; o >>= 1) mv += __shfl_xor_sync(0xffffffffu, mv, o);
     if (lane == 0) red[4 * t + quarter] = mv;
     named_bar_sync(1 + t, 128);
-    if (ok && active && erole != 1 && rank == 0 && quarter == 0 && lane == 0) {
+    if (ok && active && erole != 1 && rank == 0 && !(DUAL && t == 1) && quarter == 0 && lane == 0) {
       const int idx = (erole == 0) ? tile : p.q_tiles[0] + tile;
       p.mass_partial[(int64_t(eb) * p.H + eh) * p.mpl + idx] =
           ((red[4 * t] + red[4 * t + 1]) + red[4 * t + 2]) + red[4 * t + 3];
@@ -762,13 +856,13 @@ struct KernelInfo {
   Kernel fn;
   int smem;
 };
-inline KernelInfo kernel_of(int d, bool split) {
-  if (d == 128)
-    return split ? KernelInfo{joint_attn_kernel<128, true>, Cfg<128>::SPLIT_ALLOC}
-                 : KernelInfo{joint_attn_kernel<128, false>, Cfg<128>::SMEM_ALLOC};
-  return split ? KernelInfo{joint_attn_kernel<64, true>, Cfg<64>::SPLIT_ALLOC}
-               : KernelInfo{joint_attn_kernel<64, false>, Cfg<64>::SMEM_ALLOC};
+template <int D>
+KernelInfo kernel_of(int kind) {
+  if (kind == KIND_SPLIT) return {joint_attn_kernel<D, KIND_SPLIT>, Cfg<D>::SPLIT_ALLOC};
+  if (kind == KIND_DUAL) return {joint_attn_kernel<D, KIND_DUAL>, Cfg<D, true>::SMEM_ALLOC};
+  return {joint_attn_kernel<D, KIND_PAIR>, Cfg<D>::SMEM_ALLOC};
 }
+inline KernelInfo kernel_of(int d, int kind) { return d == 128 ? kernel_of<128>(kind) : kernel_of<64>(kind); }
 
 // Clusters of cs CTAs of the split kernel that can run at once on the current
 // device (they live inside one GPC, so the floorplan decides); cached per
@@ -784,7 +878,7 @@ int max_clusters(int d, int cs) {
   std::lock_guard<std::mutex> lk(mu);
   int& n = cache[dev][d == 128 ? 1 : 0][cs];
   if (n == 0) {
-    const KernelInfo k = kernel_of(d, true);
+    const KernelInfo k = kernel_of(d, KIND_SPLIT);
     cudaError_t e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, k.smem);
     cudaLaunchConfig_t cfg;
     std::memset(&cfg, 0, sizeof(cfg));
@@ -817,7 +911,7 @@ ra_status launch(const Params& p, int d, int64_t items, int cs, cudaStream_t st)
     set_error("%s: too many rows", who);
     return RA_EINVAL;
   }
-  const KernelInfo k = kernel_of(d, cs > 1);
+  const KernelInfo k = kernel_of(d, p.group == 1 ? KIND_DUAL : cs > 1 ? KIND_SPLIT : KIND_PAIR);
   const ra_status as = ensure_dynamic_smem(reinterpret_cast<const void*>(k.fn), k.smem, who);
   if (as != RA_OK) return as;
   cudaLaunchConfig_t cfg;
@@ -849,7 +943,7 @@ ra_status launch(const Params& p, int d, int64_t items, int cs, cudaStream_t st)
 
 // How a call's items are launched.
 struct Plan {
-  int group;     // Q tiles per item
+  int group;     // Q tiles per item: 2, or 1 with two streams of key tiles
   int cs;        // CTAs per split item, 1: nothing is split
   int rest_max;  // whole rounds unsplit and a rest of at most this many items split; 0: one launch
 };
@@ -864,31 +958,40 @@ Live live_items(const Params& p, int group, int nb) {
   return {int64_t(p.H) * nb * (q[0] + q[1] + q[2]), int64_t(p.H) * nb * (q[0] + q[2])};
 }
 
-// The cheapest launch by a model of a CTA's time (microseconds on a GB300,
-// from clock counters and whole launches): a fixed part (first mode load,
-// set-up, first loads, cold instruction fetches, epilogue), so much per key tile
-// with two Q tiles or one, and the merge of a split item. A split pays where an
-// unsplit launch leaves SMs idle for long: 72 items of 98 key tiles (every 8th
-// target row of the image-edit shape) take 82 us in clusters of two, 145 us
-// unsplit; 312 items of 26 key tiles (two rounds of 152 and 8) 112 us with the
-// rest in clusters of four, 133 us in three rounds. One Q tile per item pays
-// when all items fit one round (two samples of 77 + 1000 + 500 rows, 8 heads,
-// d = 64: 21.5 against 23.9 us). Modes are on the device, so a call with modes
-// is weighed with and without its reference rows.
+// The cheapest launch by a model of a CTA's time (microseconds, fitted to whole
+// launches on a GB300): a fixed part (launch, mode load, set-up, first loads of
+// all CTAs at once, cold instruction fetches, epilogue), so much per key tile of
+// a pair of Q tiles, or per two key tiles of one Q tile in two streams, and the
+// merge of a split item. What each form is for:
+//   pairs unsplit         full rounds: the least traffic per product;
+//   clusters              few items of many keys: every 8th target row of the
+//                         image-edit shape (72 items of 98 key tiles) 82 us in
+//                         clusters of two, 143 unsplit, 87 in two streams;
+//   rounds, rest split    312 items of 26 key tiles (two rounds of 152 and 8)
+//                         112 us, 131 in three rounds;
+//   one tile, two streams items that fit few rounds: 8 heads, d = 64, of
+//                         32 + 256 + 256 rows 8.5 against 11.4 us, of 77 + 1000
+//                         + 500 rows 16.5 against 22.9 (half the latency per
+//                         key, but twice the K and V traffic per product: 55
+//                         against 46 us where it takes a second round).
+// Modes are on the device, so a call with modes is weighed with all its
+// reference rows, with none and (several samples) with half.
 ra_status make_plan(const Params& p, int d, int nb, int slots, Plan* out) {
   const int n = p.kv_tiles[0] + p.kv_tiles[1] + p.kv_tiles[2];
-  const double merge = 6.0, second_launch = 2.0, fixed[3] = {0, 3.7, 4.7};
-  const double tile[3] = {0, d == 128 ? 1.22 : 1.15, d == 128 ? 1.41 : 1.3};
+  const bool wide = d == 128;
+  const double merge = 6.8;
   auto cta = [&](int group, int cs) {
-    return fixed[group] + (n + cs - 1) / cs * tile[group] + (cs > 1 ? merge : 0.0);
+    if (group == 1) return (wide ? 7.5 : 5.5) + (n + 1) / 2 * (wide ? 1.64 : 1.25);
+    return (wide ? 8.7 : 6.5) + (n + cs - 1) / cs * (wide ? 1.37 : 1.19) + (cs > 1 ? merge : 0.0);
   };
   auto rounds = [](int64_t items, int64_t width) { return double((items + width - 1) / width); };
   *out = Plan{2, 1, 0};
   double best = 0;
   for (int group = 2; group >= 1; --group) {
     const Live lv = live_items(p, group, nb);
-    const int64_t cases[2] = {lv.most, p.mode ? lv.least : lv.most};
-    for (int cs = 1; cs <= MAX_SPLIT && cs <= n; cs *= 2) {
+    const int64_t cases[3] = {lv.most, p.mode ? lv.least : lv.most, (lv.most + lv.least) / 2};
+    const int n_cases = p.mode ? (nb > 1 ? 3 : 2) : 1;
+    for (int cs = 1; cs <= (group == 2 ? MAX_SPLIT : 1) && cs <= n; cs *= 2) {
       int clusters = slots;
       if (cs > 1) {
         clusters = max_clusters(d, cs);
@@ -897,22 +1000,23 @@ ra_status make_plan(const Params& p, int d, int nb, int slots, Plan* out) {
       }
       int rest_max = 0;
       if (cs > 1 && lv.most >= slots) {
-        const double whole = cta(group, 1) - second_launch;
-        rest_max = int(whole / cta(group, cs)) * clusters;
+        rest_max = int(cta(group, 1) / cta(group, cs)) * clusters;
         if (rest_max > slots - 1) rest_max = slots - 1;
-        if (rest_max == 0 || group == 1 || lv.most > 2147483647) continue;
+        if (rest_max == 0 || lv.most > 2147483647) continue;
       }
       double us = 0;
-      for (int64_t live : cases) {
+      for (int i = 0; i < n_cases; ++i) {
+        const int64_t live = cases[i];
         if (rest_max == 0) {
           us += rounds(live, clusters) * cta(group, cs);
           continue;
         }
         const int64_t whole = round_items(int(live), slots, rest_max);
-        us += rounds(whole, slots) * cta(group, 1) + second_launch;
+        us += rounds(whole, slots) * cta(group, 1);
         if (live > whole) us += rounds(live - whole, clusters) * cta(group, cs);
       }
-      if (best == 0 || us < 0.97 * best) {
+      // A second launch has to promise a little more than the model's error.
+      if (best == 0 || us < (rest_max > 0 ? 0.96 : 0.99) * best) {
         best = us;
         *out = Plan{group, cs, rest_max};
       }

@@ -1,6 +1,6 @@
 """Launches of the attention that split an item's keys over a cluster, run whole
-rounds and a split rest, or take one Q tile per item: against the oracle on a
-few heads, and bit for bit on a second run.
+rounds and a split rest, or take one Q tile per item in two streams of key
+tiles: against the oracle on a few heads, and bit for bit on a second run.
 
 Element bound: P and the output are rounded to bf16 (unit roundoff 2^-9 each),
 two independent errors that leave O with a 2-norm error of at most 2^-9 sqrt(2)
@@ -22,14 +22,16 @@ def _assert_close(got, ref, what=""):
 
 # text, ref, tgt rows, heads, d, modes; what the launch model picks is named.
 CASES = [
-    ((33, 5000, 130), 2, 128, [REUSE]),              # clusters of four (4 items of 43 key tiles)
-    ((33, 5000, 130), 2, 64, [BOUNDARY, REUSE]),     # clusters of four, reference items live in one sample
-    ((33, 700, 1500), 24, 64, None),                 # whole rounds, then clusters
-    ((100, 900, 1900), 12, 128, [FULL]),             # 152 items and a rest of 4
-    ((100, 900, 1900), 18, 128, [REUSE]),            # a rest of 10 that only reusing leaves
-    ((100, 300, 1900), 10, 64, [REUSE, COMPUTE]),    # the rest in clusters of two
-    ((40, 100, 200), 3, 64, [COMPUTE, REUSE]),       # one Q tile per item
-    ((0, 0, 77), 3, 128, None),                      # one key tile: nothing to split
+    ((33, 5000, 130), 2, 128, [REUSE]),              # one tile, two streams: 43 key tiles
+    ((33, 5000, 130), 2, 64, [BOUNDARY, REUSE]),     # the same, reference items live in one sample
+    ((33, 700, 1500), 24, 64, None),                 # the same in three rounds, 19 key tiles
+    ((40, 100, 200), 3, 64, [COMPUTE, REUSE]),       # few key tiles
+    ((0, 0, 77), 3, 128, None),                      # one key tile: no second stream
+    ((0, 0, 200), 2, 64, None),                      # two: one each
+    ((100, 900, 1900), 12, 128, [FULL]),             # 152 items, a rest of 4 in clusters of four
+    ((200, 900, 1700), 22, 128, [REUSE]),            # a rest of 24 that only reusing leaves
+    ((100, 1800, 1800), 12, 128, [FULL]),            # a rest of 52 in clusters of two
+    ((100, 300, 1900), 10, 64, [REUSE, COMPUTE]),    # mixed modes over more than a round
 ]
 
 
@@ -59,29 +61,37 @@ def test_split_launches_match_oracle(cuda_ok, rows, H, d, modes):
         assert torch.equal(out[r].view(torch.int16), again[r].view(torch.int16)), r
 
 
-@pytest.mark.parametrize("d", [64, 128])
-def test_split_item_without_reference_queries(cuda_ok, d):
-    """Sampled target rows, no reference queries: 48 items in clusters of two."""
+@pytest.mark.parametrize("H,d", [(8, 64), (8, 128), (24, 128)])
+def test_split_item_without_reference_queries(cuda_ok, H, d):
+    """Sampled target rows, no reference queries, 72 key tiles: 16 items in
+    clusters of four, 48 in clusters of two. Head 0's reference bias of -inf
+    leaves whole key ranges of its items with probability 0."""
     from paper_2609_32415_gb300 import api
-    B, H, n = 1, 24, {"text": 40, "ref": 1500, "tgt": 1000}
+    B, n = 1, {"text": 40, "ref": 8000, "tgt": 1000}
     segs = make_segments(B, H, d, n, gen=torch.Generator().manual_seed(d), std=1.0)
     q = [segs["text"][0], None, segs["tgt"][0][:, :, ::5, :]]
     out = [torch.zeros_like(q[0]), None, torch.zeros((B, H, 200, d), dtype=torch.bfloat16, device="cuda")]
     mp = api.alloc_mass_partial(B, H, 40, 200)
     err = torch.zeros(1, dtype=torch.int32, device="cuda")
-    api.refadapt_joint_attn(q, [segs[r][1] for r in ROLES], [segs[r][2] for r in ROLES], out, mp, err_word=err)
+    bias = torch.zeros(H, device="cuda")
+    bias[0] = float("-inf")
+    api.refadapt_joint_attn(q, [segs[r][1] for r in ROLES], [segs[r][2] for r in ROLES], out, mp, err_word=err,
+                            ref_logit_bias=bias)
     torch.cuda.synchronize()
     api.refadapt_check_error(err)
-    hs = [0, 11, 23]
+    hs = [1, H - 1]
     ref = oracle_block({r: [x[:, hs] for x in segs[r]] for r in ROLES}, 0, FULL, d ** -0.5)
     _assert_close(out[2][0, hs], ref["O"]["tgt"][:, ::5])
     _assert_close(out[0][0, hs], ref["O"]["text"])
+    cut = {r: [x[:, :1, :0] if r == "ref" else x[:, :1] for x in segs[r]] for r in ROLES}
+    _assert_close(out[2][0, :1], oracle_block(cut, 0, REUSE, d ** -0.5)["O"]["tgt"][:, ::5])
+    assert float(mp[0, 0].abs().max()) == 0.0
 
 
 @pytest.mark.parametrize("d", [64, 128])
 def test_split_range_of_masked_keys(cuda_ok, d):
-    """A reference bias of -inf leaves whole key ranges of a split item with
-    probability 0: the target rows attend to text and target keys alone."""
+    """A reference bias of -inf: a stream of key tiles starts with keys of
+    probability 0; the target rows attend to text and target keys alone."""
     B, H, n = 1, 2, {"text": 33, "ref": 5000, "tgt": 130}
     segs = make_segments(B, H, d, n, gen=torch.Generator().manual_seed(d + 1), std=1.0)
     out, mp = _run(segs, B, H, d, n, [REUSE], bias=[float("-inf"), 0.5])
@@ -95,29 +105,30 @@ def test_split_range_of_masked_keys(cuda_ok, d):
     assert abs(float(m2.double().sum()) / n["tgt"] - full["M"][0]) <= M_ABS
 
 
-@pytest.mark.parametrize("rows,H", [((33, 5000, 130), 2), ((100, 1000, 1800), 11)])
-def test_split_launches_write_the_cache(cuda_ok, rows, H):
-    """The fused cache write with each rank of a cluster storing its own key
-    range: the refreshing sample's slot equals the fresh rows, the reusing
-    one's is untouched, a_b is stamped."""
+@pytest.mark.parametrize("rows,H,modes", [((33, 5000, 130), 2, [COMPUTE, REUSE]), ((100, 1800, 1800), 12, [FULL])])
+def test_split_launches_write_the_cache(cuda_ok, rows, H, modes):
+    """The fused cache write from two streams, and from whole rounds and split
+    rest items (each rank of a cluster stores its own key range): a refreshing
+    sample's slot equals the fresh rows, a reusing one's is untouched, a_b is
+    stamped."""
     from paper_2609_32415_gb300 import api
-    B, d, n = 2, 128, dict(zip(ROLES, rows))
+    B, d, n = len(modes), 128, dict(zip(ROLES, rows))
     segs = make_segments(B, H, d, n, gen=torch.Generator().manual_seed(H))
     slot = [torch.full_like(x, 0.25) for x in segs["ref"]]
     a_b = torch.full((B,), -1, dtype=torch.int32, device="cuda")
     out = empty_outputs(B, H, d, n)
     mp = api.alloc_mass_partial(B, H, n["text"], n["tgt"])
     err = torch.zeros(1, dtype=torch.int32, device="cuda")
-    mode = torch.tensor([COMPUTE, REUSE], dtype=torch.int32, device="cuda")
+    mode = torch.tensor(modes, dtype=torch.int32, device="cuda")
     api.refadapt_joint_attn([segs["text"][0], slot[0], segs["tgt"][0]], [segs["text"][1], slot[1], segs["tgt"][1]],
                             [segs["text"][2], slot[2], segs["tgt"][2]], [out[r] for r in ROLES], mp, mode=mode,
                             err_word=err, ref_fresh=tuple(segs["ref"]), a_b=a_b, step=5)
     torch.cuda.synchronize()
     api.refadapt_check_error(err)
-    assert a_b.tolist() == [5, -1]
+    assert a_b.tolist() == [5 if m != REUSE else -1 for m in modes]
     for got, fresh in zip(slot, segs["ref"]):
-        assert torch.equal(got[0], fresh[0])
-        assert bool((got[1] == 0.25).all())
+        for s, m in enumerate(modes):
+            assert torch.equal(got[s], fresh[s]) if m != REUSE else bool((got[s] == 0.25).all())
     hs = [0, H - 1]
     ref = oracle_block({r: [x[:, hs] for x in segs[r]] for r in ROLES}, 0, COMPUTE, d ** -0.5)
     for r in ROLES:
