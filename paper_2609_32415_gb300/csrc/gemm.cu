@@ -94,7 +94,7 @@ constexpr int P_SMEM_ALLOC = P_SMEM_BYTES + 1024;
 static_assert(P_SMEM_ALLOC <= 232448, "shared memory budget");
 
 struct Seg {
-  int32_t rows, m_tiles, gated, pos_offset;
+  int32_t pos_offset, reserved;
   const float* bias;
   __nv_bfloat16* out;
   int64_t out_ss, out_sr;
@@ -107,17 +107,22 @@ struct Seg {
   const float* norm_w[2];  // QKV: q, k
 };
 
+// What every role reads before its first tile comes first: a kernel starts with
+// a cold constant cache, and each line it touches costs hundreds of cycles.
 struct Params {
-  CUtensorMap tm_a[3], tm_w[3];
-  Seg seg[3];
-  int32_t n_seg, B, N, K, C, kblocks;
-  int32_t bn;          // columns of a tile
+  int32_t n_seg, B, N, C, kblocks;
+  int32_t bn;                // columns of a tile
+  int32_t cols, cols_q;      // column tiles of N; of the query part (QKV)
+  int32_t rows[3], m_tiles[3], gated[3];
+  int32_t K;
   const int32_t* mode;
+  int32_t* err_word;
+  uint64_t budget_ns;
   const float4* rope;  // [pos][d/4]: (cos, sin) of two consecutive pairs
   int32_t rope_len;
   float norm_eps;
-  int32_t* err_word;
-  uint64_t budget_ns;
+  Seg seg[3];
+  CUtensorMap tm_a[3], tm_w[3];
 };
 
 struct Tile {
@@ -136,18 +141,18 @@ struct Walk {
   int64_t begin = 0;            // first tile of the piece
 
   __device__ __forceinline__ int piece_cols(const Params& p) const {
-    if (p.seg[g].gated) {
+    if (p.gated[g]) {
       const int m = __ldg(p.mode + s);
       if (m == RA_MODE_REUSE) return 0;
-      if (EPI == RA_EPI_QKV && m == RA_MODE_BOUNDARY) return p.C / p.bn;
+      if (EPI == RA_EPI_QKV && m == RA_MODE_BOUNDARY) return p.cols_q;
     }
-    return (p.N + p.bn - 1) / p.bn;
+    return p.cols;
   }
   // Tile t, or false past the last one.
   __device__ __forceinline__ bool at(const Params& p, int64_t t, Tile& r) {
     if (cols < 0) cols = piece_cols(p);
-    while (t - begin >= int64_t(p.seg[g].m_tiles) * cols) {
-      begin += int64_t(p.seg[g].m_tiles) * cols;
+    while (t - begin >= int64_t(p.m_tiles[g]) * cols) {
+      begin += int64_t(p.m_tiles[g]) * cols;
       if (++s == p.B) {
         s = 0;
         if (++g == p.n_seg) return false;
@@ -164,7 +169,7 @@ struct Walk {
     const uint32_t band_tiles = uint32_t(GROUP_M) * uint32_t(cols);
     const uint32_t band = rem / band_tiles, idx = rem - band * band_tiles;
     const int m_first = int(band) * GROUP_M;
-    const uint32_t rows = uint32_t(min(GROUP_M, p.seg[g].m_tiles - m_first));
+    const uint32_t rows = uint32_t(min(GROUP_M, p.m_tiles[g] - m_first));
     r.m0 = (m_first + int(idx % rows)) * TM;
     r.n0 = int(idx / rows) * p.bn;
     return true;
@@ -439,16 +444,17 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
   const uint32_t tmem = *tmem_slot;
   const WaitCtl ctl{abort_flag, p.err_word, p.budget_ns};
   pdl_launch();
-  pdl_wait();
+  if (warp != 0) pdl_wait();
 
   if (warp == 0) {
     if (lane == 0) {
       // -------------------------------------------------------------- producer
       for (int g = 0; g < p.n_seg; ++g)
-        if (p.seg[g].rows > 0) {
+        if (p.rows[g] > 0) {
           tma_prefetch_desc(&p.tm_a[g]);
           tma_prefetch_desc(&p.tm_w[g]);
         }
+      pdl_wait();
       int64_t it = 0;  // K steps issued
       bool ok = true;
       Walk<BM, EPI> walk;
@@ -520,7 +526,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
     for (int64_t t = blockIdx.x; walk.at(p, t, tl); t += gridDim.x) {
       const int buf = i & 1, use = i >> 1;
       w.row0 = tl.m0 + quarter * 32;
-      w.nrow = min(32, p.seg[tl.seg].rows - w.row0);
+      w.nrow = min(32, p.rows[tl.seg] - w.row0);
       w.acc = tmem + (uint32_t(quarter * 32) << 16) + uint32_t(buf * BN);
       if (!epilogue_tile<EPI, D>(p, tl, w, [&] {
             const bool ok = __all_sync(0xffffffffu, mbar_wait(tfull + buf, uint32_t(use & 1), ctl));
@@ -588,16 +594,17 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_pair_kernel(const __grid_cons
   const uint32_t tmem = *tmem_slot;
   const WaitCtl ctl{abort_flag, p.err_word, p.budget_ns};
   pdl_launch();
-  pdl_wait();
+  if (warp != 0) pdl_wait();
 
   if (warp == 0) {
     if (lane == 0) {
       // -------------------------------------------------------------- producer (both CTAs)
       for (int g = 0; g < p.n_seg; ++g)
-        if (p.seg[g].rows > 0) {
+        if (p.rows[g] > 0) {
           tma_prefetch_desc(&p.tm_a[g]);
           tma_prefetch_desc(&p.tm_w[g]);
         }
+      pdl_wait();
       const uint32_t full0 = mapa_shared(smem_u32(full), 0);  // rank 0's full barriers
       int64_t it = 0;
       bool ok = true;
@@ -688,7 +695,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_pair_kernel(const __grid_cons
     for (int64_t t = cid; walk.at(p, t, tl); t += ncl) {
       const int buf = i & 1, use = i >> 1;
       w.row0 = tl.m0 + int(rank) * 128 + quarter * 32;
-      w.nrow = min(32, p.seg[tl.seg].rows - w.row0);
+      w.nrow = min(32, p.rows[tl.seg] - w.row0);
       w.acc = tmem + (uint32_t(quarter * 32) << 16) + uint32_t(buf * BN);
       if (!epilogue_tile<EPI, D>(p, tl, w, [&] {
             const bool ok = __all_sync(0xffffffffu, mbar_wait(tfull + buf, uint32_t(use & 1), ctl));
@@ -858,6 +865,8 @@ extern "C" ra_status refadapt_gemm(const ra_gemm_args* a, void* stream) {
   const int tm = pair ? P_TM : BM;
   p.bn = plan.bn;
   const int64_t cols = (a->N + plan.bn - 1) / plan.bn;
+  p.cols = int32_t(cols);
+  p.cols_q = p.C / plan.bn;
   int64_t tiles = 0;
   for (int g = 0; g < a->n_seg; ++g) {
     const ra_gemm_seg& s = a->seg[g];
@@ -866,9 +875,9 @@ extern "C" ra_status refadapt_gemm(const ra_gemm_args* a, void* stream) {
       set_error("refadapt_gemm: seg %d rows < 0", g);
       return RA_EINVAL;
     }
-    d.rows = s.rows;
-    d.m_tiles = (s.rows + tm - 1) / tm;
-    d.gated = s.gated ? 1 : 0;
+    p.rows[g] = s.rows;
+    p.m_tiles[g] = (s.rows + tm - 1) / tm;
+    p.gated[g] = s.gated ? 1 : 0;
     d.pos_offset = s.pos_offset;
     d.bias = s.bias;
     if (s.gated && !a->mode) {
@@ -940,11 +949,11 @@ extern "C" ra_status refadapt_gemm(const ra_gemm_args* a, void* stream) {
     if (!encode_seg(&p.tm_a[g], as, a->B, 1, a->K, BK, BM, true) ||
         !encode_seg(&p.tm_w[g], ws, 1, 1, a->K, BK, pair ? plan.bn / 2 : plan.bn, true))
       return RA_EINVAL;
-    if (int64_t(d.m_tiles) * cols > 2147483647) {
+    if (int64_t(p.m_tiles[g]) * cols > 2147483647) {
       set_error("refadapt_gemm: seg %d: too many rows", g);
       return RA_EINVAL;
     }
-    tiles += int64_t(a->B) * d.m_tiles * cols;
+    tiles += int64_t(a->B) * p.m_tiles[g] * cols;
   }
   if (tiles == 0) return RA_OK;
   const Kernels kn = pick(a->epilogue, a->d);
