@@ -273,30 +273,36 @@ __device__ __forceinline__ bool epilogue_linear(const Params& p, const Tile& tl,
     if (EPI == RA_EPI_RESID) w.vec1[32 * j + lane] = __ldg(sg.gate + int64_t(tl.s) * sg.gate_ss + n0 + 64 * j + lane);
   }
   const char* res = nullptr;
-  uint4 rnext[4];
+  uint4 ra[4], rb[4];  // residuals of the next even and odd chunk
   if (EPI == RA_EPI_RESID && chunks > 0) {
     res = reinterpret_cast<const char*>(sg.resid + int64_t(tl.s) * sg.res_ss + int64_t(w.row0) * sg.res_sr + n0);
-    rows_fetch(res, 2 * sg.res_sr, w.nrow, rnext);
+    rows_fetch(res, 2 * sg.res_sr, w.nrow, ra);
+    if (chunks > 1) rows_fetch(res + 128, 2 * sg.res_sr, w.nrow, rb);
   }
   char* out = reinterpret_cast<char*>(sg.out + int64_t(tl.s) * sg.out_ss + int64_t(w.row0) * sg.out_sr + n0);
   __syncwarp();
   if (!ready()) return false;
   if (w.nrow <= 0 || chunks <= 0) return true;
   uint32_t v[32];
-  tmem_ld32(w.acc + 32 * w.half, v);
-#pragma unroll 1
-  for (int j = 0; j < chunks; ++j) {
+  if (EPI != RA_EPI_RESID) tmem_ld32(w.acc + 32 * w.half, v);
+  auto chunk = [&](int j, uint4 (&rc)[4]) {
     float x[32];
+    uint4 r[4];
+    if (EPI == RA_EPI_RESID) {
+      // Residuals two chunks ahead (one ahead left about 1000 cycles of global
+      // latency in every chunk); the accumulators are not loaded ahead in
+      // exchange, the registers allow one of the two without spills.
+      tmem_ld32(w.acc + 32 * w.half + 64 * j, v);
+      rows_turn(w.stage, rc, r);
+      if (j + 2 < chunks) rows_fetch(res + 128 * (j + 2), 2 * sg.res_sr, w.nrow, rc);
+    }
     tmem_ld_wait_for(v);
     add_cols(v, w.vec0 + 32 * j, x);
-    if (j + 1 < chunks) tmem_ld32(w.acc + 32 * w.half + 64 * (j + 1), v);
+    if (EPI != RA_EPI_RESID && j + 1 < chunks) tmem_ld32(w.acc + 32 * w.half + 64 * (j + 1), v);
     if (EPI == RA_EPI_GELU) {
 #pragma unroll
       for (int i = 0; i < 32; i += 2) gelu_tanh2(x[i], x[i + 1]);
     } else if (EPI == RA_EPI_RESID) {
-      uint4 r[4];
-      rows_turn(w.stage, rnext, r);
-      if (j + 1 < chunks) rows_fetch(res + 128 * (j + 1), 2 * sg.res_sr, w.nrow, rnext);
       const float4* g4 = reinterpret_cast<const float4*>(w.vec1 + 32 * j);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -311,6 +317,11 @@ __device__ __forceinline__ bool epilogue_linear(const Params& p, const Tile& tl,
       }
     }
     rows_store(w.stage, x, out + 128 * j, 2 * sg.out_sr, w.nrow);
+  };
+#pragma unroll 1
+  for (int j = 0; j < chunks; j += 2) {
+    chunk(j, ra);
+    if (j + 1 < chunks) chunk(j + 1, rb);
   }
   return true;
 }
