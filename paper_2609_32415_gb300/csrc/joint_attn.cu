@@ -196,6 +196,20 @@ __device__ __forceinline__ float max64(const float (&v)[64], int col0, int nvali
   return fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
 }
 
+// Sets the logits of columns >= nvalid (v[] holds columns col0 .. col0 + 63) to
+// -inf, so their probabilities are 0; returns the maximum of the rest.
+__device__ __forceinline__ float mask64(float (&v)[64], int col0, int nvalid) {
+  float m0 = -INFINITY, m1 = m0;
+#pragma unroll
+  for (int c = 0; c < 64; c += 4) {
+#pragma unroll
+    for (int e = c; e < c + 4; ++e) v[e] = (col0 + e < nvalid) ? v[e] : -INFINITY;
+    m0 = fmax3f(m0, v[c], v[c + 1]);
+    m1 = fmax3f(m1, v[c + 2], v[c + 3]);
+  }
+  return fmaxf(m0, m1);
+}
+
 __device__ __forceinline__ void tmem_ld64(uint32_t taddr, float (&v)[64]) {
   tmem_ld32(taddr, *reinterpret_cast<uint32_t(*)[32]>(&v[0]));
   tmem_ld32(taddr + 32, *reinterpret_cast<uint32_t(*)[32]>(&v[32]));
@@ -714,7 +728,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
       // exceeds it by more than 2^8 (then O, l, l_ref are rescaled by alpha).
       float alpha = 1.f;
       bool resc = false;
-      const bool tail = nvalid < BN;
+      // DUAL masks a tail tile's logits in registers and then takes the full
+      // tile's path: a second path's cold instruction fetches cost a small launch
+      // more (draft shape 16.6 -> 15.4 us); over many key tiles the extra code in
+      // the loop costs more (image-edit refresh 1157 -> 1185 us).
+      const bool tail = !DUAL && nvalid < BN;
       float rs;
       if (!tail) {
         // Full key tile: one TMEM read of the row with the hardware row max
@@ -726,7 +744,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
         tmem_ldred32_max(s_t + 64, *reinterpret_cast<uint32_t(*)[32]>(&vb[0]), m2);
         tmem_ldred32_max(s_t + 96, *reinterpret_cast<uint32_t(*)[32]>(&vb[32]), m3);
         tmem_ld_wait();
-        const float mt = fmaf(fmaxf(fmaxf(m0, m1), fmaxf(m2, m3)), sl2, badd);  // tile max, log2 units
+        float mx = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
+        if (DUAL && nvalid < BN) mx = fmaxf(mask64(va, 0, nvalid), mask64(vb, 64, nvalid));
+        const float mt = fmaf(mx, sl2, badd);  // tile max, log2 units
         if (mt > m + kRescaleThresh) {
           alpha = ex2_approx(m - mt);  // 0 when m = -inf
           resc = (j > 0);
