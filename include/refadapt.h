@@ -131,9 +131,9 @@ typedef struct {
  * K/V (and the reference query) are read from ref_fresh_k / ref_fresh_v /
  * ref_fresh_q (this step's reference projections) instead of k/v/q[RA_REF],
  * and copied into k/v/q[RA_REF] (the block's cache slot) as a by-product:
- * the first CTA of each (sample, head) bulk-stores every reference K/V tile
- * it streams through shared memory for its MMAs, each reference-row CTA its
- * own query tiles, and a_b[b] = step. Samples in REUSE or BOUNDARY read the
+ * one item of each (sample, head) bulk-stores every reference K/V tile it
+ * streams through shared memory for its MMAs, each reference-row item its own
+ * query tiles, and a_b[b] = step. Samples in REUSE or BOUNDARY read the
  * cache slot as before and leave it untouched. This replaces a separate
  * refadapt_ref_cache_update (and its reads of the fresh tensors) on the
  * attention's own pass over them.

@@ -12,12 +12,12 @@
 // in bands of GROUP_M row tiles, rows fastest inside a band (so the CTAs that
 // run at once share a few A row blocks and a few W column blocks, both held in
 // L2); CTA c takes tiles c, c + G, c + 2G, ...
-//   warp 0      TMA producer: per K step one 128 x 64 A box and one 256 x 64 W
-//               box (128-byte swizzle, rows past a segment's end read as
+//   warp 0      TMA producer: per K step one 128 x 64 A box and one W box of the
+//               tile's width x 64 (128-byte swizzle, rows past a segment's end read as
 //               zeros) into a 4-stage ring.
 //   warp 1      TMEM allocator (512 columns: two 256-column accumulators) and
-//               MMA issuer: tcgen05.mma kind::f16, M = 128, N = 256, K = 16,
-//               four per stage; commits free the stage and, after a tile's
+//               MMA issuer: tcgen05.mma kind::f16, M = 128, N = the tile's
+//               width, K = 16, four per stage; commits free the stage and, after a tile's
 //               last step, hand the accumulator to the epilogue.
 //   warps 2..9  epilogue: two warps per TMEM lane quarter (quarter = warp % 4,
 //               thread = output row = TMEM lane), which take the tile's 32-column

@@ -2,10 +2,19 @@
 // per-tile reference mass, on tcgen05 tensor cores (sm_103a).
 //
 // One CTA computes an item: a pair of 128-row Q tiles (A, B) of one role for
-// one (sample, head), or one tile where that fits the launch in one round; both
-// tiles share every K/V tile it streams. Where items are too few for the SMs,
-// or leave a small rest after whole rounds, the CTAs of a cluster share an
-// item's keys (make_plan, merge_split):
+// one (sample, head); both tiles share every K/V tile it streams. Where items
+// are too few for the SMs, or leave a small rest after whole rounds, the CTAs of
+// a cluster share an item's keys (merge_split); where items fit few rounds, an
+// item is one Q tile whose even and odd key tiles run as two streams (DUAL,
+// merge_dual). make_plan chooses and says what each form measured.
+// What bounds it: over many key tiles the shared-memory port. A key tile of a
+// pair (d = 128) is 2048 cycles of MMA and as many of shared-memory reads and
+// writes (Q 2 x 32 KB, K 2 x 32, V 2 x 32 read; K and V written), and takes 2712
+// in all; at the largest sizes the power limit follows (joint attention of 53.5k
+// keys 1650 TFLOP/s). Small launches are bound by a CTA's fixed cost (launch,
+// set-up, first loads, cold code: about 5 of the 8 us of an 8-head launch of 544
+// rows) and by the softmax latency of its key tiles.
+// The roles of a CTA's warps, for a pair:
 //   warp 0      TMA producer: Q tiles A and B once, then K and V tiles of the
 //               text, reference (cache slot) and target segments in that order
 //               into a STAGES-deep ring of 128-byte-swizzled shared buffers.
@@ -34,19 +43,21 @@
 // step's reference projections: samples in COMPUTE or FULL read reference
 // Q/K/V from them, and the producer thread copies what it streams into the
 // cache slot with TMA bulk-tensor stores from the swizzled stage buffers. The
-// first CTA of each (sample, head) stores every reference K/V tile one tile
-// after its load (the stage is refilled only once the store has read it);
-// each reference-row CTA stores its two Q tiles. Each byte of the fresh
+// first item of each (sample, head) stores every reference K/V tile one tile
+// after its load (the stage is refilled only once the store has read it; the
+// CTAs of a split item each store their own keys' tiles); each reference-row
+// item stores its Q tiles. Each byte of the fresh
 // reference rows is read from HBM once for both the MMAs and the copy.
 // Segment tails: TMA zero-fills rows past a segment's end; tail key tiles mask
 // the padded columns to -inf (probability 0) and the epilogue skips padded
-// query rows; TMA stores clip rows past a segment's end. Every mbarrier wait is bounded (WaitCtl); on a timeout the CTA
-// drains its own TMA and MMA work, frees TMEM, flags the caller's error word
-// and returns.
+// query rows; TMA stores clip rows past a segment's end. Every mbarrier wait is
+// bounded (WaitCtl); on a timeout the CTA drains its own TMA and MMA work, frees
+// TMEM, flags the caller's error word and returns.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <cfloat>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -64,7 +75,7 @@ constexpr int NUM_THREADS = 384;
 constexpr int MAX_SPLIT = 4;     // CTAs of a cluster that share one item's keys
 constexpr int MAX_SAMPLES = 32;  // samples per launch (one lane each)
 constexpr float kLog2e = 1.4426950408889634f;
-constexpr float kLowestMax = -1e30f;
+constexpr float kLowestMax = -FLT_MAX;
 constexpr float kRescaleThresh = 8.0f;  // log2 units: p <= 2^8 between rescales
 
 // DUAL: one Q tile and a deeper ring for two streams of key tiles.
@@ -710,8 +721,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
     const bool active = (t == 0) || second;
     const float sl2 = p.scale_log2;
     const float bias_l2 = (role == 2 && p.bias) ? __ldg(p.bias + h) * kLog2e : 0.f;
-    // A range of a split item may hold masked keys alone (a reference bias of
-    // -inf): a finite start keeps their probabilities 0.
+    // A rank's or a stream's keys may all be masked (a reference bias of -inf):
+    // the lowest finite start keeps their probabilities 0.
     float m = KIND != KIND_PAIR ? kLowestMax : -INFINITY, l = 0.f, lref = 0.f;
     bool ok = active;
     // DUAL: this warpgroup's key tiles are t, t + 2, ...
@@ -730,7 +741,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
       bool resc = false;
       // DUAL masks a tail tile's logits in registers and then takes the full
       // tile's path: a second path's cold instruction fetches cost a small launch
-      // more (draft shape 16.6 -> 15.4 us); over many key tiles the extra code in
+      // more (draft shape 16.6 -> 15.5 us); over many key tiles the extra code in
       // the loop costs more (image-edit refresh 1157 -> 1185 us).
       const bool tail = !DUAL && nvalid < BN;
       float rs;
@@ -990,8 +1001,8 @@ Live live_items(const Params& p, int group, int nb) {
 //   rounds, rest split    312 items of 26 key tiles (two rounds of 152 and 8)
 //                         112 us, 131 in three rounds;
 //   one tile, two streams items that fit few rounds: 8 heads, d = 64, of
-//                         32 + 256 + 256 rows 8.5 against 11.4 us, of 77 + 1000
-//                         + 500 rows 16.5 against 22.9 (half the latency per
+//                         32 + 256 + 256 rows 8.2 against 11.4 us, of 77 + 1000
+//                         + 500 rows 15.7 against 22.9 (half the latency per
 //                         key, but twice the K and V traffic per product: 55
 //                         against 46 us where it takes a second round).
 // Modes are on the device, so a call with modes is weighed with all its
