@@ -7,7 +7,9 @@
 //
 // Two kernels: CTA pairs on 256-row output tiles (gemm_pair_kernel, below) and
 // one CTA per SM on 128-row tiles (gemm_kernel), both persistent, tiles up to
-// 256 columns wide; make_plan() picks the kernel and the width. Live tiles
+// 256 columns wide. Calls of few tiles and a long K go to a third form, where
+// the CTAs of a cluster share a 128-row tile's K (gemm_kernel, SPLIT). make_plan()
+// picks the form and the width. Live tiles
 // (those the modes do not skip) are numbered segment-major, then sample, then
 // in bands of GROUP_M row tiles, rows fastest inside a band (so the CTAs that
 // run at once share a few A row blocks and a few W column blocks, both held in
@@ -61,7 +63,7 @@ constexpr int A_BYTES = BM * BK * 2;
 constexpr int B_BYTES = BN * BK * 2;
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr int OFF_BAR = STAGES * STAGE_BYTES;
-constexpr int NUM_BARS = 2 * STAGES + 2 + 2 + 1;  // full, empty, tfull[2], tempty[2], drain
+constexpr int NUM_BARS = 2 * STAGES + 2 + 2 + 1 + 1;  // full, empty, tfull[2], tempty[2], drain, parts_full
 constexpr int OFF_MISC = OFF_BAR + NUM_BARS * 8;
 constexpr int EPI_WARPS = 8;
 constexpr int EPI_STAGE_BYTES = 32 * 64;                  // 32 rows x 32 bf16 (or 16 fp32) of one warp
@@ -71,7 +73,10 @@ constexpr int SMEM_BYTES = OFF_EPI + EPI_WARPS * EPI_WARP_BYTES;
 constexpr int SMEM_ALLOC = SMEM_BYTES + 1024;
 constexpr int THREADS = 64 + 32 * EPI_WARPS;
 constexpr int TMEM_COLS = 512;
+constexpr int MAX_SPLIT = 4;  // CTAs of a cluster that share one tile's K
 static_assert(SMEM_ALLOC <= 232448, "shared memory budget");
+// split tiles: the parts to send and those received take the place of the stages
+static_assert(2 * (MAX_SPLIT - 1) * (BM * BN * 4 / MAX_SPLIT) <= OFF_BAR, "parts fit the stages");
 
 // CTA-pair kernel: 256-row output tiles; each CTA stages its 128 rows of A
 // and its half of the W tile (up to 128 columns), 128 of K per stage (two 128-byte
@@ -237,9 +242,9 @@ __device__ __forceinline__ void rows_store(uint8_t* stage, const float (&x)[32],
 // What an epilogue warp works on: its 32 rows (row0 + lane, nrow of them in
 // the segment), its share of the tile's columns (half 0 or 1), its shared
 // memory (staging buffer, two vectors of 128 per-column values) and the TMEM
-// address of its lanes in the tile's accumulator.
+// address of its lanes in the tile's accumulator; cols: columns of the tile.
 struct EpiWarp {
-  int row0, nrow, half;
+  int row0, nrow, half, cols;
   uint8_t* stage;
   float* vec0;
   float* vec1;
@@ -265,7 +270,7 @@ __device__ __forceinline__ bool epilogue_linear(const Params& p, const Tile& tl,
   const Seg& sg = p.seg[tl.seg];
   const int lane = threadIdx.x & 31, n0 = tl.n0 + 32 * w.half;
   // this warp's; the last tile of a row may reach past N (a multiple of 32)
-  const int chunks = (min(p.bn, p.N - tl.n0) / 32 + 1 - w.half) >> 1;
+  const int chunks = (min(w.cols, p.N - tl.n0) / 32 + 1 - w.half) >> 1;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     if (j >= chunks) break;
@@ -422,7 +427,80 @@ __device__ __forceinline__ bool epilogue_tile(const Params& p, const Tile& tl, c
     return epilogue_linear<EPI>(p, tl, w, ready);
 }
 
-template <int EPI, int D>
+// A split tile: each CTA of the cluster has the sums over its part of K in its
+// own TMEM; afterwards rank r has columns [r, r + 1) * bn / cs of the whole sums
+// there. Each rank hands every other rank that one's columns, in fp32, by a bulk
+// copy between the CTAs' shared memory (the stages are idle by then), and adds
+// its own columns up in rank order. Every thread of the cluster takes part in
+// the cluster barrier: before it every rank's stages are idle and its parts are
+// written, after it they are copied. ok: this warp's accumulator is complete.
+// The merge of a 128 x 256 tile between two CTAs (64 KB each way) takes 2.6 us.
+__device__ __forceinline__ bool merge_parts(const WaitCtl& ctl, uint8_t* smem, uint64_t* parts_full, uint32_t acc,
+                                            bool ok, int bn, int half, int quarter, int rank, int cs) {
+  const int lane = threadIdx.x & 31, row = quarter * 32 + lane;
+  const int cw = bn / cs;                            // columns per rank
+  const uint32_t part_bytes = uint32_t(BM) * cw * 4;  // [column / 4][row] of 16 bytes
+  uint8_t* send = smem;                              // parts for the other ranks, in rank order
+  uint8_t* recv = smem + (cs - 1) * part_bytes;      // parts from the other ranks, in rank order
+  const bool leader = quarter == 0 && half == 0 && lane == 0;
+  if (leader) mbar_arrive_expect_tx(parts_full, (cs - 1) * part_bytes);
+  if (ok) {
+#pragma unroll 1
+    for (int c0 = 32 * half; c0 < bn; c0 += 64) {
+      const int q = c0 / cw;
+      if (q == rank) continue;
+      uint32_t v[32];
+      tmem_ld32(acc + c0, v);
+      tmem_ld_wait_for(v);
+      uint4* dst = reinterpret_cast<uint4*>(send + (q - (q > rank ? 1 : 0)) * part_bytes) +
+                   ((c0 - q * cw) >> 2) * BM + row;
+#pragma unroll
+      for (int i = 0; i < 32; i += 4) dst[(i >> 2) * BM] = make_uint4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+    }
+  }
+  fence_proxy_async_smem();  // the parts are next read by bulk copies
+  cluster_sync_all();
+  if (leader && !*ctl.abort_flag)
+    for (int q = 0; q < cs; ++q)
+      if (q != rank)
+        bulk_copy_to_cta(mapa_shared(smem_u32(recv + (rank - (rank > q ? 1 : 0)) * part_bytes), q),
+                         send + (q - (q > rank ? 1 : 0)) * part_bytes, part_bytes,
+                         mapa_shared(smem_u32(parts_full), q));
+  if (!__all_sync(0xffffffffu, mbar_wait(parts_full, 0, ctl)) || !ok) return false;
+#pragma unroll 1
+  for (int c0 = 32 * half; c0 < cw; c0 += 64) {
+    uint32_t v[32];
+    float x[32];
+    tmem_ld32(acc + rank * cw + c0, v);
+    tmem_ld_wait_for(v);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) x[i] = 0.f;
+#pragma unroll 1
+    for (int r = 0; r < cs; ++r) {
+      const float4* src = reinterpret_cast<const float4*>(recv + (r - (r > rank ? 1 : 0)) * part_bytes) +
+                          (c0 >> 2) * BM + row;
+#pragma unroll
+      for (int i = 0; i < 32; i += 4) {
+        const float4 y = r == rank ? make_float4(__uint_as_float(v[i]), __uint_as_float(v[i + 1]),
+                                                 __uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]))
+                                   : src[(i >> 2) * BM];
+        x[i] += y.x;
+        x[i + 1] += y.y;
+        x[i + 2] += y.z;
+        x[i + 3] += y.w;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(x[i]);
+    tmem_st32(acc + rank * cw + c0, v);
+  }
+  tmem_st_wait();
+  return true;
+}
+
+// SPLIT: a cluster takes one tile, each rank a contiguous part of its K
+// (merge_parts adds them up), then its share of the columns in the epilogue.
+template <int EPI, int D, bool SPLIT = false>
 __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant__ Params p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -432,9 +510,14 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
   uint64_t* tfull = bars + 2 * STAGES;
   uint64_t* tempty = bars + 2 * STAGES + 2;
   uint64_t* drain = bars + 2 * STAGES + 4;
+  uint64_t* parts_full = bars + 2 * STAGES + 5;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + OFF_MISC);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + OFF_MISC + 4);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = SPLIT ? int(cluster_rank()) : 0, cs = SPLIT ? int(cluster_size()) : 1;
+  const int64_t t0 = SPLIT ? blockIdx.x / cs : blockIdx.x, step = SPLIT ? gridDim.x / cs : gridDim.x;
+  const int kb0 = SPLIT ? p.kblocks * rank / cs : 0;  // this CTA's K steps
+  const int kb1 = SPLIT ? p.kblocks * (rank + 1) / cs : p.kblocks;
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(full + s, 1);
@@ -445,12 +528,14 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
       mbar_init(tempty + b, EPI_WARPS);
     }
     mbar_init(drain, 1);
+    mbar_init(parts_full, 1);
     *abort_flag = 0;
     fence_mbar_init();
   }
   if (warp == 1) tmem_alloc(tmem_slot, TMEM_COLS);
   tc_fence_before();
   __syncthreads();
+  if (SPLIT) cluster_sync_all();  // every CTA's barriers exist
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const WaitCtl ctl{abort_flag, p.err_word, p.budget_ns};
@@ -470,8 +555,8 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
       bool ok = true;
       Walk<BM, EPI> walk;
       Tile tl;
-      for (int64_t t = blockIdx.x; ok && walk.at(p, t, tl); t += gridDim.x) {
-        for (int kb = 0; kb < p.kblocks; ++kb, ++it) {
+      for (int64_t t = t0; ok && walk.at(p, t, tl); t += step) {
+        for (int kb = kb0; kb < kb1; ++kb, ++it) {
           const int st = int(it % STAGES);
           if (it >= STAGES && !(ok = mbar_wait(empty + st, uint32_t((it / STAGES - 1) & 1), ctl))) break;
           uint8_t* sa = smem + st * STAGE_BYTES;
@@ -497,12 +582,12 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
       bool ok = true, issued = false;
       Walk<BM, EPI> walk;
       Tile tl;
-      for (int64_t t = blockIdx.x; ok && walk.at(p, t, tl); t += gridDim.x) {
+      for (int64_t t = t0; ok && walk.at(p, t, tl); t += step) {
         const int buf = i & 1, use = i >> 1;
         if (use > 0 && !(ok = mbar_wait(tempty + buf, uint32_t((use - 1) & 1), ctl))) break;
         tc_fence_after();
         const uint32_t d_t = tmem + uint32_t(buf * BN);
-        for (int kb = 0; kb < p.kblocks; ++kb, ++it) {
+        for (int kb = kb0; kb < kb1; ++kb, ++it) {
           const int st = int(it % STAGES);
           if (!(ok = mbar_wait(full + st, uint32_t((it / STAGES) & 1), ctl))) break;
           tc_fence_after();
@@ -510,7 +595,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
 #pragma unroll
           for (int kk = 0; kk < BK / 16; ++kk)
             umma_ss(d_t, sdesc_sw128(sa + kk * 32, 16, 1024), sdesc_sw128(sb + kk * 32, 16, 1024), idesc,
-                    (kb > 0 || kk > 0) ? 1u : 0u);
+                    (kb > kb0 || kk > 0) ? 1u : 0u);
           umma_commit(empty + st);
           issued = true;
         }
@@ -534,14 +619,22 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
     int i = 0;
     Walk<BM, EPI> walk;
     Tile tl;
-    for (int64_t t = blockIdx.x; walk.at(p, t, tl); t += gridDim.x) {
+    for (int64_t t = t0; walk.at(p, t, tl); t += step) {
       const int buf = i & 1, use = i >> 1;
       w.row0 = tl.m0 + quarter * 32;
       w.nrow = min(32, p.rows[tl.seg] - w.row0);
       w.acc = tmem + (uint32_t(quarter * 32) << 16) + uint32_t(buf * BN);
+      w.cols = p.bn;
+      const uint32_t acc = w.acc;
+      if (SPLIT) {
+        w.cols /= cs;
+        w.acc += uint32_t(rank * w.cols);
+        tl.n0 += rank * w.cols;
+      }
       if (!epilogue_tile<EPI, D>(p, tl, w, [&] {
-            const bool ok = __all_sync(0xffffffffu, mbar_wait(tfull + buf, uint32_t(use & 1), ctl));
+            bool ok = __all_sync(0xffffffffu, mbar_wait(tfull + buf, uint32_t(use & 1), ctl));
             tc_fence_after();
+            if (SPLIT) ok = merge_parts(ctl, smem, parts_full, acc, ok, p.bn, w.half, quarter, rank, cs);
             return ok;
           }))
         break;
@@ -550,6 +643,15 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
       if (lane == 0) mbar_arrive(tempty + buf);
       ++i;
     }
+  }
+  if (SPLIT) {
+    // Warps 0 and 1 meet the epilogue's cluster barrier here. No CTA exits before
+    // every part has been read from it and received.
+    Walk<BM, EPI> walk;
+    Tile tl;
+    __syncwarp();
+    if (warp < 2 && walk.at(p, t0, tl)) cluster_sync_all();
+    cluster_sync_all();
   }
   tc_fence_before();
   __syncthreads();
@@ -706,6 +808,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_pair_kernel(const __grid_cons
     for (int64_t t = cid; walk.at(p, t, tl); t += ncl) {
       const int buf = i & 1, use = i >> 1;
       w.row0 = tl.m0 + int(rank) * 128 + quarter * 32;
+      w.cols = p.bn;
       w.nrow = min(32, p.rows[tl.seg] - w.row0);
       w.acc = tmem + (uint32_t(quarter * 32) << 16) + uint32_t(buf * BN);
       if (!epilogue_tile<EPI, D>(p, tl, w, [&] {
@@ -748,26 +851,63 @@ __global__ void rope_table_kernel(float* table, int32_t n_pos, int32_t d, double
 // The kernels by epilogue (QKV: by head dim too), one CTA per tile and CTA pairs.
 using Kernel = void (*)(Params);
 struct Kernels {
-  Kernel single, pair;
+  Kernel single, pair, split;  // split: STORE, GELU and RESID
 };
 Kernels pick(int epi, int d) {
   switch (epi) {
-    case RA_EPI_STORE: return {gemm_kernel<RA_EPI_STORE, 0>, gemm_pair_kernel<RA_EPI_STORE, 0>};
-    case RA_EPI_GELU: return {gemm_kernel<RA_EPI_GELU, 0>, gemm_pair_kernel<RA_EPI_GELU, 0>};
-    case RA_EPI_RESID: return {gemm_kernel<RA_EPI_RESID, 0>, gemm_pair_kernel<RA_EPI_RESID, 0>};
+    case RA_EPI_STORE: return {gemm_kernel<RA_EPI_STORE, 0>, gemm_pair_kernel<RA_EPI_STORE, 0>, gemm_kernel<RA_EPI_STORE, 0, true>};
+    case RA_EPI_GELU: return {gemm_kernel<RA_EPI_GELU, 0>, gemm_pair_kernel<RA_EPI_GELU, 0>, gemm_kernel<RA_EPI_GELU, 0, true>};
+    case RA_EPI_RESID: return {gemm_kernel<RA_EPI_RESID, 0>, gemm_pair_kernel<RA_EPI_RESID, 0>, gemm_kernel<RA_EPI_RESID, 0, true>};
     default:
-      return d == 128 ? Kernels{gemm_kernel<RA_EPI_QKV, 128>, gemm_pair_kernel<RA_EPI_QKV, 128>}
-                      : Kernels{gemm_kernel<RA_EPI_QKV, 64>, gemm_pair_kernel<RA_EPI_QKV, 64>};
+      return d == 128 ? Kernels{gemm_kernel<RA_EPI_QKV, 128>, gemm_pair_kernel<RA_EPI_QKV, 128>, nullptr}
+                      : Kernels{gemm_kernel<RA_EPI_QKV, 64>, gemm_pair_kernel<RA_EPI_QKV, 64>, nullptr};
   }
 }
 
 bool aligned16(const void* ptr) { return (reinterpret_cast<uintptr_t>(ptr) & 15u) == 0; }
 
-// How a call is cut into tiles: CTA pairs or single CTAs, and tile columns.
+// How a call is cut into tiles: CTA pairs or single CTAs, tile columns, and the
+// CTAs of a cluster that share a tile's K (1: a CTA has a tile of its own).
 struct Plan {
   bool pair;
-  int bn;
+  int bn, cs;
 };
+
+// Clusters of cs CTAs of a split kernel that can run at once on the current
+// device (they live inside one GPC, so the floorplan decides; every split kernel
+// has the same launch shape); cached per device. 0: none, or the query failed,
+// and nothing is split.
+int max_clusters(Kernel fn, int cs) {
+  static std::mutex mu;
+  static int cache[64][MAX_SPLIT + 1];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+    cudaGetLastError();
+    return 0;
+  }
+  std::lock_guard<std::mutex> lk(mu);
+  int& n = cache[dev][cs];
+  if (n > 0) return n;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cs;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg;
+  std::memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(cs, 1, 1);
+  cfg.blockDim = dim3(THREADS, 1, 1);
+  cfg.dynamicSmemBytes = SMEM_ALLOC;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int found = 0;
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_ALLOC) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&found, fn, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n = found;
+}
 
 // The cheapest cut by a model of the two kernels' time (microseconds), fitted to
 // single waves of 256 to 64 columns at K = 1024 and 4096 on a GB300 (each within
@@ -778,22 +918,33 @@ struct Plan {
 // pays only where it saves a round: 13 row tiles of 256 by N = 3072 make 156
 // tiles of 256 columns (three rounds of 76 pairs, the last one nearly empty;
 // 188 us at K = 12288) or 208 of 192 columns (three shorter rounds, 164 us).
+// Few tiles of a long K leave SMs idle (a small model's MLP output, 377 rows by
+// N = 1024, K = 4096, is 64 narrow tiles, 19.2 us): there two or four CTAs of a
+// cluster share a tile's K, which costs a merge and pays from about K = 3072 up
+// while the clusters fit the GPU at once (12.2 us in clusters of four on tiles of
+// 128 columns; 516 rows, K = 12288, N = 3072 58.9 -> 50.3 in clusters of two;
+// at K = 1024 it loses, 7.3 -> 8.2). Not for QKV, whose epilogue needs whole heads,
+// nor where the caller chose the tiles.
 // Calls with gated segments are weighed with and without them.
 Plan make_plan(const ra_gemm_args& a, int sms) {
-  Plan best{false, 256};
+  Plan best{false, 256, 1};
   double best_us = 1e30;
+  auto tiles_of = [&](int tm, int bn, int64_t* all, int64_t* open) {
+    const int64_t cols = (a.N + bn - 1) / bn;
+    *all = *open = 0;  // tiles, and those of segments that are not gated
+    for (int g = 0; g < a.n_seg; ++g) {
+      const int64_t t = a.seg[g].rows > 0 ? int64_t(a.B) * ((a.seg[g].rows + tm - 1) / tm) * cols : 0;
+      *all += t;
+      if (!a.seg[g].gated) *open += t;
+    }
+  };
   for (int pair = 0; pair < 2; ++pair) {
     if ((a.tile_mode == 1 && pair) || (a.tile_mode == 2 && !pair) || (pair && sms < 2)) continue;
     const int tm = pair ? P_TM : BM, slots = pair ? sms / 2 : sms;
     for (int bn = 256; bn >= 64; bn -= 32) {
       if (a.epilogue == RA_EPI_QKV && (bn % a.d != 0 || (a.H * a.d) % bn != 0)) continue;
-      const int64_t cols = (a.N + bn - 1) / bn;
-      int64_t all = 0, open = 0;  // tiles, and those of segments that are not gated
-      for (int g = 0; g < a.n_seg; ++g) {
-        const int64_t t = a.seg[g].rows > 0 ? int64_t(a.B) * ((a.seg[g].rows + tm - 1) / tm) * cols : 0;
-        all += t;
-        if (!a.seg[g].gated) open += t;
-      }
+      int64_t all, open;
+      tiles_of(tm, bn, &all, &open);
       const double epilogue = 0.0085 * bn;  // of a tile, hidden behind the next one's MMAs
       double round = a.K / 1024.0 * (pair ? 3.11 + 0.00766 * bn : 3.4 + 0.0127 * bn);
       round = round > epilogue ? round : epilogue;
@@ -802,7 +953,24 @@ Plan make_plan(const ra_gemm_args& a, int sms) {
       if (open > 0 && open < all) us += fixed + round * double((open + slots - 1) / slots);
       if (us < best_us) {
         best_us = us;
-        best = Plan{pair != 0, bn};
+        best = Plan{pair != 0, bn, 1};
+      }
+    }
+  }
+  if (a.epilogue == RA_EPI_QKV || a.tile_mode != 0) return best;
+  for (int cs = 2; cs <= MAX_SPLIT; cs *= 2) {
+    if (a.K / BK < 4 * cs) break;
+    const int clusters = max_clusters(pick(a.epilogue, a.d).split, cs);
+    if (clusters == 0) continue;
+    for (int bn = 256; bn >= 32 * cs; bn /= 2) {
+      int64_t all, open;
+      tiles_of(BM, bn, &all, &open);
+      const double wave = 3.6 + 4.0 + a.K / 1024.0 / cs * (3.4 + 0.0127 * bn);
+      double us = wave * double((all + clusters - 1) / clusters);
+      if (open > 0 && open < all) us += wave * double((open + clusters - 1) / clusters);
+      if (us < 0.97 * best_us) {
+        best_us = us;
+        best = Plan{false, bn, cs};
       }
     }
   }
@@ -968,8 +1136,9 @@ extern "C" ra_status refadapt_gemm(const ra_gemm_args* a, void* stream) {
   }
   if (tiles == 0) return RA_OK;
   const Kernels kn = pick(a->epilogue, a->d);
-  const ra_status as = ensure_dynamic_smem(reinterpret_cast<const void*>(pair ? kn.pair : kn.single),
-                                           pair ? P_SMEM_ALLOC : SMEM_ALLOC, "refadapt_gemm");
+  const Kernel fn = pair ? kn.pair : plan.cs > 1 ? kn.split : kn.single;
+  const ra_status as =
+      ensure_dynamic_smem(reinterpret_cast<const void*>(fn), pair ? P_SMEM_ALLOC : SMEM_ALLOC, "refadapt_gemm");
   if (as != RA_OK) return as;
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaLaunchConfig_t cfg;
@@ -980,14 +1149,17 @@ extern "C" ra_status refadapt_gemm(const ra_gemm_args* a, void* stream) {
   cudaLaunchAttribute attr[2];
   attr[0] = pdl_attribute();
   attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = 2;
+  attr[1].val.clusterDim.x = pair ? 2 : plan.cs;
   attr[1].val.clusterDim.y = 1;
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = pair ? 2 : 1;
+  cfg.numAttrs = pair || plan.cs > 1 ? 2 : 1;
   const int64_t slots = pair ? (sms / 2 > 0 ? sms / 2 : 1) : sms;
-  cfg.gridDim = dim3(unsigned((tiles < slots ? tiles : slots) * (pair ? 2 : 1)), 1, 1);
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, pair ? kn.pair : kn.single, p);
+  if (plan.cs > 1)
+    cfg.gridDim = dim3(unsigned(tiles * plan.cs), 1, 1);
+  else
+    cfg.gridDim = dim3(unsigned((tiles < slots ? tiles : slots) * (pair ? 2 : 1)), 1, 1);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, fn, p);
   if (e != cudaSuccess) {
     set_error("refadapt_gemm: launch failed: %s", cudaGetErrorString(e));
     cudaGetLastError();

@@ -364,6 +364,9 @@ __device__ __forceinline__ void bulk_copy_to_cta(uint32_t dst_cluster_addr, cons
                "r"(smem_u32(src)), "r"(bytes), "r"(bar_cluster_addr)
                : "memory");
 }
+// Orders this thread's shared-memory accesses, and the TMA loads it has waited
+// for, before bulk copies and TMA stores that read the same bytes.
+__device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 // Arrive (release, cluster scope) on an mbarrier in another CTA of the cluster.
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");

@@ -193,6 +193,18 @@ def test_gemm_tile_widths_match_oracle(cuda_ok, epi, tile_mode, N):
                tile_mode=tile_mode)
 
 
+# Calls of few tiles and a long K, whose tiles are shared by the CTAs of a cluster: one row, ragged
+# rows, K steps that do not divide by the CTAs, tiles of 64 to 256 columns, a gated segment.
+@pytest.mark.parametrize("epi", [0, 1, 2])
+@pytest.mark.parametrize("B,K,N,rows", [(1, 4160, 256, [1]), (1, 4160, 256, [1, 129, 77]), (2, 4096, 1024, [77, 300]),
+                                        (2, 4160, 1024, [77, 500, 300]), (1, 12352, 768, [130, 257]),
+                                        (1, 16384, 512, [640])])
+def test_gemm_split_k_matches_oracle(cuda_ok, epi, B, K, N, rows):
+    gated = [i == 1 for i in range(len(rows))]
+    _gemm_case(B, K, N, rows, epi, torch.Generator().manual_seed(K + N), gated=gated, modes=[REUSE, COMPUTE][:B],
+               inplace=epi == 2)
+
+
 @pytest.mark.parametrize("tile_mode", TILE_MODES)
 @pytest.mark.parametrize("H,d,modes", [(4, 64, [FULL, BOUNDARY]), (2, 128, [REUSE, COMPUTE])])
 def test_gemm_qkv_epilogue_matches_oracle(cuda_ok, H, d, modes, tile_mode):
