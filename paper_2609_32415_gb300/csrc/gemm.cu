@@ -117,6 +117,7 @@ struct Seg {
 struct Params {
   int32_t n_seg, B, N, C, kblocks;
   int32_t bn;                // columns of a tile
+  int32_t slots, rest_max;   // rest_max > 0: whole rounds of `slots` pair tiles, a rest of up to rest_max split
   int32_t cols, cols_q;      // column tiles of N; of the query part (QKV)
   int32_t rows[3], m_tiles[3], gated[3];
   int32_t K;
@@ -180,6 +181,32 @@ struct Walk {
     return true;
   }
 };
+
+// The tiles of a call's whole rounds; those past them, if at most p.rest_max, are
+// its rest. Every tile where the call has no rest.
+template <int TM, int EPI>
+__device__ __forceinline__ int64_t round_tiles(const Params& p) {
+  if (p.rest_max == 0) return INT64_MAX;
+  Walk<TM, EPI> w;
+  int64_t live = 0;
+  for (w.g = 0; w.g < p.n_seg; ++w.g)
+    for (w.s = 0; w.s < p.B; ++w.s) live += int64_t(p.m_tiles[w.g]) * w.piece_cols(p);
+  const int64_t rest = live % p.slots;
+  return rest <= p.rest_max ? live - rest : live;
+}
+
+// The tile of item t of a launch. SPLIT: where the call has a rest, a quarter
+// (128 rows by REST_BN columns) of a pair tile of it; p.m_tiles and p.bn are the
+// pair kernel's then.
+constexpr int REST_BN = 128;
+template <int EPI, bool SPLIT>
+__device__ __forceinline__ bool tile_at(const Params& p, Walk<BM, EPI>& walk, int64_t t, Tile& tl) {
+  if (!SPLIT || p.rest_max == 0) return walk.at(p, t, tl);
+  if (!walk.at(p, round_tiles<P_TM, EPI>(p) + (t >> 2), tl)) return false;
+  tl.m0 = 2 * tl.m0 + (t & 1 ? BM : 0);
+  tl.n0 += t & 2 ? REST_BN : 0;
+  return tl.m0 < p.rows[tl.seg];
+}
 
 // GELU, tanh form, of two values through the identity
 // 0.5 x (1 + tanh(u)) = x / (1 + e^(-2u)), u = sqrt(2/pi) (x + 0.044715 x^3),
@@ -518,6 +545,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
   const int64_t t0 = SPLIT ? blockIdx.x / cs : blockIdx.x, step = SPLIT ? gridDim.x / cs : gridDim.x;
   const int kb0 = SPLIT ? p.kblocks * rank / cs : 0;  // this CTA's K steps
   const int kb1 = SPLIT ? p.kblocks * (rank + 1) / cs : p.kblocks;
+  const int bn = SPLIT && p.rest_max > 0 ? REST_BN : p.bn;
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(full + s, 1);
@@ -555,12 +583,12 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
       bool ok = true;
       Walk<BM, EPI> walk;
       Tile tl;
-      for (int64_t t = t0; ok && walk.at(p, t, tl); t += step) {
+      for (int64_t t = t0; ok && tile_at<EPI, SPLIT>(p, walk, t, tl); t += step) {
         for (int kb = kb0; kb < kb1; ++kb, ++it) {
           const int st = int(it % STAGES);
           if (it >= STAGES && !(ok = mbar_wait(empty + st, uint32_t((it / STAGES - 1) & 1), ctl))) break;
           uint8_t* sa = smem + st * STAGE_BYTES;
-          mbar_arrive_expect_tx(full + st, A_BYTES + p.bn * BK * 2);
+          mbar_arrive_expect_tx(full + st, A_BYTES + bn * BK * 2);
           tma_load_4d(sa, &p.tm_a[tl.seg], full + st, kb * BK, tl.m0, 0, tl.s);
           tma_load_4d(sa + A_BYTES, &p.tm_w[tl.seg], full + st, kb * BK, tl.n0, 0, 0);
         }
@@ -575,14 +603,14 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
   } else if (warp == 1) {
     if (lane == 0) {
       // -------------------------------------------------------------- MMA issuer
-      const uint32_t idesc = idesc_bf16_f32(BM, p.bn, 0, 0);
+      const uint32_t idesc = idesc_bf16_f32(BM, bn, 0, 0);
       const uint32_t s0 = smem_u32(smem);
       int64_t it = 0;
       int i = 0;
       bool ok = true, issued = false;
       Walk<BM, EPI> walk;
       Tile tl;
-      for (int64_t t = t0; ok && walk.at(p, t, tl); t += step) {
+      for (int64_t t = t0; ok && tile_at<EPI, SPLIT>(p, walk, t, tl); t += step) {
         const int buf = i & 1, use = i >> 1;
         if (use > 0 && !(ok = mbar_wait(tempty + buf, uint32_t((use - 1) & 1), ctl))) break;
         tc_fence_after();
@@ -619,12 +647,12 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
     int i = 0;
     Walk<BM, EPI> walk;
     Tile tl;
-    for (int64_t t = t0; walk.at(p, t, tl); t += step) {
+    for (int64_t t = t0; tile_at<EPI, SPLIT>(p, walk, t, tl); t += step) {
       const int buf = i & 1, use = i >> 1;
       w.row0 = tl.m0 + quarter * 32;
       w.nrow = min(32, p.rows[tl.seg] - w.row0);
       w.acc = tmem + (uint32_t(quarter * 32) << 16) + uint32_t(buf * BN);
-      w.cols = p.bn;
+      w.cols = bn;
       const uint32_t acc = w.acc;
       if (SPLIT) {
         w.cols /= cs;
@@ -634,7 +662,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
       if (!epilogue_tile<EPI, D>(p, tl, w, [&] {
             bool ok = __all_sync(0xffffffffu, mbar_wait(tfull + buf, uint32_t(use & 1), ctl));
             tc_fence_after();
-            if (SPLIT) ok = merge_parts(ctl, smem, parts_full, acc, ok, p.bn, w.half, quarter, rank, cs);
+            if (SPLIT) ok = merge_parts(ctl, smem, parts_full, acc, ok, bn, w.half, quarter, rank, cs);
             return ok;
           }))
         break;
@@ -650,7 +678,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
     Walk<BM, EPI> walk;
     Tile tl;
     __syncwarp();
-    if (warp < 2 && walk.at(p, t0, tl)) cluster_sync_all();
+    if (warp < 2 && tile_at<EPI, SPLIT>(p, walk, t0, tl)) cluster_sync_all();
     cluster_sync_all();
   }
   tc_fence_before();
@@ -723,7 +751,8 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_pair_kernel(const __grid_cons
       bool ok = true;
       Walk<P_TM, EPI> walk;
       Tile tl;
-      for (int64_t t = cid; ok && walk.at(p, t, tl); t += ncl) {
+      const int64_t end = round_tiles<P_TM, EPI>(p);
+      for (int64_t t = cid; ok && t < end && walk.at(p, t, tl); t += ncl) {
         for (int kb = 0; kb < (p.kblocks + 1) / 2; ++kb, ++it) {
           const int st = int(it % P_STAGES);
           if (it >= P_STAGES && !(ok = mbar_wait(empty + st, uint32_t((it / P_STAGES - 1) & 1), ctl))) break;
@@ -763,7 +792,8 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_pair_kernel(const __grid_cons
       bool ok = true, issued = false;
       Walk<P_TM, EPI> walk;
       Tile tl;
-      for (int64_t t = cid; ok && walk.at(p, t, tl); t += ncl) {
+      const int64_t end = round_tiles<P_TM, EPI>(p);
+      for (int64_t t = cid; ok && t < end && walk.at(p, t, tl); t += ncl) {
         const int buf = i & 1, use = i >> 1;
         if (use > 0 && !(ok = mbar_wait_cluster(tempty + buf, uint32_t((use - 1) & 1), ctl))) break;
         tc_fence_after();
@@ -805,7 +835,8 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_pair_kernel(const __grid_cons
     int i = 0;
     Walk<P_TM, EPI> walk;
     Tile tl;
-    for (int64_t t = cid; walk.at(p, t, tl); t += ncl) {
+    const int64_t end = round_tiles<P_TM, EPI>(p);
+    for (int64_t t = cid; t < end && walk.at(p, t, tl); t += ncl) {
       const int buf = i & 1, use = i >> 1;
       w.row0 = tl.m0 + int(rank) * 128 + quarter * 32;
       w.cols = p.bn;
@@ -866,11 +897,40 @@ Kernels pick(int epi, int d) {
 
 bool aligned16(const void* ptr) { return (reinterpret_cast<uintptr_t>(ptr) & 15u) == 0; }
 
+// Launches `ctas` CTAs in clusters of cs.
+ra_status launch(const Params& p, Kernel fn, int smem, int64_t ctas, int cs, cudaStream_t st) {
+  const ra_status as = ensure_dynamic_smem(reinterpret_cast<const void*>(fn), smem, "refadapt_gemm");
+  if (as != RA_OK) return as;
+  cudaLaunchAttribute attr[2];
+  attr[0] = pdl_attribute();
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cs;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg;
+  std::memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = dim3(unsigned(ctas), 1, 1);
+  cfg.blockDim = dim3(THREADS, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = cs > 1 ? 2 : 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, fn, p);
+  if (e != cudaSuccess) {
+    set_error("refadapt_gemm: launch failed: %s", cudaGetErrorString(e));
+    cudaGetLastError();
+    return RA_ECUDA;
+  }
+  return launch_status("refadapt_gemm");
+}
+
 // How a call is cut into tiles: CTA pairs or single CTAs, tile columns, and the
 // CTAs of a cluster that share a tile's K (1: a CTA has a tile of its own).
+// rest_max > 0: pair tiles of 256 columns in whole rounds, and a rest of at most
+// this many split, each into four tiles of clusters of cs CTAs, by a second launch.
 struct Plan {
   bool pair;
-  int bn, cs;
+  int bn, cs, rest_max;
 };
 
 // Clusters of cs CTAs of a split kernel that can run at once on the current
@@ -925,9 +985,14 @@ int max_clusters(Kernel fn, int cs) {
 // 128 columns; 516 rows, K = 12288, N = 3072 58.9 -> 50.3 in clusters of two;
 // at K = 1024 it loses, 7.3 -> 8.2). Not for QKV, whose epilogue needs whole heads,
 // nor where the caller chose the tiles.
+// Whole rounds of pair tiles and a small rest: the rest's tiles are cut into
+// quarters and split in the same way by a second launch, which costs 13 us and
+// its share of K, so only a long K gains (K = 12288, N = 3072: 13 row tiles, two
+// rounds and 4 tiles, 162 -> 157 us; 1572 rows, one round and 8, 105 -> 95). Its
+// 256-column tiles also suit what the modes leave better than narrow ones.
 // Calls with gated segments are weighed with and without them.
 Plan make_plan(const ra_gemm_args& a, int sms) {
-  Plan best{false, 256, 1};
+  Plan best{false, 256, 1, 0};
   double best_us = 1e30;
   auto tiles_of = [&](int tm, int bn, int64_t* all, int64_t* open) {
     const int64_t cols = (a.N + bn - 1) / bn;
@@ -953,11 +1018,12 @@ Plan make_plan(const ra_gemm_args& a, int sms) {
       if (open > 0 && open < all) us += fixed + round * double((open + slots - 1) / slots);
       if (us < best_us) {
         best_us = us;
-        best = Plan{pair != 0, bn, 1};
+        best = Plan{pair != 0, bn, 1, 0};
       }
     }
   }
   if (a.epilogue == RA_EPI_QKV || a.tile_mode != 0) return best;
+  const double merge = 4.0;
   for (int cs = 2; cs <= MAX_SPLIT; cs *= 2) {
     if (a.K / BK < 4 * cs) break;
     const int clusters = max_clusters(pick(a.epilogue, a.d).split, cs);
@@ -965,13 +1031,32 @@ Plan make_plan(const ra_gemm_args& a, int sms) {
     for (int bn = 256; bn >= 32 * cs; bn /= 2) {
       int64_t all, open;
       tiles_of(BM, bn, &all, &open);
-      const double wave = 3.6 + 4.0 + a.K / 1024.0 / cs * (3.4 + 0.0127 * bn);
+      const double wave = 3.6 + merge + a.K / 1024.0 / cs * (3.4 + 0.0127 * bn);
       double us = wave * double((all + clusters - 1) / clusters);
       if (open > 0 && open < all) us += wave * double((open + clusters - 1) / clusters);
       if (us < 0.97 * best_us) {
         best_us = us;
-        best = Plan{false, bn, cs};
+        best = Plan{false, bn, cs, 0};
       }
+    }
+    const int slots = sms / 2;
+    const double round = a.K / 1024.0 * (3.11 + 0.00766 * BN), fixed = 4.4 + 0.0088 * BN;
+    const double wave = 13.3 + a.K / 1024.0 / cs * (3.4 + 0.0127 * REST_BN);
+    int64_t all, open;
+    tiles_of(P_TM, BN, &all, &open);
+    int64_t rest_max = int64_t(round / wave) * clusters / 4;
+    if (rest_max > slots - 1) rest_max = slots - 1;
+    if (slots < 1 || rest_max < 1 || all < slots) continue;
+    auto time = [&](int64_t tiles) {
+      const int64_t rest = tiles % slots;
+      const bool split = rest <= rest_max;
+      return fixed + round * double(split ? tiles / slots : tiles / slots + 1) +
+             wave * double(split ? (4 * rest + clusters - 1) / clusters : 0);
+    };
+    const double us = time(all) + (open > 0 && open < all ? time(open) : 0.0);
+    if (us < 0.97 * best_us) {
+      best_us = us;
+      best = Plan{true, BN, cs, int(rest_max)};
     }
   }
   return best;
@@ -1136,34 +1221,18 @@ extern "C" ra_status refadapt_gemm(const ra_gemm_args* a, void* stream) {
   }
   if (tiles == 0) return RA_OK;
   const Kernels kn = pick(a->epilogue, a->d);
-  const Kernel fn = pair ? kn.pair : plan.cs > 1 ? kn.split : kn.single;
-  const ra_status as =
-      ensure_dynamic_smem(reinterpret_cast<const void*>(fn), pair ? P_SMEM_ALLOC : SMEM_ALLOC, "refadapt_gemm");
-  if (as != RA_OK) return as;
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
-  cudaLaunchConfig_t cfg;
-  std::memset(&cfg, 0, sizeof(cfg));
-  cfg.blockDim = dim3(THREADS, 1, 1);
-  cfg.dynamicSmemBytes = pair ? P_SMEM_ALLOC : SMEM_ALLOC;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0] = pdl_attribute();
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = pair ? 2 : plan.cs;
-  attr[1].val.clusterDim.y = 1;
-  attr[1].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = pair || plan.cs > 1 ? 2 : 1;
   const int64_t slots = pair ? (sms / 2 > 0 ? sms / 2 : 1) : sms;
-  if (plan.cs > 1)
-    cfg.gridDim = dim3(unsigned(tiles * plan.cs), 1, 1);
-  else
-    cfg.gridDim = dim3(unsigned((tiles < slots ? tiles : slots) * (pair ? 2 : 1)), 1, 1);
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, fn, p);
-  if (e != cudaSuccess) {
-    set_error("refadapt_gemm: launch failed: %s", cudaGetErrorString(e));
-    cudaGetLastError();
-    return RA_ECUDA;
+  p.slots = int32_t(slots);
+  p.rest_max = plan.rest_max;
+  if (plan.rest_max > 0) {
+    // No modes leave more whole rounds than all tiles do, or a larger split rest.
+    const int64_t rest = tiles % slots, whole = rest <= plan.rest_max ? tiles - rest : tiles;
+    const ra_status r = launch(p, kn.pair, P_SMEM_ALLOC, 2 * (whole < slots ? whole : slots), 2, st);
+    if (r != RA_OK) return r;
+    return launch(p, kn.split, SMEM_ALLOC, int64_t(4) * plan.rest_max * plan.cs, plan.cs, st);
   }
-  return launch_status("refadapt_gemm");
+  if (pair) return launch(p, kn.pair, P_SMEM_ALLOC, 2 * (tiles < slots ? tiles : slots), 2, st);
+  if (plan.cs > 1) return launch(p, kn.split, SMEM_ALLOC, tiles * plan.cs, plan.cs, st);
+  return launch(p, kn.single, SMEM_ALLOC, tiles < slots ? tiles : slots, 1, st);
 }

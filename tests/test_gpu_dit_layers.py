@@ -205,6 +205,19 @@ def test_gemm_split_k_matches_oracle(cuda_ok, epi, B, K, N, rows):
                inplace=epi == 2)
 
 
+# A little more than whole rounds of pair tiles (77 to 81 of them): the rest is split, its tiles
+# cut into quarters, of which some have no rows; with modes that leave no rest or no whole round.
+@pytest.mark.parametrize("epi,B,N,rows,modes", [(2, 1, 2816, [200, 1000, 300], [COMPUTE]),
+                                                (2, 1, 2816, [200, 1000, 300], [REUSE]),
+                                                (1, 2, 1280, [100, 700, 900], [COMPUTE, COMPUTE]),
+                                                (0, 2, 1280, [100, 700, 900], [REUSE, COMPUTE]),
+                                                (2, 3, 2304, [1, 257], [COMPUTE, REUSE, COMPUTE]),
+                                                (0, 3, 2304, [1, 385], [COMPUTE, COMPUTE, COMPUTE])])
+def test_gemm_split_rest_matches_oracle(cuda_ok, epi, B, N, rows, modes):
+    _gemm_case(B, 4160, N, rows, epi, torch.Generator().manual_seed(N + B), gated=[i == 1 for i in range(len(rows))],
+               modes=modes, inplace=epi == 2)
+
+
 @pytest.mark.parametrize("tile_mode", TILE_MODES)
 @pytest.mark.parametrize("H,d,modes", [(4, 64, [FULL, BOUNDARY]), (2, 128, [REUSE, COMPUTE])])
 def test_gemm_qkv_epilogue_matches_oracle(cuda_ok, H, d, modes, tile_mode):
