@@ -137,6 +137,10 @@ typedef struct {
  * cache slot as before and leave it untouched. This replaces a separate
  * refadapt_ref_cache_update (and its reads of the fresh tensors) on the
  * attention's own pass over them.
+ *
+ * Results are deterministic for given arguments and modes. How a row's keys are
+ * divided among CTAs (which sets the order of the fp32 sums) follows from the
+ * sizes of the call and the modes of its samples.
  *  ref_fresh_k/v    segments with n = k[RA_REF].n (16-byte aligned as above;
  *                   ptr NULL only when n = 0).
  *  ref_fresh_q      n = q[RA_REF].n when q[RA_REF] is given; ptr NULL and
@@ -419,7 +423,11 @@ ra_status refadapt_ln_modulate(const ra_lnmod_args* args, void* stream);
  * MMA on a tile of 256 rows, each SM staging half of the operands) or one CTA
  * per tile of 128 rows, whichever a model of the call's time prefers; 1 and 2
  * force either. Tiles are up to 256 columns wide, narrower where that saves a
- * round of tiles. Results are the same in every case.
+ * round of tiles; modes 1 and 2 give the same results. Mode 0 also lets the CTAs
+ * of a cluster share a tile's K where tiles are few and K is long: the fp32 sums
+ * of up to four parts of K are then added in a fixed order, so a call's results
+ * are deterministic, but a row's last rounding may depend on the call's other
+ * rows and on the modes.
  */
 typedef enum { RA_EPI_STORE = 0, RA_EPI_GELU = 1, RA_EPI_RESID = 2, RA_EPI_QKV = 3 } ra_epilogue;
 
