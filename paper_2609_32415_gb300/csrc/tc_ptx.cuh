@@ -343,17 +343,12 @@ __device__ __forceinline__ uint32_t cluster_size() {
   return r;
 }
 // The two halves of a cluster barrier, the arrival without release: it says
-// that this CTA has started and publishes nothing.
+// that this thread needs nothing more of the other CTAs and publishes nothing.
 __device__ __forceinline__ void cluster_arrive() {
   asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// 16 bytes into the shared memory of a CTA of the cluster.
-__device__ __forceinline__ void st_cluster_f4(uint32_t cluster_addr, float x, float y, float z, float w) {
-  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "f"(x), "f"(y), "f"(z), "f"(w)
-               : "memory");
 }
 // Bulk copy from this CTA's shared memory into another's; counted on an
 // mbarrier of the destination CTA (both shared::cluster addresses).
