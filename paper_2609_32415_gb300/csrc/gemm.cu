@@ -459,8 +459,9 @@ __device__ __forceinline__ bool epilogue_tile(const Params& p, const Tile& tl, c
 // there. Each rank hands every other rank that one's columns, in fp32, by a bulk
 // copy between the CTAs' shared memory (the stages are idle by then), and adds
 // its own columns up in rank order. Every thread of the cluster takes part in
-// the cluster barrier: before it every rank's stages are idle and its parts are
-// written, after it they are copied. ok: this warp's accumulator is complete.
+// the cluster barrier: before it every rank's barriers exist, its stages are idle
+// and its parts are written, after it they are copied (a cluster barrier of its
+// own in the set-up cost 0.2 us). ok: this warp's accumulator is complete.
 // The merge of a 128 x 256 tile between two CTAs (64 KB each way) takes 2.6 us.
 __device__ __forceinline__ bool merge_parts(const WaitCtl& ctl, uint8_t* smem, uint64_t* parts_full, uint32_t acc,
                                             bool ok, int bn, int half, int quarter, int rank, int cs) {
@@ -573,12 +574,11 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem0 = SPLIT ? 0 : *tmem_slot;  // SPLIT reads it per role: 0.3 us less there, 0.1 more without
   if (SPLIT && !*live) {  // uniform over the cluster
-    if (warp == 1) tmem_dealloc(tmem, TMEM_COLS);
+    if (warp == 1) tmem_dealloc(*tmem_slot, TMEM_COLS);
     return;
   }
-  if (SPLIT) cluster_sync_all();  // every CTA's barriers exist
   const WaitCtl ctl{abort_flag, p.err_word, p.budget_ns};
   pdl_launch();
   if (warp != 0) pdl_wait();
@@ -617,7 +617,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
     if (lane == 0) {
       // -------------------------------------------------------------- MMA issuer
       const uint32_t idesc = idesc_bf16_f32(BM, bn, 0, 0);
-      const uint32_t s0 = smem_u32(smem);
+      const uint32_t s0 = smem_u32(smem), tmem = SPLIT ? *tmem_slot : tmem0;
       int64_t it = 0;
       int i = 0;
       bool ok = true, issued = false;
@@ -652,6 +652,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
   } else {
     // ---------------------------------------------------------------- epilogue
     const int quarter = warp & 3;
+    const uint32_t tmem = SPLIT ? *tmem_slot : tmem0;
     EpiWarp w;
     w.half = (warp - 2) >> 2;
     w.stage = smem + OFF_EPI + (warp - 2) * EPI_WARP_BYTES;
@@ -696,7 +697,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem, TMEM_COLS);
+    tmem_dealloc(SPLIT ? *tmem_slot : tmem0, TMEM_COLS);
   }
 }
 
@@ -992,7 +993,7 @@ int max_clusters(Kernel fn, int cs) {
 // Few tiles of a long K leave SMs idle (a small model's MLP output, 377 rows by
 // N = 1024, K = 4096, is 64 narrow tiles, 19.2 us): there two or four CTAs of a
 // cluster share a tile's K, which costs a merge and pays from about K = 3072 up
-// while the clusters fit the GPU at once (12.2 us in clusters of four on tiles of
+// while the clusters fit the GPU at once (12.1 us in clusters of four on tiles of
 // 128 columns; 516 rows, K = 12288, N = 3072 58.9 -> 50.3 in clusters of two;
 // at K = 1024 it loses, 7.3 -> 8.2). Not for QKV, whose epilogue needs whole heads,
 // nor where the caller chose the tiles.
