@@ -1013,10 +1013,10 @@ Live live_items(const Params& p, int group, int nb) {
 // merge of a split item. What each form is for:
 //   pairs unsplit         full rounds: the least traffic per product;
 //   clusters              few items of many keys: every 8th target row of the
-//                         image-edit shape (72 items of 98 key tiles) 82 us in
+//                         image-edit shape (72 items of 98 key tiles) 81 us in
 //                         clusters of two, 143 unsplit, 87 in two streams;
 //   rounds, rest split    312 items of 26 key tiles (two rounds of 152 and 8)
-//                         112 us, 131 in three rounds;
+//                         111 us, 131 in three rounds;
 //   one tile, two streams items that fit few rounds: 8 heads, d = 64, of
 //                         32 + 256 + 256 rows 8.2 against 11.4 us, of 77 + 1000
 //                         + 500 rows 15.7 against 22.9 (half the latency per
