@@ -369,15 +369,18 @@ __device__ __forceinline__ void merge_split(const WaitCtl& ctl, uint8_t* smem, u
 }
 
 // Merge of the two streams of an item (both warpgroups; thread = row): each
-// reads the other's row maximum and sums (through the Q buffer, idle by then),
-// then combines both accumulators over its half of the columns. Leaves the
-// item's l and l_ref in l, lref.
+// reads the other's row maximum and sums (through the Q buffer), then combines
+// both accumulators over its half of the columns. Leaves the item's l and l_ref
+// in l, lref. The Q buffer is idle once the products are done, unless the item
+// copies its Q tile into the cache slot (q_stored): then the producer says when
+// that store has read it (barrier 4).
 template <int D>
-__device__ __forceinline__ void merge_dual(const WaitCtl& ctl, uint8_t* smem, uint64_t* o_done, uint32_t o_tmem, bool ok,
-                                           bool second, bool valid, int t, int row, float m, float& l, float& lref,
-                                           __nv_bfloat16* orow) {
+__device__ __forceinline__ void merge_dual(const WaitCtl& ctl, uint8_t* smem, uint64_t* o_done, uint32_t o_tmem,
+                                           bool ok, bool second, bool q_stored, bool valid, int t, int row, float m,
+                                           float& l, float& lref, __nv_bfloat16* orow) {
   float4* st = reinterpret_cast<float4*>(smem + Cfg<D, true>::OFF_Q);  // [stream][row]
   const bool done = __all_sync(0xffffffffu, mbar_wait(o_done, 0, ctl) && (!second || mbar_wait(o_done + 1, 0, ctl)));
+  if (q_stored) named_bar_sync(4, 288);
   if (done) st[t * BM + row] = make_float4(m, ok ? l : NAN, lref, 0.f);
   named_bar_sync(3, 256);
   if (!done) return;
@@ -532,6 +535,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
   const int j0 = SPLIT ? nkv_all * rank / nrank : 0;  // this CTA's first key tile
   const int nkv = SPLIT ? nkv_all * (rank + 1) / nrank - j0 : nkv_all;
   const bool second = DUAL ? nkv > 1 : has_b;  // the second softmax warpgroup works
+  const bool store_q = p.fresh && refreshes(mode) && p.store_q && role == 1 && rank == 0;
   // Register split: warpgroup 0 (producer, MMA issuer, two idle warps) gives
   // up registers to the two softmax warpgroups: 4 x 56 + 8 x 224 = 12 x 168,
   // the launch allocation.
@@ -542,7 +546,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
         // ------------------------------------------------------------ TMA producer
         const bool fresh = p.fresh && refreshes(mode);
         const bool store_kv = fresh && p.store_kv && first == 0;
-        const bool store_q = fresh && p.store_q && role == 1 && rank == 0;
         const CUtensorMap* tq = (role == 1 && fresh) ? &p.tm_qf : &p.tm_q[role];
         if (fresh && first == 0 && h == 0 && rank == 0 && p.a_b) p.a_b[b] = p.step;
         tma_prefetch_desc(tq);
@@ -611,9 +614,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
           if (j >= 1 && (store_kv || store_q) && !store_tiles(j - 1)) break;
         }
         if ((store_kv || store_q) && !*abort_flag && v_issued == nkv) store_tiles(nkv - 1);
-        // Shared memory must outlive the reads of every store issued; the
-        // cache slot is complete when the kernel is.
-        if (store_kv || store_q) bulk_wait_all();
+        // Shared memory must outlive the reads of every store issued.
+        if (store_kv || store_q) bulk_wait_read_all();
         if (*abort_flag) {
           // Let every load this thread issued land before the CTA exits: stage s
           // received loads for j = s, s + S, ...; wait for the last one's phase.
@@ -626,6 +628,11 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
           }
         }
       }
+      if (DUAL && store_q) {  // the store of Q has read its buffer (merge_dual)
+        __syncwarp();
+        named_bar_arrive(4, 288);
+      }
+      if (lane == 0) bulk_wait_all();  // the cache slot is complete when the kernel is
     } else if (warp == 1) {
       if (lane == 0) {
         // ------------------------------------------------------------ MMA issuer
@@ -726,7 +733,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
     if (lane == 0) {
       item_sh->x = b;
       item_sh->y = h;
-      item_sh->z = role;
+      item_sh->z = role + (store_q ? 4 : 0);
       item_sh->w = DUAL ? tileA : tileA + t;
     }
     __syncwarp();
@@ -837,7 +844,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
       mbar_arrive(p_ready + t);
     }
     if (ok) ok = __all_sync(0xffffffffu, mbar_wait(o_done + t, 0, ctl));
-    const int eb = item_sh->x, eh = item_sh->y, erole = item_sh->z, tile = item_sh->w;
+    const int eb = item_sh->x, eh = item_sh->y, erole = item_sh->z & 3, tile = item_sh->w;
+    const bool q_stored = item_sh->z >= 4;
     const int grow = tile * BM + row;
     const bool valid = (active || DUAL) && grow < p.nq[erole];
     __nv_bfloat16* orow = p.o_ptr[erole] + eb * p.o_sb[erole] + eh * p.o_sh[erole] + int64_t(grow) * p.o_sn[erole];
@@ -846,7 +854,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
       merge_split<D>(ctl, smem, parts_full, o_t, ok && active, has_b, valid, rank, nrank, t, row, m, l, lref, orow);
       inv_l = 1.f / l;
     } else if (DUAL) {
-      merge_dual<D>(ctl, smem, o_done, tmem + lane_off + C::TM_O, ok && active, second, valid, t, row, m, l, lref, orow);
+      merge_dual<D>(ctl, smem, o_done, tmem + lane_off + C::TM_O, ok && active, second, q_stored, valid, t, row, m, l,
+                    lref, orow);
       inv_l = 1.f / l;
     } else {
       inv_l = 1.f / l;

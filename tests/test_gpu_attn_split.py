@@ -133,3 +133,30 @@ def test_split_launches_write_the_cache(cuda_ok, rows, H, modes):
     ref = oracle_block({r: [x[:, hs] for x in segs[r]] for r in ROLES}, 0, COMPUTE, d ** -0.5)
     for r in ROLES:
         _assert_close(out[r][0, hs], ref["O"][r], r)
+
+
+@pytest.mark.parametrize("rows,H", [((0, 128, 20), 76), ((0, 90, 128), 20), ((5, 100, 40), 50), ((20, 250, 20), 30)])
+@pytest.mark.parametrize("d", [64, 128])
+def test_two_streams_keep_the_stored_query(cuda_ok, rows, H, d):
+    """Two to four key tiles: a reference-row item's merge comes soon after the
+    copy of its Q tile into the cache slot left the buffer the merge writes to.
+    The slot equals the fresh rows bit for bit, over repeated launches."""
+    from paper_2609_32415_gb300 import api
+    n = dict(zip(ROLES, rows))
+    segs = make_segments(1, H, d, n, gen=torch.Generator().manual_seed(H + d))
+    slot = [torch.zeros_like(x) for x in segs["ref"]]
+    a_b = torch.full((1,), -1, dtype=torch.int32, device="cuda")
+    out = empty_outputs(1, H, d, n)
+    mp = api.alloc_mass_partial(1, H, n["text"], n["tgt"])
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    mode = torch.tensor([COMPUTE], dtype=torch.int32, device="cuda")
+    for step in range(20):
+        for x in slot:
+            x.fill_(0.25)
+        api.refadapt_joint_attn([segs["text"][0], slot[0], segs["tgt"][0]], [segs["text"][1], slot[1], segs["tgt"][1]],
+                                [segs["text"][2], slot[2], segs["tgt"][2]], [out[r] for r in ROLES], mp, mode=mode,
+                                err_word=err, ref_fresh=tuple(segs["ref"]), a_b=a_b, step=step)
+        for got, fresh in zip(slot, segs["ref"]):
+            assert torch.equal(got, fresh)
+    api.refadapt_check_error(err)
+    assert a_b.tolist() == [19]
