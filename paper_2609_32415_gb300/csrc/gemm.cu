@@ -461,7 +461,9 @@ __device__ __forceinline__ bool epilogue_tile(const Params& p, const Tile& tl, c
 // its own columns up in rank order. Every thread of the cluster takes part in
 // the cluster barrier: before it every rank's barriers exist, its stages are idle
 // and its parts are written, after it they are copied (a cluster barrier of its
-// own in the set-up cost 0.2 us). ok: this warp's accumulator is complete.
+// own in the set-up cost 0.2 us). ok: this warp's accumulator is complete. Every
+// rank sends and waits for what it receives, also after a wait of this CTA was
+// given up: no CTA exits with a copy into it, or out of it, in flight.
 // The merge of a 128 x 256 tile between two CTAs (64 KB each way) takes 2.6 us.
 __device__ __forceinline__ bool merge_parts(const WaitCtl& ctl, uint8_t* smem, uint64_t* parts_full, uint32_t acc,
                                             bool ok, int bn, int half, int quarter, int rank, int cs) {
@@ -472,29 +474,33 @@ __device__ __forceinline__ bool merge_parts(const WaitCtl& ctl, uint8_t* smem, u
   uint8_t* recv = smem + (cs - 1) * part_bytes;      // parts from the other ranks, in rank order
   const bool leader = quarter == 0 && half == 0 && lane == 0;
   if (leader) mbar_arrive_expect_tx(parts_full, (cs - 1) * part_bytes);
-  if (ok) {
 #pragma unroll 1
-    for (int c0 = 32 * half; c0 < bn; c0 += 64) {
-      const int q = c0 / cw;
-      if (q == rank) continue;
-      uint32_t v[32];
-      tmem_ld32(acc + c0, v);
-      tmem_ld_wait_for(v);
-      uint4* dst = reinterpret_cast<uint4*>(send + (q - (q > rank ? 1 : 0)) * part_bytes) +
-                   ((c0 - q * cw) >> 2) * BM + row;
+  for (int c0 = 32 * half; c0 < bn; c0 += 64) {
+    const int q = c0 / cw;
+    if (q == rank) continue;
+    uint32_t v[32];
+    tmem_ld32(acc + c0, v);
+    tmem_ld_wait_for(v);
+    if (!ok) {  // what was given up is NaN on every rank
 #pragma unroll
-      for (int i = 0; i < 32; i += 4) dst[(i >> 2) * BM] = make_uint4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+      for (int i = 0; i < 32; ++i) v[i] = 0x7fffffffu;
     }
+    uint4* dst = reinterpret_cast<uint4*>(send + (q - (q > rank ? 1 : 0)) * part_bytes) +
+                 ((c0 - q * cw) >> 2) * BM + row;
+#pragma unroll
+    for (int i = 0; i < 32; i += 4) dst[(i >> 2) * BM] = make_uint4(v[i], v[i + 1], v[i + 2], v[i + 3]);
   }
   fence_proxy_async_smem();  // the parts are next read by bulk copies
   cluster_sync_all();
-  if (leader && !*ctl.abort_flag)
+  if (leader)
     for (int q = 0; q < cs; ++q)
       if (q != rank)
         bulk_copy_to_cta(mapa_shared(smem_u32(recv + (rank - (rank > q ? 1 : 0)) * part_bytes), q),
                          send + (q - (q > rank ? 1 : 0)) * part_bytes, part_bytes,
                          mapa_shared(smem_u32(parts_full), q));
-  if (!__all_sync(0xffffffffu, mbar_wait(parts_full, 0, ctl)) || !ok) return false;
+  const bool got = __all_sync(0xffffffffu, mbar_wait(parts_full, 0, ctl) ||
+                                               mbar_wait_drain(parts_full, 0, ctl.budget_ns));
+  if (!got || !ok) return false;
 #pragma unroll 1
   for (int c0 = 32 * half; c0 < cw; c0 += 64) {
     uint32_t v[32];
