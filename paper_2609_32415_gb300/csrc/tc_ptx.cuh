@@ -75,11 +75,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const 
   }
 }
 
-// Drain-time wait: ignores the abort flag, still bounded.
+// Drain-time wait, for copies and MMAs of this CTA that will end: ignores the
+// abort flag, still bounded. A caller's short budget does not shorten it, or the
+// CTA would exit with its copies in flight.
+constexpr uint64_t kDrainNs = 500000000;
 __device__ __forceinline__ bool mbar_wait_drain(uint64_t* bar, uint32_t parity, uint64_t budget_ns) {
+  if (mbar_try_wait(bar, parity)) return true;
   const uint64_t t0 = globaltimer_ns();
   while (!mbar_try_wait(bar, parity)) {
-    if (globaltimer_ns() - t0 > budget_ns) return false;
+    if (globaltimer_ns() - t0 > (budget_ns > kDrainNs ? budget_ns : kDrainNs)) return false;
   }
   return true;
 }
