@@ -372,7 +372,9 @@ ra_status refadapt_rope_table(float* table, int32_t n_pos, int32_t d, double bas
  * the variance; shift and scale are the block's AdaLN vectors for the row's
  * stream and sample, fp32 [B][C] (row stride mod_stride_s). bf16 in and out;
  * h and x must not overlap. C a multiple of 256, at most 4096; pointers
- * 16-byte aligned, row strides >= C and multiples of 8 elements. */
+ * 16-byte aligned, row strides >= C and multiples of 8 elements. The call waits
+ * only for its own copies and has no error word: rows whose copy did not end
+ * within the wait budget (at least 0.5 s) become NaN. */
 typedef struct {
   const void* h;
   int64_t h_stride_s, h_stride_r;

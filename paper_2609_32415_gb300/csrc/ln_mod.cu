@@ -80,6 +80,28 @@ struct Piece {
   }
 };
 
+// A warp whose own copy of row i did not end within the budget: it lets the
+// copies on their way (of its next S - 1 rows) land, and its rows from i on
+// become NaN.
+template <int G>
+__device__ __noinline__ void give_up(const Params& p, uint64_t* full, int stage, uint32_t phase, int64_t i, int64_t hi) {
+  using L = Layout<G>;
+  for (int k = 1; k < L::S && i + k * L::WARPS < hi; ++k) {
+    if (++stage == L::S) {
+      stage = 0;
+      phase ^= 1;
+    }
+    mbar_wait_drain(full + stage, phase, p.budget_ns);
+  }
+  Piece w{0, 0, 0};
+  for (; i < hi; i += L::WARPS) {
+    w.seek(p, i);
+    const Seg& sg = p.seg[w.g];
+    uint4* dst = reinterpret_cast<uint4*>(sg.x + w.s * sg.x_ss + (i - w.begin) * sg.x_sr);
+    for (int q = 0; q < G; ++q) dst[q * 32 + (threadIdx.x & 31)] = make_uint4(~0u, ~0u, ~0u, ~0u);
+  }
+}
+
 template <int G>  // 8-feature groups per lane: C = 256 G
 __global__ void __launch_bounds__(32 * Layout<G>::WARPS, 1) ln_mod_kernel(const __grid_constant__ Params p) {
   using L = Layout<G>;
@@ -125,7 +147,6 @@ __global__ void __launch_bounds__(32 * Layout<G>::WARPS, 1) ln_mod_kernel(const 
   for (int k = 0; k < S; ++k) load(k);
   int stage = 0;
   uint32_t phase = 0;
-  bool ok = true;
   for (int64_t piece_lo = lo; piece_lo < hi;) {
     w.seek(p, piece_lo);
     const Seg& sg = p.seg[w.g];
@@ -144,10 +165,11 @@ __global__ void __launch_bounds__(32 * Layout<G>::WARPS, 1) ln_mod_kernel(const 
     }
     __syncthreads();
     for (; i < piece_hi; i += W) {
-      // This warp's own bulk copy ends, or the budget does (then the warp
-      // writes no more rows).
-      ok = ok && __all_sync(0xffffffffu, mbar_wait_drain(full + stage, phase, p.budget_ns));
-      if (!ok) continue;
+      if (!__all_sync(0xffffffffu, mbar_wait_drain(full + stage, phase, p.budget_ns))) {
+        give_up<G>(p, full, stage, phase, i, hi);
+        i = hi;
+        break;
+      }
       uint4 u[G];
       const uint4* src = reinterpret_cast<const uint4*>(ring + stage * L::ROW_BYTES);
 #pragma unroll

@@ -102,6 +102,26 @@ def test_ln_modulate_pieces(cuda_ok, C, B, rows):
             assert ok, (i, s, nbad, eq)
 
 
+def test_ln_modulate_with_a_short_wait_budget(cuda_ok):
+    """The rows' own copies end; a wait budget that does not cover them leaves no row unwritten."""
+    from paper_2609_32415_gb300 import api
+    g = torch.Generator().manual_seed(3)
+    C, n = 3072, 1500
+    sd = {"h": _bf((2, n, C), g).cuda(), "shift": torch.randn((2, C), generator=g).cuda(),
+          "scale": torch.randn((2, C), generator=g).cuda()}
+    x = [torch.full((2, n, C), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    api.refadapt_ln_modulate([dict(sd, x=x[0])], C)
+    api.refadapt_set_wait_budget_ns(1)
+    try:
+        for _ in range(10):
+            api.refadapt_ln_modulate([dict(sd, x=x[1])], C)
+            torch.cuda.synchronize()
+            assert torch.equal(x[0].view(torch.int16), x[1].view(torch.int16))
+            x[1].fill_(float("nan"))
+    finally:
+        api.refadapt_set_wait_budget_ns(500_000_000)
+
+
 def _gemm_case(B, K, N, rows_list, epi, g, gated=None, modes=None, inplace=False, tile_mode=0):
     from paper_2609_32415_gb300 import api
     from paper_2609_32415_gb300._lib import RA_EPI_GELU, RA_EPI_RESID, RA_EPI_STORE
