@@ -293,11 +293,14 @@ class Executor:
         are those of the one-stream order. Every event is recorded inside the
         step, which can be captured as a CUDA graph."""
         if not self.overlap or self.n_blocks == 1:  # one block: nothing to run beside
-            for b in range(self.n_blocks):
-                out = outs[b] if outs is not None else self.scratch_outputs(b % 2)
-                self.block(t, b, inputs[b], out, log_index, stream)
-                if after_block is not None:
-                    after_block(t, b)
+            # with overlap the hooks see the attention's stream as the current one
+            on = self.overlap and stream is not None and (after_block is not None or self.attn_hook is not None)
+            with torch.cuda.stream(stream) if on else contextlib.nullcontext():
+                for b in range(self.n_blocks):
+                    out = outs[b] if outs is not None else self.scratch_outputs(b % 2)
+                    self.block(t, b, inputs[b], out, log_index, stream)
+                    if after_block is not None:
+                        after_block(t, b)
             return
         caller = torch.cuda.current_stream() if stream is None else stream
         side = self._side
