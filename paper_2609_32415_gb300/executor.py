@@ -24,6 +24,7 @@ from . import api
 from ._lib import RA_MODE_BOUNDARY, RA_MODE_COMPUTE, RA_MODE_FULL, RA_MODE_REUSE  # noqa: F401
 
 ROLES = ("text", "ref", "tgt")
+_NULL = contextlib.nullcontext()
 
 
 def roles_from_joint(X, offsets, n):
@@ -146,20 +147,35 @@ class Executor:
                                             device=dev)
             self._o_fresh = [{"text": torch.empty((B, H, n_text, d), dtype=torch.bfloat16, device=dev),
                               "tgt": torch.empty((B, H, n_s, d), dtype=torch.bfloat16, device=dev)} for _ in range(2)]
-        # The views a block's launches take, made once: indexing a tensor costs
-        # microseconds of host time, and a block takes ten of them.
-        self._block = list(zip(self.cache_x.unbind(0), self.cache_k.unbind(0), self.cache_v.unbind(0),
-                               self.a_b.unbind(0), self.mass.unbind(0), self.D.unbind(0)))
-        self._logs = [list(zip(m.unbind(0), g.unbind(0), e.unbind(0)))
-                      for m, g, e in zip(self.modes.unbind(0), self.gbar.unbind(0), self.M.unbind(0))]
+        self._make_views()
         self._out = [None, None]
         self.attn_hook = None   # optional callable(phase in {"pre", "post"}, t, b), e.g. CUDA events
         self.nvtx = bool(nvtx)
 
+    # The views that a block's launches take: indexing a tensor costs microseconds
+    # of host time, and a block takes ten of them. They are made once, and again
+    # when one of their buffers was assigned.
+    _VIEWED = frozenset(("cache_x", "cache_k", "cache_v", "a_b", "mass", "D", "modes", "gbar", "M"))
+
+    def __setattr__(self, name, value):
+        object.__setattr__(self, name, value)
+        if name in self._VIEWED:
+            object.__setattr__(self, "_views", None)
+
+    def _make_views(self):
+        """(blocks, logs): blocks[b] = cache_x, cache_k, cache_v, a_b, mass and D
+        of block b, logs[step][b] = its modes, gbar and M."""
+        blocks = list(zip(self.cache_x.unbind(0), self.cache_k.unbind(0), self.cache_v.unbind(0), self.a_b.unbind(0),
+                          self.mass.unbind(0), self.D.unbind(0)))
+        logs = [list(zip(m.unbind(0), g.unbind(0), e.unbind(0)))
+                for m, g, e in zip(self.modes.unbind(0), self.gbar.unbind(0), self.M.unbind(0))]
+        self._views = blocks, logs
+        return self._views
+
     def _range(self, name):
         """An NVTX range around the launches it encloses (nvtx=True), for
         timeline profilers; nothing otherwise."""
-        return torch.cuda.nvtx.range(name) if self.nvtx else contextlib.nullcontext()
+        return torch.cuda.nvtx.range(name) if self.nvtx else _NULL
 
     def scratch_outputs(self, parity=0):
         """A set of O buffers (text, ref, tgt) reused by every block of one
@@ -186,15 +202,16 @@ class Executor:
         not read). The caller keeps qt alive until step t + 1's gate of this
         block has been enqueued (it is read as q_{t-1})."""
         li = (t % self.log_steps) if log_index is None else log_index
-        mode = self._logs[li][b][0]
+        mode = (self._views or self._make_views())[1][li][b][0]
         have_prev = t >= 1 and self._prev_qtgt[b] is not None
         with self._range("t%d b%d decision" % (t, b)):
             self._decide(t, b, qt, li, mode, have_prev, stream)
         self._prev_qtgt[b] = qt
 
     def _decide(self, t, b, qt, li, mode, have_prev, stream):
-        _, gbar, M = self._logs[li][b]
-        mass, D = self._block[b][4:]
+        blocks, logs = self._views
+        mass, D = blocks[b][4:]
+        _, gbar, M = logs[li][b]
         if have_prev:
             # Eq. 1 and the decision in one call (one launch on the cluster path)
             ref_q = self.anchor[b] if self.anchor is not None else self._prev_qtgt[b]
@@ -229,8 +246,10 @@ class Executor:
         cache slot and stamp a_b = t."""
         li = (t % self.log_steps) if log_index is None else log_index
         qr, kr, vr = x["ref"]
-        api.refadapt_ref_cache_update(kr, vr, self.cache_k[b], self.cache_v[b], self.modes[li, b], t, self.a_b[b],
-                                      x_src=qr, x_cache=self.cache_x[b], stream=stream)
+        blocks, logs = self._views or self._make_views()
+        cache_x, cache_k, cache_v, a_b = blocks[b][:4]
+        api.refadapt_ref_cache_update(kr, vr, cache_k, cache_v, logs[li][b][0], t, a_b, x_src=qr, x_cache=cache_x,
+                                      stream=stream)
 
     def attend(self, t, b, x, out, log_index=None, stream=None):
         """Block b's joint attention of step t (after its gate, and after its
@@ -238,7 +257,7 @@ class Executor:
         step's gate reads. With fused_cache, materialising samples read x[ref]
         and the kernel writes it into the cache slot and stamps a_b = t."""
         li = (t % self.log_steps) if log_index is None else log_index
-        mode = self._logs[li][b][0]
+        mode = (self._views or self._make_views())[1][li][b][0]
         qt = x["tgt"][0]
         if self.attn_hook is not None:
             self.attn_hook("pre", t, b)
@@ -250,7 +269,7 @@ class Executor:
             self._diagnose(t, b, li, x, out, stream)
 
     def _attend(self, t, b, x, out, mode, qt, stream):
-        cache_x, cache_k, cache_v, a_b, mass, _ = self._block[b]
+        cache_x, cache_k, cache_v, a_b, mass, _ = self._views[0][b]
         api.refadapt_joint_attn(
             (x["text"][0], cache_x, qt), (x["text"][1], cache_k, x["tgt"][1]), (x["text"][2], cache_v, x["tgt"][2]),
             (out["text"], out["ref"], out["tgt"]), mass, mode=mode, softmax_scale=self.softmax_scale, ref_logit_bias=self.bias,
@@ -262,8 +281,9 @@ class Executor:
         k = self.diag_row_stride
         ws, of = self.workspace_diag[b % 2], self._o_fresh[b % 2]
         qr, kr, vr = x["ref"]
-        api.refadapt_q_delta(kr, self.cache_k[b], self.E_K[li, b], ws, self.eps, stream)
-        api.refadapt_q_delta(vr, self.cache_v[b], self.E_V[li, b], ws, self.eps, stream)
+        _, cache_k, cache_v = self._views[0][b][:3]
+        api.refadapt_q_delta(kr, cache_k, self.E_K[li, b], ws, self.eps, stream)
+        api.refadapt_q_delta(vr, cache_v, self.E_V[li, b], ws, self.eps, stream)
         q_s = x["tgt"][0][:, :, ::k, :]
         api.refadapt_joint_attn(
             (x["text"][0], None, q_s), (x["text"][1], kr, x["tgt"][1]), (x["text"][2], vr, x["tgt"][2]),
@@ -295,7 +315,7 @@ class Executor:
         if not self.overlap or self.n_blocks == 1:  # one block: nothing to run beside
             # with overlap the hooks see the attention's stream as the current one
             on = self.overlap and stream is not None and (after_block is not None or self.attn_hook is not None)
-            with torch.cuda.stream(stream) if on else contextlib.nullcontext():
+            with torch.cuda.stream(stream) if on else _NULL:
                 for b in range(self.n_blocks):
                     out = outs[b] if outs is not None else self.scratch_outputs(b % 2)
                     self.block(t, b, inputs[b], out, log_index, stream)
@@ -319,7 +339,7 @@ class Executor:
             self._decided[b].record(side)
             main.wait_event(self._decided[b])
             # the attention's hook records on the current stream
-            with torch.cuda.stream(main) if self.attn_hook is not None else contextlib.nullcontext():
+            with torch.cuda.stream(main) if self.attn_hook is not None else _NULL:
                 self.attend(t, b, inputs[b], out, log_index, main)
             self._attn_done[b].record(main)
             if after_block is not None:

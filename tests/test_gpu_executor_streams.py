@@ -1,4 +1,4 @@
-"""The stream that the Executor's hooks run on."""
+"""Where the Executor's hooks run, and which buffers its launches take."""
 import pytest
 import torch
 
@@ -42,3 +42,24 @@ def test_hooks_run_behind_the_attention(cuda_ok, n_blocks, explicit):
     ex.check()
     assert len(seen) == 3 * n_blocks and all(any(s == a for a in allowed) for s in seen)
     assert all(torch.equal(c, o["tgt"]) for c, o in zip(copies, outs))
+
+
+@pytest.mark.parametrize("fused", [True, False])
+def test_assigned_buffers_are_used(cuda_ok, fused):
+    """A buffer that the caller assigns to the executor is the one that its next launches take."""
+    wl, ex, xs = _setup(2, fused_cache=fused)
+    _, same, _ = _setup(2, fused_cache=fused)
+    names = ("cache_k", "cache_v", "cache_x", "a_b", "mass", "D", "modes", "gbar", "M")
+    old = {k: getattr(ex, k) for k in names}
+    kept = {k: x.clone() for k, x in old.items()}
+    for k in names:
+        setattr(ex, k, old[k].clone())
+    for t in range(2):
+        ex.step(t, xs[t])
+        same.step(t, xs[t])
+    torch.cuda.synchronize()
+    ex.check()
+    for k in names:
+        assert torch.equal(old[k], kept[k]), k
+        assert torch.equal(getattr(ex, k).nan_to_num(), getattr(same, k).nan_to_num()), k
+    assert (ex.modes[0] == 3).all() and (ex.a_b >= 0).all()
