@@ -749,9 +749,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
     const bool active = (t == 0) || second;
     const float sl2 = p.scale_log2;
     const float bias_l2 = (role == 2 && p.bias) ? __ldg(p.bias + h) * kLog2e : 0.f;
-    // A rank's or a stream's keys may all be masked (a reference bias of -inf):
-    // the lowest finite start keeps their probabilities 0.
-    float m = KIND != KIND_PAIR ? kLowestMax : -INFINITY, l = 0.f, lref = 0.f;
+    // The first keys may all be masked (a reference bias of -inf): the lowest
+    // finite start keeps their probabilities 0.
+    float m = kLowestMax, l = 0.f, lref = 0.f;
     bool ok = active;
     // DUAL: this warpgroup's key tiles are t, t + 2, ...
     for (int j = 0; ok && (DUAL ? 2 * j + t : j) < nkv; ++j) {
@@ -787,7 +787,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
         if (DUAL && nvalid < BN) mx = fmaxf(mask64(va, 0, nvalid), mask64(vb, 64, nvalid));
         const float mt = fmaf(mx, sl2, badd);  // tile max, log2 units
         if (mt > m + kRescaleThresh) {
-          alpha = ex2_approx(m - mt);  // 0 when m = -inf
+          alpha = ex2_approx(m - mt);  // 0 at the start
           resc = (j > 0);
           l *= alpha;
           lref *= alpha;

@@ -160,3 +160,23 @@ def test_two_streams_keep_the_stored_query(cuda_ok, rows, H, d):
             assert torch.equal(got, fresh)
     api.refadapt_check_error(err)
     assert a_b.tolist() == [19]
+
+
+@pytest.mark.parametrize("rows,H,d", [((0, 128, 4000), 24, 64), ((0, 130, 5000), 8, 128), ((0, 128, 77), 3, 64),
+                                      ((0, 1800, 1800), 12, 128)])
+def test_masked_reference_without_text(cuda_ok, rows, H, d):
+    """A reference bias of -inf where the first key tile is the reference's:
+    target rows attend to the target keys alone, in every launch form (pairs,
+    two streams, whole rounds and a split rest)."""
+    n = dict(zip(ROLES, rows))
+    segs = make_segments(1, H, d, n, gen=torch.Generator().manual_seed(d + H), std=1.0)
+    bias = [float("-inf")] + [0.25] * (H - 1)
+    out, mp = _run(segs, 1, H, d, n, [FULL], bias=bias)
+    cut = {r: [x[:, :1, :0] if r == "ref" else x[:, :1] for x in segs[r]] for r in ROLES}
+    _assert_close(out["tgt"][0, :1], oracle_block(cut, 0, REUSE, d ** -0.5)["O"]["tgt"])
+    assert float(mp[0, 0].abs().max()) == 0.0
+    s2, o2, m2 = _heads(segs, out, mp, [H - 1])
+    full = oracle_block(s2, 0, FULL, d ** -0.5, np.array([0.25]))
+    for r in ("ref", "tgt"):
+        _assert_close(o2[r][0], full["O"][r], r)
+    assert abs(float(m2.double().sum()) / n["tgt"] - full["M"][0]) <= M_ABS
