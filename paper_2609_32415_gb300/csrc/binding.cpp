@@ -39,6 +39,15 @@ long long integer(PyObject* o) {
   return v;
 }
 int32_t integer32(PyObject* o) { return int32_t(integer(o)); }
+// int(o): any number, or its text.
+int32_t as_int32(PyObject* o) {
+  PyObject* v = PyNumber_Long(o);
+  if (!v) throw Raised{};
+  const long long x = PyLong_AsLongLong(v);
+  Py_DECREF(v);
+  if (x == -1 && PyErr_Occurred()) throw Raised{};
+  return int32_t(x);
+}
 double real(PyObject* o) {
   const double v = PyFloat_AsDouble(o);
   if (v == -1.0 && PyErr_Occurred()) throw Raised{};
@@ -143,6 +152,11 @@ struct Map {
     if (!v && PyErr_Occurred()) throw Raised{};
     return v ? v : Py_None;
   }
+  bool has(PyObject* key) const {
+    const int v = PyDict_Contains(dict, key);
+    if (v < 0) throw Raised{};
+    return v != 0;
+  }
   PyObject* need(PyObject* key) const {
     PyObject* v = PyDict_GetItemWithError(dict, key);
     if (!v) {
@@ -219,7 +233,7 @@ PyObject* joint_attn(PyObject*, PyObject* const* g, Py_ssize_t n) {
     a.err_word = static_cast<int32_t*>(address(g[9]));
     a.mass_row_stride = integer32(g[10]);
     if (g[11] != Py_None) {
-      const Seq f(g[11], 3);
+      const Seq f(g[11], 0);
       if (f.size() != 3) raise(PyExc_ValueError, "ref_fresh: expected (q, k, v)");
       a.ref_fresh_q = seg(f[0]);
       a.ref_fresh_k = seg(f[1]);
@@ -386,7 +400,7 @@ PyObject* gemm(PyObject*, PyObject* const* g, Py_ssize_t n) {
         s.v_out = seg(sd.need(N.v));
         s.q_norm = static_cast<const float*>(address(sd.need(N.q_norm)));
         s.k_norm = static_cast<const float*>(address(sd.need(N.k_norm)));
-        if (PyObject* po = sd.get(N.pos_offset); po != Py_None) s.pos_offset = integer32(po);
+        s.pos_offset = sd.has(N.pos_offset) ? as_int32(sd.need(N.pos_offset)) : 0;
       }
     }
     if (segs.size() == 0) raise(PyExc_TypeError, "refadapt_gemm: no segments");

@@ -254,6 +254,25 @@ def test_gemm_qkv_wide_tiles_match_oracle(cuda_ok, H, d, tgt, tile_mode):
     _qkv_case(H, d, [BOUNDARY, COMPUTE], tile_mode, {"text": 37, "ref": 300, "tgt": tgt})
 
 
+def test_gemm_qkv_position_offset_is_any_number(cuda_ok):
+    """pos_offset is taken as int() takes it."""
+    from paper_2609_32415_gb300 import api
+    from paper_2609_32415_gb300._lib import RA_EPI_QKV
+    H, d, C = 4, 64, 256
+    g = torch.Generator().manual_seed(4)
+    sd = {"a": _bf((1, 9, C), g).cuda(), "w": _bf((3 * C, C), g).cuda(), "q_norm": torch.ones(d, device="cuda"),
+          "k_norm": torch.ones(d, device="cuda")}
+    got = []
+    for pos in (7, 7.0, np.float32(7.5), "7"):
+        out = {z: torch.empty((1, H, 9, d), dtype=torch.bfloat16, device="cuda") for z in "qkv"}
+        api.refadapt_gemm([dict(sd, **out, pos_offset=pos)], 3 * C, C, RA_EPI_QKV, rope=api.rope_table(16, d), H=H, d=d)
+        got.append(out)
+    with pytest.raises(TypeError):
+        api.refadapt_gemm([dict(sd, **out, pos_offset=None)], 3 * C, C, RA_EPI_QKV, rope=api.rope_table(16, d), H=H, d=d)
+    torch.cuda.synchronize()
+    assert all(torch.equal(o[z], got[0][z]) for o in got for z in "qkv")
+
+
 def _qkv_case(H, d, modes, tile_mode, n):
     from paper_2609_32415_gb300 import api
     from paper_2609_32415_gb300._lib import RA_EPI_QKV
