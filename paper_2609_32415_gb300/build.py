@@ -5,7 +5,8 @@ Each .cu under csrc/ is compiled in parallel to an object file, then all are
 linked into paper_2609_32415_gb300/librefadapt.so (static CUDA runtime, no
 torch dependency). csrc/binding.cpp is compiled with the host compiler against
 the installed torch's headers meanwhile and linked to that library. Rebuilds
-only when a source or header is newer than the libraries.
+only when a source or header is newer than the libraries, or when _binding.so was
+made for another torch or Python than the ones that run.
 """
 import glob
 import os
@@ -22,6 +23,7 @@ BUILD_DIR = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "librefadapt.so")
 BINDING_SRC = os.path.join(CSRC, "binding.cpp")
 BINDING = os.path.join(PKG, "_binding.so")
+BINDING_FOR = os.path.join(BUILD_DIR, "binding.for")  # what _binding.so was made for
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -41,9 +43,17 @@ def _deps():
         glob.glob(os.path.join(INCLUDE, "*.h")) + [os.path.abspath(__file__)]
 
 
+def _binding_for() -> str:
+    import torch
+    return "torch %s, %s" % (torch.__version__, sys.implementation.cache_tag)
+
+
 def up_to_date() -> bool:
-    if not os.path.exists(LIB) or not os.path.exists(BINDING):
+    if not os.path.exists(LIB) or not os.path.exists(BINDING) or not os.path.exists(BINDING_FOR):
         return False
+    with open(BINDING_FOR) as f:
+        if f.read() != _binding_for():
+            return False
     t = min(os.path.getmtime(LIB), os.path.getmtime(BINDING))
     return all(os.path.getmtime(f) <= t for f in _deps())
 
@@ -77,6 +87,8 @@ def _link_binding(obj):
     _run([os.environ.get("CXX", "g++"), "-shared", "-o", tmp, obj, "-L", PKG, "-l:librefadapt.so", "-Wl,-rpath,$ORIGIN",
           "-L", lib, "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"], "linking _binding.so")
     os.replace(tmp, BINDING)
+    with open(BINDING_FOR, "w") as f:
+        f.write(_binding_for())
 
 
 def build(force: bool = False, verbose: bool = False, extra_flags=None) -> str:

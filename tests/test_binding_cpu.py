@@ -33,3 +33,11 @@ def test_row_segments_are_checked():
         api.refadapt_gemm([{"a": x, "w": x[0], "out": x}], 256, 256, 0)
     with pytest.raises(TypeError):
         api.refadapt_gemm([], 256, 256, 0)
+
+
+def test_a_binding_for_another_torch_is_rebuilt(monkeypatch):
+    from paper_2609_32415_gb300 import build
+    build.build()
+    assert build.up_to_date()
+    monkeypatch.setattr(torch, "__version__", "0.0.0")
+    assert not build.up_to_date()
