@@ -148,7 +148,7 @@ struct Walk {
 
   __device__ __forceinline__ int piece_cols(const Params& p) const {
     if (p.gated[g]) {
-      const int m = __ldg(p.mode + s);
+      const int m = p.mode[s];
       if (m == RA_MODE_REUSE) return 0;
       if (EPI == RA_EPI_QKV && m == RA_MODE_BOUNDARY) return p.cols_q;
     }
@@ -301,8 +301,8 @@ __device__ __forceinline__ bool epilogue_linear(const Params& p, const Tile& tl,
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     if (j >= chunks) break;
-    w.vec0[32 * j + lane] = sg.bias ? __ldg(sg.bias + n0 + 64 * j + lane) : 0.f;
-    if (EPI == RA_EPI_RESID) w.vec1[32 * j + lane] = __ldg(sg.gate + int64_t(tl.s) * sg.gate_ss + n0 + 64 * j + lane);
+    w.vec0[32 * j + lane] = sg.bias ? sg.bias[n0 + 64 * j + lane] : 0.f;
+    if (EPI == RA_EPI_RESID) w.vec1[32 * j + lane] = sg.gate[int64_t(tl.s) * sg.gate_ss + n0 + 64 * j + lane];
   }
   const char* res = nullptr;
   uint4 ra[4], rb[4];  // residuals of the next even and odd chunk
@@ -371,8 +371,8 @@ __device__ __forceinline__ bool epilogue_qkv(const Params& p, const Tile& tl, co
   for (int j = 0; j < 4; ++j) {
     if (j / CH >= heads) break;
     const int c = 32 * (j % CH) + lane;  // column within head h0 + 2 (j / CH)
-    w.vec0[32 * j + lane] = sg.bias ? __ldg(sg.bias + part * p.C + (h0 + 2 * (j / CH)) * D + c) : 0.f;
-    if (part < 2) w.vec1[32 * j + lane] = __ldg(sg.norm_w[part] + c);
+    w.vec0[32 * j + lane] = sg.bias ? sg.bias[part * p.C + (h0 + 2 * (j / CH)) * D + c] : 0.f;
+    if (part < 2) w.vec1[32 * j + lane] = sg.norm_w[part][c];
   }
   __syncwarp();
   // RoPE rows of the warp's positions: (cos, sin) of D / 2 pairs, 64 bytes = 16 columns at a time

@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
   pdl_launch();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = SPLIT ? int(cluster_rank()) : 0, nrank = SPLIT ? int(cluster_size()) : 1;
-  const int lane_mode = (lane < p.nb && p.mode) ? __ldg(p.mode + p.b0 + lane) : int(RA_MODE_FULL);
+  const int lane_mode = (lane < p.nb && p.mode) ? p.mode[p.b0 + lane] : int(RA_MODE_FULL);
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -748,7 +748,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
     const uint32_t o_t = tmem + lane_off + C::TM_O + 128 * t;
     const bool active = (t == 0) || second;
     const float sl2 = p.scale_log2;
-    const float bias_l2 = (role == 2 && p.bias) ? __ldg(p.bias + h) * kLog2e : 0.f;
+    const float bias_l2 = (role == 2 && p.bias) ? p.bias[h] * kLog2e : 0.f;
     // The first keys may all be masked (a reference bias of -inf): the lowest
     // finite start keeps their probabilities 0.
     float m = kLowestMax, l = 0.f, lref = 0.f;

@@ -60,7 +60,7 @@ struct Params {
 };
 
 __device__ __forceinline__ bool live(const Params& p, int g, int s) {
-  return !p.seg[g].gated || __ldg(p.mode + s) != RA_MODE_REUSE;
+  return !p.seg[g].gated || p.mode[s] != RA_MODE_REUSE;
 }
 
 // Live rows in order: segments, samples within, rows within. A piece is the
@@ -158,8 +158,8 @@ __global__ void __launch_bounds__(32 * Layout<G>::WARPS, 1) ln_mod_kernel(const 
       // Four columns: half f % 2 of lane (f / 2) % 32 in group f / 64; kept as
       // [group][half][lane], so the rows' 16-byte reads have no bank conflicts.
       const int at = ((f >> 6) * 2 + (f & 1)) * 32 + ((f >> 1) & 31);
-      reinterpret_cast<float4*>(shift_sh)[at] = __ldg(reinterpret_cast<const float4*>(shift) + f);
-      float4 v = __ldg(reinterpret_cast<const float4*>(scale) + f);
+      reinterpret_cast<float4*>(shift_sh)[at] = reinterpret_cast<const float4*>(shift)[f];
+      float4 v = reinterpret_cast<const float4*>(scale)[f];
       v.x += 1.f, v.y += 1.f, v.z += 1.f, v.w += 1.f;
       reinterpret_cast<float4*>(scale_sh)[at] = v;
     }

@@ -491,7 +491,9 @@ __device__ __forceinline__ uint64_t bf2_unpack(uint32_t w) {
 // Programmatic dependent launch. A kernel launched with it may start while the
 // previous kernel of its stream finishes: pdl_wait() returns once that one is
 // complete and its writes are visible, and comes before anything that depends
-// on it (every global access). pdl_launch() lets the next kernel of the stream
+// on it (every global access). Such a kernel reads what the previous one may have
+// written with plain loads: __ldg asks for memory that nothing writes while the
+// kernel runs, and the kernel runs by then. pdl_launch() lets the next kernel of the stream
 // start its own set-up (once every CTA of this grid got there or ended).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
