@@ -102,6 +102,47 @@ def test_ln_modulate_pieces(cuda_ok, C, B, rows):
             assert ok, (i, s, nbad, eq)
 
 
+@pytest.mark.parametrize("C", [256, 512, 768, 2048, 3072, 4096])
+def test_ln_modulate_by_row_and_persistent_agree(cuda_ok, C):
+    """A call of many rows of a few samples, and calls of one and of a few rows of
+    each: a row's result does not depend on the kernel that the call takes."""
+    from paper_2609_32415_gb300 import api
+    g = torch.Generator().manual_seed(C)
+    B, n = 2, 9000
+    h, mods = _bf((B, n, C), g).cuda(), [torch.randn((B, C), generator=g).cuda() for _ in range(2)]
+    seg = {"shift": mods[0], "scale": mods[1]}
+    x = torch.empty_like(h)
+    api.refadapt_ln_modulate([dict(seg, h=h, x=x)], C)
+    for lo, hi in ((0, 1), (4000, 4007), (n - 1, n)):
+        y = torch.empty((B, hi - lo, C), dtype=torch.bfloat16, device="cuda")
+        api.refadapt_ln_modulate([dict(seg, h=h[:, lo:hi], x=y)], C)
+        assert torch.equal(y, x[:, lo:hi])
+    ref = torch.nn.functional.layer_norm(h[:, ::500].double(), (C,), eps=1e-6)
+    ref = ref * (1 + mods[1].double()[:, None]) + mods[0].double()[:, None]
+    assert (x[:, ::500].double() - ref).abs().max() <= 2.0 ** -8 * ref.abs().max()
+
+
+@pytest.mark.parametrize("C,B,rows", [(1280, 300, (3, 0, 20)), (3072, 70, (1, 200, 2)), (512, 33, (0, 1, 400)),
+                                      (3072, 9, (40, 300, 2000))])
+def test_ln_modulate_many_samples(cuda_ok, C, B, rows):
+    from paper_2609_32415_gb300 import api
+    g = torch.Generator().manual_seed(B)
+    modes = [int(m) for m in torch.randint(0, 4, (B,), generator=g)]
+    segs = [{"h": _bf((B, n, C), g).cuda(), "x": torch.full((B, n, C), float("nan"), dtype=torch.bfloat16, device="cuda"),
+             "shift": torch.randn((B, C), generator=g).cuda(), "scale": torch.randn((B, C), generator=g).cuda(),
+             "gated": i == 1} for i, n in enumerate(rows)]
+    api.refadapt_ln_modulate(segs, C, mode=torch.tensor(modes, dtype=torch.int32, device="cuda"))
+    reuse = torch.tensor([m == REUSE for m in modes], device="cuda")
+    for i, sd in enumerate(segs):
+        if sd["h"].numel() == 0:
+            continue
+        ref = torch.nn.functional.layer_norm(sd["h"].double(), (C,), eps=1e-6)
+        ref = ref * (1 + sd["scale"].double()[:, None]) + sd["shift"].double()[:, None]
+        live = ~reuse if i == 1 else torch.ones_like(reuse)
+        assert bool(torch.isnan(sd["x"][~live]).all())
+        assert (sd["x"][live].double() - ref[live]).abs().max() <= 2.0 ** -8 * ref.abs().max()
+
+
 def test_ln_modulate_with_a_short_wait_budget(cuda_ok):
     """The rows' own copies end; a wait budget that does not cover them leaves no row unwritten."""
     from paper_2609_32415_gb300 import api
