@@ -73,7 +73,7 @@ constexpr int BM = 128;  // query rows per tile (= TMEM lanes)
 constexpr int BN = 128;  // keys per tile
 constexpr int NUM_THREADS = 384;
 constexpr int MAX_SPLIT = 4;     // CTAs of a cluster that share one item's keys
-constexpr int MAX_SAMPLES = 32;  // samples per launch (one lane each)
+constexpr int MAX_SAMPLES = 32;  // samples of a launch that numbers the live items (one lane each)
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLowestMax = -FLT_MAX;
 constexpr float kRescaleThresh = 8.0f;  // log2 units: p <= 2^8 between rescales
@@ -119,6 +119,7 @@ struct Params {
   int32_t group;        // Q tiles per item: 2, or 1 (KIND_DUAL)
   uint32_t per_inv[2];  // 2^32 / items per head, rounded up (with reference rows, without), or 0: divide
   int32_t b0, nb;       // samples of this launch: [b0, b0 + nb)
+  int32_t per_sample;   // > 0: this many items a sample, dead ones among them; b0 + item / per_sample, nb = 1
   int32_t part;         // PART_ALL, PART_ROUNDS or PART_REST of the live items
   int32_t slots;        // CTAs of a full round
   int32_t rest_max;     // largest rest that PART_REST takes
@@ -145,7 +146,10 @@ struct Params {
 };
 
 // A launch runs all live items (reference items of reusing samples are not
-// live), or the whole rounds of them that fill the GPU, or the rest.
+// live), or the whole rounds of them that fill the GPU, or the rest. Over more
+// samples than lanes every item has a CTA, and a dead one's ends after its set-up
+// (launches of 32 samples each, one after another, took up to twice as long: 256
+// samples of 4 heads of 128 rows 67 us, 42 in one).
 enum { PART_ALL = 0, PART_ROUNDS = 1, PART_REST = 2 };
 
 // Live items in whole rounds, given all of them.
@@ -442,7 +446,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
   pdl_launch();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = SPLIT ? int(cluster_rank()) : 0, nrank = SPLIT ? int(cluster_size()) : 1;
-  const int lane_mode = (lane < p.nb && p.mode) ? p.mode[p.b0 + lane] : int(RA_MODE_FULL);
+  int item = SPLIT ? int(blockIdx.x) / nrank : int(blockIdx.x), b0 = p.b0;
+  if (!SPLIT && p.per_sample > 0) {
+    const int s = item / p.per_sample;
+    b0 += s;
+    item -= s * p.per_sample;
+  }
+  const int lane_mode = (lane < p.nb && p.mode) ? p.mode[b0 + lane] : int(RA_MODE_FULL);
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -498,7 +508,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
   // share their K/V tiles in L2).
   const uint32_t reuse = __ballot_sync(0xffffffffu, lane < p.nb && lane_mode == RA_MODE_REUSE);
   const int per_reuse = p.q_blocks[0] + p.q_blocks[2];
-  int item = SPLIT ? int(blockIdx.x) / nrank : int(blockIdx.x);
   {
     const int live = p.H * (p.nb * per_reuse + (p.nb - __popc(reuse)) * p.q_blocks[1]);
     const int rounds = p.part == PART_ALL ? live : round_items(live, p.slots, p.rest_max);
@@ -514,7 +523,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
     if (item < p.H * per) break;
     item -= p.H * per;
   }
-  const int b = p.b0 + bl, mode = __shfl_sync(0xffffffffu, lane_mode, bl);
+  const int b = b0 + bl, mode = __shfl_sync(0xffffffffu, lane_mode, bl);
   const uint32_t inv = p.per_inv[per == per_reuse ? 1 : 0];
   const int h = inv ? int(__umulhi(uint32_t(item), inv)) : item / per;
   const int first = item - h * per;  // 0: the first item of its (sample, head)
@@ -1043,11 +1052,13 @@ ra_status make_plan(const Params& p, int d, int nb, int slots, Plan* out) {
   auto rounds = [](int64_t items, int64_t width) { return double((items + width - 1) / width); };
   *out = Plan{2, 1, 0};
   double best = 0;
-  for (int group = 2; group >= 1; --group) {
+  const int least_group = n > 1 ? 1 : 2;  // one key tile has no second stream (24 heads of 128 rows 6.0 and 5.3 us)
+  for (int group = 2; group >= least_group; --group) {
     const Live lv = live_items(p, group, nb);
+    const int max_cs = group == 2 && nb <= MAX_SAMPLES ? MAX_SPLIT : 1;
     const int64_t cases[3] = {lv.most, p.mode ? lv.least : lv.most, (lv.most + lv.least) / 2};
     const int n_cases = p.mode ? (nb > 1 ? 3 : 2) : 1;
-    for (int cs = 1; cs <= (group == 2 ? MAX_SPLIT : 1) && cs <= n; cs *= 2) {
+    for (int cs = 1; cs <= max_cs && cs <= n; cs *= 2) {
       int clusters = slots;
       if (cs > 1) {
         clusters = max_clusters(d, cs);
@@ -1081,13 +1092,17 @@ ra_status make_plan(const Params& p, int d, int nb, int slots, Plan* out) {
   return RA_OK;
 }
 
-// Plans and launches a call, MAX_SAMPLES samples at a time.
+// Plans and launches a call: in one go, unless its items are more than a grid has
+// CTAs.
 ra_status run(Params& p, int d, cudaStream_t st) {
   p.slots = num_sms();
-  for (p.b0 = 0; p.b0 < p.B; p.b0 += MAX_SAMPLES) {
-    p.nb = p.B - p.b0 < MAX_SAMPLES ? p.B - p.b0 : MAX_SAMPLES;
+  const int64_t most = int64_t(p.H) * (int64_t(p.q_tiles[0]) + p.q_tiles[1] + p.q_tiles[2]);  // items of a sample
+  const int64_t fit = most > 0 ? 2147483647 / most : p.B;
+  const int step = p.B <= MAX_SAMPLES ? p.B : int(fit < 1 ? 1 : fit < p.B ? fit : p.B);
+  for (p.b0 = 0; p.b0 < p.B; p.b0 += step) {
+    const int nb = p.B - p.b0 < step ? p.B - p.b0 : step;
     Plan plan;
-    ra_status s = make_plan(p, d, p.nb, p.slots, &plan);
+    ra_status s = make_plan(p, d, nb, p.slots, &plan);
     if (s != RA_OK) return s;
     p.group = plan.group;
     for (int r = 0; r < 3; ++r) p.q_blocks[r] = (p.q_tiles[r] + plan.group - 1) / plan.group;
@@ -1096,7 +1111,13 @@ ra_status run(Params& p, int d, cudaStream_t st) {
       const uint64_t per = uint64_t(p.q_blocks[0]) + p.q_blocks[2] + (i == 0 ? p.q_blocks[1] : 0);
       p.per_inv[i] = per > 1 && per * per * p.H < (uint64_t(1) << 32) ? uint32_t(((uint64_t(1) << 32) + per - 1) / per) : 0;
     }
-    const Live lv = live_items(p, plan.group, p.nb);
+    const Live lv = live_items(p, plan.group, nb);
+    p.nb = nb;
+    p.per_sample = 0;
+    if (nb > MAX_SAMPLES) {
+      p.nb = 1;
+      p.per_sample = int32_t(lv.most / nb);
+    }
     if (plan.rest_max == 0) {
       p.part = PART_ALL;
       s = launch(p, d, lv.most, plan.cs, st);

@@ -180,3 +180,44 @@ def test_masked_reference_without_text(cuda_ok, rows, H, d):
     for r in ("ref", "tgt"):
         _assert_close(o2[r][0], full["O"][r], r)
     assert abs(float(m2.double().sum()) / n["tgt"] - full["M"][0]) <= M_ABS
+
+
+@pytest.mark.parametrize("B,rows,H,d", [(33, (3, 130, 140), 2, 64), (40, (0, 20, 30), 3, 128), (70, (20, 300, 10), 2, 128),
+                                        (257, (0, 140, 5), 1, 64)])
+def test_more_samples_than_lanes(cuda_ok, B, rows, H, d):
+    """More than 32 samples: mixed modes, the fused cache write and the stamps;
+    a sample's results are those of a call of its own."""
+    from paper_2609_32415_gb300 import api
+    n = dict(zip(ROLES, rows))
+    g = torch.Generator().manual_seed(B)
+    segs = make_segments(B, H, d, n, gen=g, std=1.0)
+    modes = [int(m) for m in torch.randint(0, 4, (B,), generator=g)]
+    slot = [torch.randn(x.shape, generator=g).to(torch.bfloat16).cuda() for x in segs["ref"]]
+    old = [x.clone() for x in slot]
+    a_b = torch.full((B,), -1, dtype=torch.int32, device="cuda")
+    out = empty_outputs(B, H, d, n)
+    mp = api.alloc_mass_partial(B, H, n["text"], n["tgt"])
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    api.refadapt_joint_attn([segs["text"][0], slot[0], segs["tgt"][0]], [segs["text"][1], slot[1], segs["tgt"][1]],
+                            [segs["text"][2], slot[2], segs["tgt"][2]], [out[r] for r in ROLES], mp,
+                            mode=torch.tensor(modes, dtype=torch.int32, device="cuda"), err_word=err,
+                            ref_fresh=tuple(segs["ref"]), a_b=a_b, step=5)
+    torch.cuda.synchronize()
+    api.refadapt_check_error(err)
+    fresh = [m in (COMPUTE, FULL) for m in modes]
+    assert a_b.tolist() == [5 if f else -1 for f in fresh]
+    for got, new, was in zip(slot, segs["ref"], old):
+        for s in range(B):
+            assert torch.equal(got[s], new[s] if fresh[s] else was[s]), s
+    for s in sorted({0, 1, 31, 32, B // 2, B - 1}):
+        seen = dict(segs, ref=[x for x in slot])
+        ref = oracle_block(seen, s, modes[s], d ** -0.5)
+        for r in ROLES:
+            if n[r] == 0:
+                continue
+            if ref["O"][r] is None:
+                assert torch.isnan(out[r][s].float()).all()
+            else:
+                _assert_close(out[r][s], ref["O"][r], (s, r))
+        assert np.abs(mass_from_partials(mp, n["tgt"])[s] - ref["M"]).max() <= M_ABS
+    assert not any(torch.isnan(out["tgt"][s].float()).any() for s in range(B))
