@@ -442,7 +442,9 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
   constexpr bool SPLIT = KIND == KIND_SPLIT, DUAL = KIND == KIND_DUAL;
   using C = Cfg<D, DUAL>;
   constexpr int S = C::STAGES;
-  pdl_wait();
+  // The rest of a call starts beside its whole rounds and depends on nothing of
+  // theirs; it starts after their pdl_launch(), so after what they wait for.
+  if (!SPLIT || p.part != PART_REST) pdl_wait();
   pdl_launch();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = SPLIT ? int(cluster_rank()) : 0, nrank = SPLIT ? int(cluster_size()) : 1;
@@ -514,6 +516,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
     if (p.part == PART_REST) item += rounds;
     if (item >= (p.part == PART_REST ? live : rounds)) {  // uniform over the cluster
       if (warp == 1) tmem_dealloc(*tmem_slot, C::TMEM_COLS);
+      if (p.part == PART_REST && blockIdx.x == 0) pdl_wait();
       return;
     }
   }
@@ -911,6 +914,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
     tc_fence_after();
     tmem_dealloc(*tmem_slot, C::TMEM_COLS);
   }
+  // PART_REST starts beside the launch of the rounds (programmatic dependent
+  // launch) and needs nothing of it, but must not complete before it: what
+  // comes next in the stream waits for this launch alone.
+  if (SPLIT && p.part == PART_REST && blockIdx.x == 0) pdl_wait();
 }
 
 // ------------------------------------------------------------------ host side
@@ -1031,9 +1038,7 @@ Live live_items(const Params& p, int group, int nb) {
 //                         image-edit shape (72 items of 98 key tiles) 81 us in
 //                         clusters of two, 143 unsplit, 87 in two streams;
 //   rounds, rest split    312 items of 26 key tiles (two rounds of 152 and 8)
-//                         114 us, 131 in three rounds (112 where the rest does
-//                         not wait for the rounds, but then nothing makes what
-//                         came before the call visible to it);
+//                         111 us, 131 in three rounds;
 //   one tile, two streams items that fit few rounds: 8 heads, d = 64, of
 //                         32 + 256 + 256 rows 8.2 against 11.4 us, of 77 + 1000
 //                         + 500 rows 15.7 against 22.9 (half the latency per
