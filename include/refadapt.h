@@ -470,6 +470,11 @@ ra_status refadapt_gemm(const ra_gemm_args* args, void* stream);
 const char* refadapt_status_string(ra_status s);
 const char* refadapt_last_error(void);
 
+/* Diagnostic: how this thread's last refadapt_joint_attn, refadapt_gemm or
+ * refadapt_ln_modulate was launched, e.g. "clusters of 2" (text for people and
+ * tests, valid until the thread's next call of this function). */
+const char* refadapt_last_launch(void);
+
 /* Budget, in nanoseconds, of every device-side mbarrier wait of kernels
  * launched afterwards by this process (default 2e9). */
 void refadapt_set_wait_budget_ns(uint64_t ns);

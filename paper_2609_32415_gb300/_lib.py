@@ -23,7 +23,7 @@ EXPORTED = (
     "refadapt_ref_cache_update", "refadapt_status_string", "refadapt_last_error",
     "refadapt_set_wait_budget_ns", "refadapt_check_error", "refadapt_version",
     "refadapt_selftest_wait_timeout", "refadapt_q_delta_noalloc", "refadapt_rope_table",
-    "refadapt_ln_modulate", "refadapt_gemm", "refadapt_q_delta_gate",
+    "refadapt_ln_modulate", "refadapt_gemm", "refadapt_q_delta_gate", "refadapt_last_launch",
 )
 RA_EPI_STORE, RA_EPI_GELU, RA_EPI_RESID, RA_EPI_QKV = 0, 1, 2, 3
 
@@ -129,6 +129,8 @@ def load():
     lib.refadapt_status_string.argtypes = [c_int32]
     lib.refadapt_last_error.restype = ctypes.c_char_p
     lib.refadapt_last_error.argtypes = []
+    lib.refadapt_last_launch.restype = ctypes.c_char_p
+    lib.refadapt_last_launch.argtypes = []
     lib.refadapt_set_wait_budget_ns.restype = None
     lib.refadapt_set_wait_budget_ns.argtypes = [c_uint64]
     lib.refadapt_check_error.restype = c_int32

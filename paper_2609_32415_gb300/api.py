@@ -16,7 +16,7 @@ from ._lib import RaSeg, check
 __all__ = ["seg", "refadapt_joint_attn", "refadapt_mass_partial_len", "refadapt_q_delta",
            "refadapt_q_delta_workspace_size", "refadapt_q_delta_noalloc", "refadapt_state_size", "refadapt_state_init",
            "refadapt_gate", "refadapt_ref_cache_update", "refadapt_set_wait_budget_ns",
-           "refadapt_check_error", "refadapt_version", "refadapt_selftest_wait_timeout", "q_delta_workspace", "new_state",
+           "refadapt_check_error", "refadapt_version", "refadapt_last_launch", "refadapt_selftest_wait_timeout", "q_delta_workspace", "new_state",
            "alloc_mass_partial", "refadapt_rope_table", "rope_table", "refadapt_ln_modulate", "refadapt_gemm"]
 
 
@@ -154,6 +154,10 @@ def refadapt_check_error(err_word, stream=None):
 def refadapt_selftest_wait_timeout(err_word, budget_ns, stream=None):
     return check("refadapt_selftest_wait_timeout",
                  _lib.load().refadapt_selftest_wait_timeout(_ptr(err_word), int(budget_ns), _stream(stream)))
+
+
+def refadapt_last_launch() -> str:
+    return _lib.load().refadapt_last_launch().decode()
 
 
 def refadapt_version() -> int:

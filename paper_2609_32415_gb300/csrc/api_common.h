@@ -14,6 +14,10 @@ namespace ra {
 void set_error(const char* fmt, ...);
 void clear_error();
 
+// Records how this thread's last call was launched, for refadapt_last_launch():
+// a printf format of up to three numbers (a literal; formatted when asked for).
+void note_launch(const char* form, int a = 0, int b = 0, int c = 0);
+
 uint64_t wait_budget_ns();
 int num_sms();  // of the current device (cached per device)
 

@@ -15,6 +15,12 @@ namespace ra {
 
 namespace {
 thread_local char g_err[512] = {0};
+struct LaunchNote {
+  const char* form;
+  int n[3];
+};
+thread_local LaunchNote g_launch = {"", {0, 0, 0}};
+thread_local char g_launch_text[160];
 std::atomic<uint64_t> g_budget_ns{2000000000ull};
 std::mutex g_sm_mu;
 int g_sm_count[64] = {0};
@@ -27,6 +33,8 @@ void set_error(const char* fmt, ...) {
   va_end(ap);
 }
 void clear_error() { g_err[0] = 0; }
+
+void note_launch(const char* form, int a, int b, int c) { g_launch = LaunchNote{form, {a, b, c}}; }
 
 uint64_t wait_budget_ns() { return g_budget_ns.load(std::memory_order_relaxed); }
 
@@ -184,6 +192,12 @@ extern "C" const char* refadapt_status_string(ra_status s) {
 }
 
 extern "C" const char* refadapt_last_error(void) { return ra::g_err; }
+
+extern "C" const char* refadapt_last_launch(void) {
+  const ra::LaunchNote& l = ra::g_launch;
+  snprintf(ra::g_launch_text, sizeof(ra::g_launch_text), l.form, l.n[0], l.n[1], l.n[2]);
+  return ra::g_launch_text;
+}
 
 extern "C" void refadapt_set_wait_budget_ns(uint64_t ns) {
   ra::g_budget_ns.store(ns == 0 ? 1 : ns, std::memory_order_relaxed);

@@ -1244,12 +1244,16 @@ extern "C" ra_status refadapt_gemm(const ra_gemm_args* a, void* stream) {
   p.slots = int32_t(slots);
   p.rest_max = plan.rest_max;
   if (plan.rest_max > 0) {
+    note_launch("rounds of CTA pairs, up to %d tiles in clusters of %d", plan.rest_max, plan.cs);
     // No modes leave more whole rounds than all tiles do, or a larger split rest.
     const int64_t rest = tiles % slots, whole = rest <= plan.rest_max ? tiles - rest : tiles;
     const ra_status r = launch(p, kn.pair, P_SMEM_ALLOC, 2 * (whole < slots ? whole : slots), 2, st);
     if (r != RA_OK) return r;
     return launch(p, kn.split, SMEM_ALLOC, int64_t(4) * plan.rest_max * plan.cs, plan.cs, st);
   }
+  if (pair) note_launch("CTA pairs, %d columns", plan.bn);
+  else if (plan.cs > 1) note_launch("clusters of %d, %d columns", plan.cs, plan.bn);
+  else note_launch("single CTAs, %d columns", plan.bn);
   if (pair) return launch(p, kn.pair, P_SMEM_ALLOC, 2 * (tiles < slots ? tiles : slots), 2, st);
   if (plan.cs > 1) return launch(p, kn.split, SMEM_ALLOC, tiles * plan.cs, plan.cs, st);
   return launch(p, kn.single, SMEM_ALLOC, tiles < slots ? tiles : slots, 1, st);

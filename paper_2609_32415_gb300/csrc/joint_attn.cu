@@ -1124,10 +1124,14 @@ ra_status run(Params& p, int d, cudaStream_t st) {
       p.per_sample = int32_t(lv.most / nb);
     }
     if (plan.rest_max == 0) {
+      if (plan.group == 1) note_launch("two streams");
+      else if (plan.cs > 1) note_launch("clusters of %d", plan.cs);
+      else note_launch("pairs");
       p.part = PART_ALL;
       s = launch(p, d, lv.most, plan.cs, st);
     } else {
       // No modes leave more whole rounds than all items do, or a larger split rest.
+      note_launch("rounds of pairs, up to %d in clusters of %d", plan.rest_max, plan.cs);
       p.rest_max = plan.rest_max;
       p.part = PART_ROUNDS;
       s = launch(p, d, round_items(int(lv.most), p.slots, p.rest_max), 1, st);

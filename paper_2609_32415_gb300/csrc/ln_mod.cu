@@ -344,6 +344,7 @@ ra_status launch(void (*fn)(Params), const Params& p, int64_t ctas, int threads,
 template <int G>
 ra_status run(const Params& p, int64_t rows, bool one_row_per_warp, cudaStream_t st) {
   using L = Layout<G>;
+  note_launch(one_row_per_warp ? "one row per warp" : "persistent");
   if (one_row_per_warp)
     return launch(ln_row_kernel<G>, p, (rows + kRowWarps<G> - 1) / kRowWarps<G>, 32 * kRowWarps<G>, 0, st);
   const int64_t sms = num_sms();

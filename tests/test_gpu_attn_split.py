@@ -20,18 +20,27 @@ def _assert_close(got, ref, what=""):
     ok, worst, normwise = o_close(got.double().cpu().numpy(), ref, 0.015)
     assert ok and normwise <= 3e-3, (what, worst, normwise)
 
-# text, ref, tgt rows, heads, d, modes; what the launch model picks is named.
+def _launched(form):
+    """The last attention call took this launch form (what the launch model picks
+    for a case is asserted, or the case would not test it)."""
+    from paper_2609_32415_gb300 import api
+    got = api.refadapt_last_launch()
+    assert got.startswith(form), (form, got)
+
+
+TWO, ROUNDS, PAIRS = "two streams", "rounds of pairs, up to ", "pairs"
+# text, ref, tgt rows, heads, d, modes, launch form.
 CASES = [
-    ((33, 5000, 130), 2, 128, [REUSE]),              # one tile, two streams: 43 key tiles
-    ((33, 5000, 130), 2, 64, [BOUNDARY, REUSE]),     # the same, reference items live in one sample
-    ((33, 700, 1500), 24, 64, None),                 # the same in three rounds, 19 key tiles
-    ((40, 100, 200), 3, 64, [COMPUTE, REUSE]),       # few key tiles
-    ((0, 0, 77), 3, 128, None),                      # one key tile: no second stream
-    ((0, 0, 200), 2, 64, None),                      # two: one each
-    ((100, 900, 1900), 12, 128, [FULL]),             # 152 items, a rest of 4 in clusters of four
-    ((200, 900, 1700), 22, 128, [REUSE]),            # a rest of 24 that only reusing leaves
-    ((100, 1800, 1800), 12, 128, [FULL]),            # a rest of 52 in clusters of two
-    ((100, 300, 1900), 10, 64, [REUSE, COMPUTE]),    # mixed modes over more than a round
+    ((33, 5000, 130), 2, 128, [REUSE], TWO),           # 43 key tiles
+    ((33, 5000, 130), 2, 64, [BOUNDARY, REUSE], TWO),  # the same, reference items live in one sample
+    ((33, 700, 1500), 24, 64, None, TWO),              # three rounds, 19 key tiles
+    ((40, 100, 200), 3, 64, [COMPUTE, REUSE], TWO),    # few key tiles
+    ((0, 0, 77), 3, 128, None, PAIRS),                 # one key tile: no second stream
+    ((0, 0, 200), 2, 64, None, TWO),                   # two: one each
+    ((100, 900, 1900), 12, 128, [FULL], ROUNDS + "36 in clusters of 4"),   # 152 items and a rest of 4
+    ((200, 900, 1700), 22, 128, [REUSE], ROUNDS + "36 in clusters of 4"),  # a rest of 24 that only reusing leaves
+    ((100, 1800, 1800), 12, 128, [FULL], ROUNDS + "76 in clusters of 2"),  # a rest of 52
+    ((100, 300, 1900), 10, 64, [REUSE, COMPUTE], ROUNDS),                  # mixed modes over more than a round
 ]
 
 
@@ -39,12 +48,13 @@ def _heads(segs, out, mp, hs):
     return ({r: [x[:, hs] for x in segs[r]] for r in ROLES}, {r: out[r][:, hs] for r in ROLES}, mp[:, hs])
 
 
-@pytest.mark.parametrize("rows,H,d,modes", CASES, ids=lambda x: str(x).replace(" ", ""))
-def test_split_launches_match_oracle(cuda_ok, rows, H, d, modes):
+@pytest.mark.parametrize("rows,H,d,modes,form", CASES, ids=lambda x: str(x).replace(" ", ""))
+def test_split_launches_match_oracle(cuda_ok, rows, H, d, modes, form):
     n = dict(zip(ROLES, rows))
     B = len(modes) if modes else 1
     segs = make_segments(B, H, d, n, gen=torch.Generator().manual_seed(H * d + rows[1]), std=1.0)
     out, mp = _run(segs, B, H, d, n, modes)
+    _launched(form)
     hs = sorted({0, H // 2, H - 1})
     s2, o2, m2 = _heads(segs, out, mp, hs)
     for s in range(B):
@@ -77,6 +87,7 @@ def test_split_item_without_reference_queries(cuda_ok, H, d):
     bias[0] = float("-inf")
     api.refadapt_joint_attn(q, [segs[r][1] for r in ROLES], [segs[r][2] for r in ROLES], out, mp, err_word=err,
                             ref_logit_bias=bias)
+    _launched("clusters of %d" % (2 if H == 24 else 4))
     torch.cuda.synchronize()
     api.refadapt_check_error(err)
     hs = [1, H - 1]
@@ -95,6 +106,7 @@ def test_split_range_of_masked_keys(cuda_ok, d):
     B, H, n = 1, 2, {"text": 33, "ref": 5000, "tgt": 130}
     segs = make_segments(B, H, d, n, gen=torch.Generator().manual_seed(d + 1), std=1.0)
     out, mp = _run(segs, B, H, d, n, [REUSE], bias=[float("-inf"), 0.5])
+    _launched(TWO)
     cut = {r: [x[:, :1, :0] if r == "ref" else x[:, :1] for x in segs[r]] for r in ROLES}
     ref = oracle_block(cut, 0, REUSE, d ** -0.5)
     _assert_close(out["tgt"][0, :1], ref["O"]["tgt"])
@@ -123,6 +135,7 @@ def test_split_launches_write_the_cache(cuda_ok, rows, H, modes):
     api.refadapt_joint_attn([segs["text"][0], slot[0], segs["tgt"][0]], [segs["text"][1], slot[1], segs["tgt"][1]],
                             [segs["text"][2], slot[2], segs["tgt"][2]], [out[r] for r in ROLES], mp, mode=mode,
                             err_word=err, ref_fresh=tuple(segs["ref"]), a_b=a_b, step=5)
+    _launched(TWO if B == 2 else ROUNDS)
     torch.cuda.synchronize()
     api.refadapt_check_error(err)
     assert a_b.tolist() == [5 if m != REUSE else -1 for m in modes]
@@ -156,15 +169,16 @@ def test_two_streams_keep_the_stored_query(cuda_ok, rows, H, d):
         api.refadapt_joint_attn([segs["text"][0], slot[0], segs["tgt"][0]], [segs["text"][1], slot[1], segs["tgt"][1]],
                                 [segs["text"][2], slot[2], segs["tgt"][2]], [out[r] for r in ROLES], mp, mode=mode,
                                 err_word=err, ref_fresh=tuple(segs["ref"]), a_b=a_b, step=step)
+        _launched(TWO)
         for got, fresh in zip(slot, segs["ref"]):
             assert torch.equal(got, fresh)
     api.refadapt_check_error(err)
     assert a_b.tolist() == [19]
 
 
-@pytest.mark.parametrize("rows,H,d", [((0, 128, 4000), 24, 64), ((0, 130, 5000), 8, 128), ((0, 128, 77), 3, 64),
-                                      ((0, 1800, 1800), 12, 128)])
-def test_masked_reference_without_text(cuda_ok, rows, H, d):
+@pytest.mark.parametrize("rows,H,d,form", [((0, 128, 4000), 24, 64, PAIRS), ((0, 130, 5000), 8, 128, ROUNDS),
+                                           ((0, 128, 77), 3, 64, TWO), ((0, 1800, 1800), 12, 128, ROUNDS)])
+def test_masked_reference_without_text(cuda_ok, rows, H, d, form):
     """A reference bias of -inf where the first key tile is the reference's:
     target rows attend to the target keys alone, in every launch form (pairs,
     two streams, whole rounds and a split rest)."""
@@ -172,6 +186,7 @@ def test_masked_reference_without_text(cuda_ok, rows, H, d):
     segs = make_segments(1, H, d, n, gen=torch.Generator().manual_seed(d + H), std=1.0)
     bias = [float("-inf")] + [0.25] * (H - 1)
     out, mp = _run(segs, 1, H, d, n, [FULL], bias=bias)
+    _launched(form)
     cut = {r: [x[:, :1, :0] if r == "ref" else x[:, :1] for x in segs[r]] for r in ROLES}
     _assert_close(out["tgt"][0, :1], oracle_block(cut, 0, REUSE, d ** -0.5)["O"]["tgt"])
     assert float(mp[0, 0].abs().max()) == 0.0
@@ -182,9 +197,9 @@ def test_masked_reference_without_text(cuda_ok, rows, H, d):
     assert abs(float(m2.double().sum()) / n["tgt"] - full["M"][0]) <= M_ABS
 
 
-@pytest.mark.parametrize("B,rows,H,d", [(33, (3, 130, 140), 2, 64), (40, (0, 20, 30), 3, 128), (70, (20, 300, 10), 2, 128),
-                                        (257, (0, 140, 5), 1, 64)])
-def test_more_samples_than_lanes(cuda_ok, B, rows, H, d):
+@pytest.mark.parametrize("B,rows,H,d,form", [(33, (3, 130, 140), 2, 64, PAIRS), (40, (0, 20, 30), 3, 128, TWO),
+                                             (70, (20, 300, 10), 2, 128, TWO), (257, (0, 140, 5), 1, 64, PAIRS)])
+def test_more_samples_than_lanes(cuda_ok, B, rows, H, d, form):
     """More than 32 samples: mixed modes, the fused cache write and the stamps;
     a sample's results are those of a call of its own."""
     from paper_2609_32415_gb300 import api
@@ -202,6 +217,7 @@ def test_more_samples_than_lanes(cuda_ok, B, rows, H, d):
                             [segs["text"][2], slot[2], segs["tgt"][2]], [out[r] for r in ROLES], mp,
                             mode=torch.tensor(modes, dtype=torch.int32, device="cuda"), err_word=err,
                             ref_fresh=tuple(segs["ref"]), a_b=a_b, step=5)
+    _launched(form)
     torch.cuda.synchronize()
     api.refadapt_check_error(err)
     fresh = [m in (COMPUTE, FULL) for m in modes]

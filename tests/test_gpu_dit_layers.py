@@ -113,18 +113,24 @@ def test_ln_modulate_by_row_and_persistent_agree(cuda_ok, C):
     seg = {"shift": mods[0], "scale": mods[1]}
     x = torch.empty_like(h)
     api.refadapt_ln_modulate([dict(seg, h=h, x=x)], C)
+    _launched("persistent" if C > 256 else "one row per warp")
     for lo, hi in ((0, 1), (4000, 4007), (n - 1, n)):
         y = torch.empty((B, hi - lo, C), dtype=torch.bfloat16, device="cuda")
         api.refadapt_ln_modulate([dict(seg, h=h[:, lo:hi], x=y)], C)
+        _launched("one row per warp")
         assert torch.equal(y, x[:, lo:hi])
     ref = torch.nn.functional.layer_norm(h[:, ::500].double(), (C,), eps=1e-6)
     ref = ref * (1 + mods[1].double()[:, None]) + mods[0].double()[:, None]
     assert (x[:, ::500].double() - ref).abs().max() <= 2.0 ** -8 * ref.abs().max()
 
 
-@pytest.mark.parametrize("C,B,rows", [(1280, 300, (3, 0, 20)), (3072, 70, (1, 200, 2)), (512, 33, (0, 1, 400)),
-                                      (3072, 9, (40, 300, 2000))])
-def test_ln_modulate_many_samples(cuda_ok, C, B, rows):
+@pytest.mark.parametrize("C,B,rows,form", [(1280, 300, (3, 0, 20), 0), (3072, 70, (1, 200, 2), 0), (512, 33, (0, 1, 400), 0),
+                                           (3072, 9, (40, 300, 2000), 1), (4096, 40, (0, 90, 300), 1),
+                                           (3328, 2, (3000, 600, 150), 1), (1280, 3, (500, 3000, 4000), 1),
+                                           (2304, 34, (0, 400, 350), 1)])
+def test_ln_modulate_many_samples(cuda_ok, C, B, rows, form):
+    """By row, and persistent with rings of two to four rows and shares that cross
+    segments, samples and skipped samples."""
     from paper_2609_32415_gb300 import api
     g = torch.Generator().manual_seed(B)
     modes = [int(m) for m in torch.randint(0, 4, (B,), generator=g)]
@@ -132,6 +138,7 @@ def test_ln_modulate_many_samples(cuda_ok, C, B, rows):
              "shift": torch.randn((B, C), generator=g).cuda(), "scale": torch.randn((B, C), generator=g).cuda(),
              "gated": i == 1} for i, n in enumerate(rows)]
     api.refadapt_ln_modulate(segs, C, mode=torch.tensor(modes, dtype=torch.int32, device="cuda"))
+    _launched("persistent" if form else "one row per warp")
     reuse = torch.tensor([m == REUSE for m in modes], device="cuda")
     for i, sd in enumerate(segs):
         if sd["h"].numel() == 0:
@@ -156,11 +163,19 @@ def test_ln_modulate_with_a_short_wait_budget(cuda_ok):
     try:
         for _ in range(10):
             api.refadapt_ln_modulate([dict(sd, x=x[1])], C)
+            _launched("persistent")
             torch.cuda.synchronize()
             assert torch.equal(x[0].view(torch.int16), x[1].view(torch.int16))
             x[1].fill_(float("nan"))
     finally:
         api.refadapt_set_wait_budget_ns(500_000_000)
+
+
+def _launched(form):
+    """The last call took this launch form."""
+    from paper_2609_32415_gb300 import api
+    got = api.refadapt_last_launch()
+    assert got == form, (form, got)
 
 
 def _gemm_case(B, K, N, rows_list, epi, g, gated=None, modes=None, inplace=False, tile_mode=0):
@@ -252,6 +267,10 @@ def test_gemm_tile_widths_match_oracle(cuda_ok, epi, tile_mode, N):
     from paper_2609_32415_gb300._lib import RA_EPI_GELU, RA_EPI_RESID
     _gemm_case(1, 512, N, [40], RA_EPI_GELU if epi == "gelu" else RA_EPI_RESID, torch.Generator().manual_seed(N),
                tile_mode=tile_mode)
+    widths = {512: 64, 5120: 96, 7424: 128, 9984: 160, 12288: 192, 14848: 224, 17152: 256}
+    if tile_mode == 1:
+        widths.update({9984: 96, 14848: 128})
+    _launched("%s, %d columns" % ("CTA pairs" if tile_mode == 2 else "single CTAs", widths[N]))
 
 
 # Calls of few tiles and a long K, whose tiles are shared by the CTAs of a cluster: one row, ragged
@@ -264,19 +283,21 @@ def test_gemm_split_k_matches_oracle(cuda_ok, epi, B, K, N, rows):
     gated = [i == 1 for i in range(len(rows))]
     _gemm_case(B, K, N, rows, epi, torch.Generator().manual_seed(K + N), gated=gated, modes=[REUSE, COMPUTE][:B],
                inplace=epi == 2)
+    _launched("clusters of %d, %d columns" % (2 if rows == [77, 500, 300] else 4, 256 if N == 1024 else 128))
 
 
-# A little more than whole rounds of pair tiles (77 to 81 of them): the rest is split, its tiles
+# A little more than whole rounds of pair tiles (81 or 84 of them): the rest is split, its tiles
 # cut into quarters, of which some have no rows; with modes that leave no rest or no whole round.
-@pytest.mark.parametrize("epi,B,N,rows,modes", [(2, 1, 2816, [200, 1000, 300], [COMPUTE]),
-                                                (2, 1, 2816, [200, 1000, 300], [REUSE]),
-                                                (1, 2, 1280, [100, 700, 900], [COMPUTE, COMPUTE]),
-                                                (0, 2, 1280, [100, 700, 900], [REUSE, COMPUTE]),
-                                                (2, 3, 2304, [1, 257], [COMPUTE, REUSE, COMPUTE]),
-                                                (0, 3, 2304, [1, 385], [COMPUTE, COMPUTE, COMPUTE])])
+@pytest.mark.parametrize("epi,B,N,rows,modes", [(2, 1, 3072, [1024, 256, 300], [COMPUTE]),
+                                                (2, 1, 3072, [1024, 256, 300], [REUSE]),
+                                                (1, 2, 1536, [100, 700, 700], [COMPUTE, COMPUTE]),
+                                                (0, 2, 1536, [100, 700, 700], [REUSE, COMPUTE]),
+                                                (2, 3, 2304, [385, 130], [COMPUTE, REUSE, COMPUTE]),
+                                                (0, 3, 2304, [385, 130], [COMPUTE, COMPUTE, COMPUTE])])
 def test_gemm_split_rest_matches_oracle(cuda_ok, epi, B, N, rows, modes):
-    _gemm_case(B, 4160, N, rows, epi, torch.Generator().manual_seed(N + B), gated=[i == 1 for i in range(len(rows))],
+    _gemm_case(B, 8256, N, rows, epi, torch.Generator().manual_seed(N + B), gated=[i == 1 for i in range(len(rows))],
                modes=modes, inplace=epi == 2)
+    _launched("rounds of CTA pairs, up to 9 tiles in clusters of 4")
 
 
 @pytest.mark.parametrize("tile_mode", TILE_MODES)
