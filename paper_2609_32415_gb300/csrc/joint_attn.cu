@@ -1087,8 +1087,12 @@ ra_status make_plan(const Params& p, int d, int nb, int slots, Plan* out) {
         us += rounds(whole, slots) * cta(group, 1);
         if (live > whole) us += rounds(live - whole, clusters) * cta(group, cs);
       }
-      // A second launch has to promise a little more than the model's error.
-      if (best == 0 || us < (rest_max > 0 ? 0.96 : 0.99) * best) {
+      // A second launch has to promise a little more than the model's error, and
+      // single tiles over many rounds more: with twice the traffic they end later
+      // than they would alone (two samples of 24 heads, d = 64, 6525 keys: 715 us,
+      // 623 in pairs).
+      const double margin = rest_max > 0 ? 0.96 : group == 1 && lv.most > 3 * int64_t(slots) ? 0.90 : 0.99;
+      if (best == 0 || us < margin * best) {
         best = us;
         *out = Plan{group, cs, rest_max};
       }

@@ -198,7 +198,7 @@ def test_masked_reference_without_text(cuda_ok, rows, H, d, form):
 
 
 @pytest.mark.parametrize("B,rows,H,d,form", [(33, (3, 130, 140), 2, 64, PAIRS), (40, (0, 20, 30), 3, 128, TWO),
-                                             (70, (20, 300, 10), 2, 128, TWO), (257, (0, 140, 5), 1, 64, PAIRS)])
+                                             (70, (20, 300, 10), 2, 128, PAIRS), (257, (0, 140, 5), 1, 64, PAIRS)])
 def test_more_samples_than_lanes(cuda_ok, B, rows, H, d, form):
     """More than 32 samples: mixed modes, the fused cache write and the stamps;
     a sample's results are those of a call of its own."""
@@ -237,3 +237,17 @@ def test_more_samples_than_lanes(cuda_ok, B, rows, H, d, form):
                 _assert_close(out[r][s], ref["O"][r], (s, r))
         assert np.abs(mass_from_partials(mp, n["tgt"])[s] - ref["M"]).max() <= M_ABS
     assert not any(torch.isnan(out["tgt"][s].float()).any() for s in range(B))
+
+
+@pytest.mark.parametrize("B,rows,H,d", [(16, (2, 0, 1068), 16, 64), (4, (0, 307, 1363), 24, 64), (8, (0, 308, 310), 24, 128)])
+def test_single_tiles_only_over_few_rounds(cuda_ok, B, rows, H, d):
+    """Over many rounds one Q tile per item (twice the K and V traffic) loses to pairs."""
+    n = dict(zip(ROLES, rows))
+    segs = make_segments(B, H, d, n, gen=torch.Generator().manual_seed(B), std=1.0)
+    out, mp = _run(segs, B, H, d, n, [FULL] * B)
+    _launched(PAIRS)
+    s2, o2, m2 = _heads(segs, out, mp, [0, H - 1])
+    ref = oracle_block(s2, B - 1, FULL, d ** -0.5)
+    for r in ROLES:
+        if n[r] > 0:
+            _assert_close(o2[r][B - 1], ref["O"][r], r)
