@@ -159,7 +159,17 @@ struct Walk {
     if (cols < 0) cols = piece_cols(p);
     while (t - begin >= int64_t(p.m_tiles[g]) * cols) {
       begin += int64_t(p.m_tiles[g]) * cols;
-      if (++s == p.B) {
+      ++s;
+      if (p.m_tiles[g] == 0) {
+        s = p.B;
+      } else if (p.B > 4 && !p.gated[g] && t - begin <= 0xffffffff) {
+        // the samples' pieces are alike: count them off at once
+        const uint32_t n = uint32_t(p.m_tiles[g]) * uint32_t(cols), k = uint32_t(t - begin) / n;
+        const int pass = int(min(k, uint32_t(p.B - s)));
+        begin += int64_t(n) * pass;
+        s += pass;
+      }
+      if (s == p.B) {
         s = 0;
         if (++g == p.n_seg) return false;
       }
