@@ -1031,11 +1031,17 @@ Plan make_plan(const ra_gemm_args& a, int sms) {
       if (!a.seg[g].gated) *open += t;
     }
   };
+  // Many column tiles that all read the same few rows of A contend for the L2
+  // lines these lie in (4 rows, K = 2048, N = 8192: 21.7 us in 128 tiles of 64
+  // columns, 11.8 in 32 of 256; from 32 rows on 10.3 and 11.9).
+  bool few_rows = false;
+  for (int g = 0; g < a.n_seg; ++g) few_rows |= a.seg[g].rows > 0 && a.seg[g].rows < 32;
   for (int pair = 0; pair < 2; ++pair) {
     if ((a.tile_mode == 1 && pair) || (a.tile_mode == 2 && !pair) || (pair && sms < 2)) continue;
     const int tm = pair ? P_TM : BM, slots = pair ? sms / 2 : sms;
     for (int bn = 256; bn >= 64; bn -= 32) {
       if (a.epilogue == RA_EPI_QKV && (bn % a.d != 0 || (a.H * a.d) % bn != 0)) continue;
+      if (few_rows && bn < 256 && a.N / bn > 40) continue;
       int64_t all, open;
       tiles_of(tm, bn, &all, &open);
       const double epilogue = 0.0085 * bn;  // of a tile, hidden behind the next one's MMAs

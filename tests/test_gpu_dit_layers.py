@@ -285,6 +285,14 @@ def test_gemm_tile_widths_match_oracle(cuda_ok, epi, tile_mode, N):
     _launched("%s, %d columns" % ("CTA pairs" if tile_mode == 2 else "single CTAs", widths[N]))
 
 
+@pytest.mark.parametrize("rows,N,narrow", [([5], 14336, False), ([40, 3], 12288, False), ([40], 12288, True), ([5], 4096, True)])
+def test_gemm_few_rows_take_wide_tiles(cuda_ok, rows, N, narrow):
+    """Many column tiles do not share a handful of rows of A."""
+    from paper_2609_32415_gb300 import api
+    _gemm_case(1, 512, N, rows, 0, torch.Generator().manual_seed(N))
+    assert ("256 columns" in api.refadapt_last_launch()) != narrow, api.refadapt_last_launch()
+
+
 # Calls of few tiles and a long K, whose tiles are shared by the CTAs of a cluster: one row, ragged
 # rows, K steps that do not divide by the CTAs, tiles of 64 to 256 columns, a gated segment.
 @pytest.mark.parametrize("epi", [0, 1, 2])
