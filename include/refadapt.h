@@ -114,7 +114,8 @@ typedef struct {
  *  B, H, d          batch, heads, head dim; d in {64, 128}.
  *  softmax_scale    > 0; pass 0 for 1/sqrt(d).
  *  ref_logit_bias   device [H] fp32 or NULL: added to the logits of target
- *                   query rows against reference keys (natural-log units).
+ *                   query rows against reference keys (natural-log units);
+ *                   -inf leaves them out.
  *  mode             device [B] int32 (ra_mode) or NULL (= every row runs).
  *  mass_partial     device [B][H][refadapt_mass_partial_len(n_text, n_tgt)].
  *  mass_row_stride  the "sampled target-query rows" of Eq. 4 / Algorithm 1:

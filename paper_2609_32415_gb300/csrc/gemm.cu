@@ -722,7 +722,7 @@ __global__ void __launch_bounds__(THREADS, 1) gemm_kernel(const __grid_constant_
 // tile sequence (cluster c takes tiles c, c + G/2, ...); per K step each CTA's
 // producer loads its own 128 A rows and its half of the W tile, and both
 // loads complete on rank 0's full barrier (rank 0 arms it for both CTAs'
-// bytes). Rank 0's MMA thread issues M = 256, N = 256 MMAs; commits are
+// bytes). Rank 0's MMA thread issues M = 256 MMAs of the tile's width; commits are
 // multicast to both CTAs (stage free, accumulator ready). Each CTA's epilogue
 // reads its own TMEM rows and arrives on rank 0's accumulator-free barrier
 // (count 16). The two CTAs meet at a cluster barrier before TMEM is freed and

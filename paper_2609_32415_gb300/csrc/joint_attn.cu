@@ -95,7 +95,7 @@ struct Cfg {
   static constexpr int OFF_ITEM = (OFF_MISC + 64 + 15) / 16 * 16;  // int4 per softmax warp
   static constexpr int SMEM_BYTES = OFF_ITEM + 8 * 16;
   static constexpr int SMEM_ALLOC = SMEM_BYTES + 1024;  // slack for 1024-byte alignment
-  // Split launches: (m, l, l_ref) of every row from every rank of the cluster.
+  // Split launches (not DUAL): (m, l, l_ref) of every row from every rank of the cluster.
   // The O parts to send and those received (up to 3/4 of 256 rows x D fp32
   // each) reuse the tile buffers.
   static constexpr int OFF_STATS = (SMEM_BYTES + 15) / 16 * 16;
@@ -186,25 +186,17 @@ __device__ __forceinline__ void kv_tile(const Params& p, int j, int& r, int& row
   }
 }
 
-// Row maximum over the 64 logits in v[] (columns col0 .. col0+63 of the tile);
-// TAIL ignores columns >= nvalid.
-template <bool TAIL>
+// Row maximum over the 64 logits in v[] (columns col0 .. col0+63 of the tile),
+// those of columns >= nvalid left out.
 __device__ __forceinline__ float max64(const float (&v)[64], int col0, int nvalid, float m_in) {
   float m0 = m_in, m1 = -INFINITY, m2 = -INFINITY, m3 = -INFINITY;
 #pragma unroll
   for (int c = 0; c < 64; c += 8) {
-    if (TAIL) {
-      const int e = col0 + c;
-      m0 = fmax3f(m0, (e < nvalid) ? v[c] : -INFINITY, (e + 1 < nvalid) ? v[c + 1] : -INFINITY);
-      m1 = fmax3f(m1, (e + 2 < nvalid) ? v[c + 2] : -INFINITY, (e + 3 < nvalid) ? v[c + 3] : -INFINITY);
-      m2 = fmax3f(m2, (e + 4 < nvalid) ? v[c + 4] : -INFINITY, (e + 5 < nvalid) ? v[c + 5] : -INFINITY);
-      m3 = fmax3f(m3, (e + 6 < nvalid) ? v[c + 6] : -INFINITY, (e + 7 < nvalid) ? v[c + 7] : -INFINITY);
-    } else {
-      m0 = fmax3f(m0, v[c], v[c + 1]);
-      m1 = fmax3f(m1, v[c + 2], v[c + 3]);
-      m2 = fmax3f(m2, v[c + 4], v[c + 5]);
-      m3 = fmax3f(m3, v[c + 6], v[c + 7]);
-    }
+    const int e = col0 + c;
+    m0 = fmax3f(m0, (e < nvalid) ? v[c] : -INFINITY, (e + 1 < nvalid) ? v[c + 1] : -INFINITY);
+    m1 = fmax3f(m1, (e + 2 < nvalid) ? v[c + 2] : -INFINITY, (e + 3 < nvalid) ? v[c + 3] : -INFINITY);
+    m2 = fmax3f(m2, (e + 4 < nvalid) ? v[c + 4] : -INFINITY, (e + 5 < nvalid) ? v[c + 5] : -INFINITY);
+    m3 = fmax3f(m3, (e + 6 < nvalid) ? v[c + 6] : -INFINITY, (e + 7 < nvalid) ? v[c + 7] : -INFINITY);
   }
   return fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
 }
@@ -443,7 +435,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
   using C = Cfg<D, DUAL>;
   constexpr int S = C::STAGES;
   // The rest of a call starts beside its whole rounds and depends on nothing of
-  // theirs; it starts after their pdl_launch(), so after what they wait for.
+  // theirs; it starts after their pdl_launch(), so after what they wait for: each
+  // of their CTAs waits first, so what came before the call is complete and
+  // written back when the rest starts, on SMs that the rounds' CTAs have left.
+  // Waiting for the rounds themselves cost 2 to 12 us, as they end unevenly.
   if (!SPLIT || p.part != PART_REST) pdl_wait();
   pdl_launch();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -816,7 +811,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) joint_attn_kernel(const __grid
         for (int hf = 0; hf < 2; ++hf) {
           float v[64];
           tmem_ld64(s_t + 64 * hf, v);
-          mx = max64<true>(v, 64 * hf, nvalid, mx);
+          mx = max64(v, 64 * hf, nvalid, mx);
         }
         const float mt = fmaf(mx, sl2, badd);
         if (mt > m + kRescaleThresh) {

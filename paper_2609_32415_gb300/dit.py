@@ -29,6 +29,10 @@ previous target Q per block, mass partials) persist across steps; the
 activations (LN outputs, Q/K/V, attention outputs, MLP hidden) are one
 shared set reused by every block. The running text and target hidden states
 are updated in place by the gated-residual epilogues.
+
+Results are deterministic, but a sample's may depend on the other samples of its
+batch in their last rounding: the rows and modes of a call decide how the
+attention divides a row's keys and the projections a tile's K.
 """
 import torch
 

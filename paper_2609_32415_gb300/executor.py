@@ -75,6 +75,11 @@ class Executor:
     ``fused_cache`` (default) lets the attention of a materialising block
     write its cache slot (refadapt_joint_attn's ref_fresh arguments) instead
     of a refadapt_ref_cache_update launch before it; the results are the same.
+
+    Results are deterministic, but a sample's may depend on the other samples of
+    its batch in their last rounding: the sizes and modes of a call decide how its
+    attention divides a row's keys (refadapt_joint_attn), and with it the sums that
+    D, M and so a decision near theta are taken from.
     """
 
     def __init__(self, n_blocks, B, H, d, n_text, n_ref, n_tgt, theta, delta_max, eps=1e-6,
