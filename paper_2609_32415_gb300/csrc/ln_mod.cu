@@ -13,8 +13,8 @@
 // row. At C = 3072: 12544 rows 34.8 -> 25.8 us (6 TB/s; a plain copy of them
 // 24.3), 4352 rows 12.3 -> 9.3, 1024 rows 6.4 -> 4.0, against one row per warp and
 // no ring (ln_row_kernel). Its set-up and its walk over the pieces cost more where
-// rows are short or samples many: C = 256, 3 x 4352 rows 4.4 us by row, 6.4
-// persistent; 256 samples of one row of 3072 4.9 and 50. by_row() chooses; a row's
+// rows are short or samples many: two rows of 256 1.3 us by row, 1.9 persistent; 64
+// samples of 1 and of 205 rows of 2560 47 and 242. by_row() chooses; a row's
 // arithmetic is the same in both.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
